@@ -183,6 +183,7 @@ int solve_fp64(Grid &g, const afg_mg_opts &o, cudaStream_t s, std::vector<std::v
             if (hist[t].empty() || hist[t].back() > o.rel_tol) hist[t].push_back(rel_of(g, t));
     };
     g.make_compatible(s);
+    g.refresh_faces(s);
     if (fmg_first) {
         run(g, {1, o.n_down, o.n_up, o.n_base, 0}, o.use_graph, s, [&](cudaStream_t cs) {
             g.fmg(g.ws64, mo, 0, forest, cs);
@@ -397,6 +398,7 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
 }
 
 void set_dirichlet_dev(Grid &g, const double *b, cudaStream_t s) {
+    g.faces_changed = true;
     if (g.n_bfaces > 0) {
         if (b) check(cudaMemcpyAsync(g.d_bc, b, g.n_bfaces * 8, cudaMemcpyDeviceToDevice, s), "copy b");
         else check(cudaMemsetAsync(g.d_bc, 0, g.n_bfaces * 8, s), "zero b");
@@ -796,6 +798,7 @@ static int one_cycle(afg_tree *t, const afg_mg_opts *opts, afg_stats *st, bool f
     const auto t0 = clk::now();
     const afg::MgOpts mo{o.n_down, o.n_up, o.n_base};
     g.make_compatible(t->stream);
+    g.refresh_faces(t->stream);
     run(g, {fmg ? 30 : 31, o.n_down, o.n_up, o.n_base, 0}, o.use_graph, t->stream, [&](cudaStream_t cs) {
         if (fmg) g.fmg(g.ws64, mo, 0, false, cs);
         else g.vcycle(g.ws64, g.lmax, mo, 0, nullptr, cs);

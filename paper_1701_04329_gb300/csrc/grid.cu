@@ -86,12 +86,12 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     N = trees[0]->N;
     T = (int)trees.size();
     // Below level 1 every root box has its coarse grids of N/2, ..., 2 cells
-    // (Sec. 3.2), connected like the roots.  A single tree whose level 1 is a
-    // block of root boxes small enough for one CTA's shared memory keeps them
-    // there only (k_bottom_block); otherwise they are device boxes, one per
+    // (Sec. 3.2), connected like the roots.  They run in one launch per cycle
+    // (the coarse launch), which keeps them in shared memory, for trees of
+    // one root box and for a single tree whose level 1 is a small block of
+    // root boxes; for several roots otherwise they are device boxes, one per
     // root and level, and the cycle runs on the per-level kernels down to the
-    // coarsest grid (several roots: `roots_levels`), or, with one root per
-    // tree, in one launch per cycle (k_bottom).
+    // coarsest grid (`roots_levels`).
     bool multi = false;
     for (const HostTree *h : trees) multi |= h->nroots() != 1;
     block = T == 1 && multi && !levels_only &&
@@ -116,13 +116,6 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
         lmax = std::max(lmax, trees[t]->L);
         tree_cells.push_back(trees[t]->n_leaf_cells);
         tree_faces.push_back(trees[t]->n_bfaces);
-    }
-    // one tree of one root box: level 2 (the root's 2^D children, one grid of
-    // 2N cells per side) joins the bottom launch where it fits shared memory
-    if (T == 1 && !multi && lmax >= 2) {
-        const long long cells2 = D == 2 ? 4LL * N * N : 8LL * N * N * N;
-        btop32 = bottom_smem(D, false, 2 * N) <= max_smem_optin() ? 2 : 1;
-        btop64 = cells2 <= 1024 && bottom_smem(D, true, 2 * N) <= max_smem_optin() ? 2 : 1;
     }
     // global box ids: level-major, then tree, then the tree's canonical order
     std::vector<std::vector<int>> gid(T), sub(T, std::vector<int>(nsub, -1));
@@ -282,17 +275,7 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     }
 
     auto &own = owned;
-    if (block) {  // the roots' box ids in block order
-        const HostTree &ht = *trees[0];
-        for (int a = 0; a < 3; ++a) block_nroot[a] = ht.nr[a];
-        for (int s2 = 0; s2 < 6; ++s2) block_bct[s2] = ht.bct[s2];
-        std::vector<int> rb(ht.nroots(), -1);
-        for (int b = ht.lstart[1]; b < ht.lstart[1] + ht.lcount[1]; ++b) {
-            const HBox &hx = ht.boxes[b];
-            rb[(hx.idx[0] - 1) + ht.nr[0] * ((hx.idx[1] - 1) + ht.nr[1] * (D == 3 ? hx.idx[2] - 1 : 0))] = gid[0][b];
-        }
-        d_root_box = upload(rb, own);
-    }
+    if (!roots_levels) plan_coarse(trees, gid);
     meta.nb = upload(nb, own);
     meta.nmask = upload(nmask, own);
     std::vector<unsigned char> cfmask(nbox, 0);
@@ -429,7 +412,7 @@ void Grid::smooth(Workspace &w, int l, int steps, int hom, const int *active, cu
 // Residual on level l restricted to l-1 with v_H <- I v_h, v'_H <- v_H, then
 // rho_H <- I r_h + A_H(v_H) on the refined boxes of l-1 (Eq. residual,
 // Eq. coarse-rhs); leaves of l-1 store v' too.
-void Grid::down_step(Workspace &w, int l, int hom, const int *active, cudaStream_t s) {
+void Grid::down_step(Workspace &w, int l, int hom, const int *active, cudaStream_t s, bool fas) {
     Level &v = L(l), &vc = L(l - 1);
     BoxMeta A = meta;
     A.active = active;
@@ -439,39 +422,125 @@ void Grid::down_step(Workspace &w, int l, int hom, const int *active, cudaStream
         return;
     }
     launch_resid_restrict(cfg(l, w.fp64, s), A, v.b0, v.nb, w.u->p, w.rho->p, w.vold->p, 1.0 / (v.h * v.h), hom);
+    if (!fas) return;  // the coarse launch completes the source of its top level
     launch_fas(cfg(l - 1, w.fp64, s), A, vc.b0, vc.nb, w.u->p, w.rho->p, w.vold->p, 1.0 / (vc.h * vc.h), hom,
                w.rhoh_p());
 }
 
-void Grid::bottom(Workspace &w, int ltop, int mode, const MgOpts &o, int hom, const int *active, cudaStream_t s) {
+// The coarse launch's top level per precision: the highest level that covers
+// the whole domain in every tree, whose grids fit one block's shared memory,
+// and whose half-sweep is not too much work for the blocks it runs on.
+void Grid::plan_coarse(const std::vector<const HostTree *> &trees, const std::vector<std::vector<int>> &gid) {
+    int full = 1;
+    for (;; ++full) {
+        bool ok = true;
+        for (const HostTree *h : trees)
+            ok = ok && full + 1 <= h->L && (long long)h->lcount[full + 1] == ((long long)h->nroots() << (D * full));
+        if (!ok) break;
+    }
+    const int *nr = trees[0]->nr;
+    std::vector<int> bc;
+    for (const HostTree *h : trees) {
+        int code = 0;
+        for (int s = 0; s < 2 * D; ++s) {
+            if (h->bct[s] == 1) code |= 1 << s;
+            if (h->bct[s] == 2) code |= 64 << (s / 2);
+        }
+        bc.push_back(code);
+    }
+    const int *d_bc_types = upload(bc, owned);
+    std::map<int, const int *> tables;  // boxes of a level by position, per tree
+    auto table = [&](int l) {
+        auto it = tables.find(l);
+        if (it != tables.end()) return it->second;
+        const int f = 1 << (l - 1);
+        const int sx = nr[0] * f, sy = nr[1] * f, sz = D == 3 ? nr[2] * f : 1;
+        std::vector<int> v((size_t)T * sx * sy * sz);
+        for (int t = 0; t < T; ++t)
+            for (int b = trees[t]->lstart[l]; b < trees[t]->lstart[l] + trees[t]->lcount[l]; ++b) {
+                const HBox &x = trees[t]->boxes[b];
+                const int z = D == 3 ? x.idx[2] - 1 : 0;
+                v[(((size_t)t * sz + z) * sy + (x.idx[1] - 1)) * sx + (x.idx[0] - 1)] = gid[t][b];
+            }
+        return tables[l] = upload(v, owned);
+    };
+    for (const bool fp64 : {false, true}) {
+        Coarse &c = fp64 ? coarse64 : coarse32;
+        for (int l = 1; l <= full; ++l) {
+            CoarseArgs plan;
+            const long long m = (long long)N << (l - 1);
+            if (m > 1024) break;
+            const size_t smem = coarse_plan(D, fp64, (int)m, N, nr, T, plan);
+            const int li = plan.nl - 1;
+            const long long work = (long long)plan.nx[li] * plan.ny[li] * plan.P[li] / 2;  // cells of a half-sweep per block
+            // up to this much the launch beats the level's 11 launches of 2.1 us (FP32)
+            // or 3.3 us (FP64): a 64^2 grid's half-sweep takes 0.75 us (FP32, one
+            // block) and 1.2 us (FP64, eight blocks), a 32^3 grid's 1.8 and 6.7 us
+            const long long most = fp64 ? 512 : 2048;
+            if (l > 1 && (smem > max_smem_optin() || work > most)) break;
+            c.top = l;
+            c.plan = plan;
+            c.smem = smem;
+        }
+        c.plan.dbox = table(c.top);
+        c.plan.tree_bc = d_bc_types;
+        // faces: the slots of every non-periodic axis in any tree (a tree's own periodic sides are not read)
+        int all = 7;
+        for (int code : bc) all &= code >> 6;
+        std::vector<std::vector<int>> slots;
+        size_t most_faces = 0;
+        for (int r = 0; r < c.plan.R; ++r) {
+            slots.push_back(coarse_faces(D, c.plan, r, all));
+            most_faces = std::max(most_faces, slots.back().size());
+        }
+        std::vector<int> flat;
+        for (auto &v : slots) {
+            v.resize(most_faces, -1);
+            flat.insert(flat.end(), v.begin(), v.end());
+        }
+        c.plan.nface = (int)most_faces;
+        c.plan.fslot = upload(flat, owned);
+        if (fp64) c.plan.fval = upload(std::vector<double>(most_faces * c.plan.R * T, 0.0), owned);
+    }
+}
+
+// the coarse launch's copy of the boundary data, after it changed (not captured)
+void Grid::refresh_faces(cudaStream_t s) {
+    if (!faces_changed || levels_path()) return;
+    CoarseArgs G = coarse64.plan;
+    G.mode = 2;
+    launch_coarse(cfg(1, true, s), meta, G, coarse64.smem, T, ws64.u->p, ws64.rho->p, ws64.vold->p);
+    faces_changed = false;
+}
+
+void Grid::coarse_cycle(Workspace &w, int mode, const MgOpts &o, int hom, const int *active, cudaStream_t s) {
     BoxMeta A = meta;
     A.active = active;
-    if (block) {  // one tree: level 1 and the grids below it in one CTA
-        launch_bottom_block(cfg(1, w.fp64, s), A, block_nroot, block_bct, d_root_box, N, mode, w.u->p, w.rho->p,
-                            w.vold->p, o.n_down, o.n_up, o.n_base, hom);
-        return;
-    }
-    const int top = btop(w);
-    int b0[kBottomLevels] = {};
-    for (int l = lmin; l <= top; ++l) b0[l - lmin] = L(l).b0;
-    launch_bottom(cfg(1, w.fp64, s), A, T, N, lmin, ltop, top, mode, w.u->p, w.rho->p, w.vold->p, o.n_down, o.n_up,
-                  o.n_base, hom, b0);
+    const Coarse &c = coarse(w);
+    CoarseArgs G = c.plan;
+    G.mode = mode;
+    G.nd = o.n_down;
+    G.nu = o.n_up;
+    G.nb = o.n_base;
+    G.hom = hom;
+    G.fas = lmax > c.top;
+    if (!w.fp64 && !hom) throw std::runtime_error("FP32 cycles run with homogeneous boundary data");
+    launch_coarse(cfg(1, w.fp64, s), A, G, c.smem, T, w.u->p, w.rho->p, w.vold->p);
 }
 
 // FAS V-cycle (Sec. 3.2) from ltop down to the coarsest grid and back.  The
-// levels at and below btop(w) (the root box, or level 2 of a one-root tree)
-// run in one launch (k_bottom).
+// levels up to coarse(w).top run in one launch.
 void Grid::vcycle(Workspace &w, int ltop, const MgOpts &o, int hom, const int *active, cudaStream_t s) {
     if (levels_path()) {
         vcycle_levels(w, ltop, o, hom, active, s);
         return;
     }
-    const int top = btop(w);
+    const int top = coarse(w).top;
     for (int l = ltop; l > top; --l) {
         smooth(w, l, o.n_down, hom, active, s);
-        down_step(w, l, hom, active, s);
+        down_step(w, l, hom, active, s, l - 1 > top);
     }
-    bottom(w, ltop < top ? ltop : top, 0, o, hom, active, s);
+    coarse_cycle(w, 0, o, hom, active, s);
     for (int l = top + 1; l <= ltop; ++l) {
         correct(w, l, active, s);
         smooth(w, l, o.n_up, hom, active, s);
@@ -483,13 +552,14 @@ void Grid::vcycle(Workspace &w, int ltop, const MgOpts &o, int hom, const int *a
 // l-1 and run a V-cycle from l.  In a forest a tree leaves the loop after its
 // own finest level (masked).
 void Grid::fmg(Workspace &w, const MgOpts &o, int hom, bool masked, cudaStream_t s) {
-    for (int l = lmax; l > lmin; --l) restrict_u(w, l, L(l).b0, L(l).nb, nullptr, s);
-    for (int l = lmax; l > lmin; --l) down_step(w, l, hom, nullptr, s);
+    // the levels up to l0 in one launch (every tree reaches level l0)
+    const bool levels = levels_path();
+    const int l0 = levels ? 1 : coarse(w).top, low = levels ? lmin : l0;
+    for (int l = lmax; l > low; --l) restrict_u(w, l, L(l).b0, L(l).nb, nullptr, s);
+    for (int l = lmax; l > low; --l) down_step(w, l, hom, nullptr, s, levels || l - 1 > low);
     const size_t es = w.fp64 ? 8 : 4;
-    // steps l = lmin..btop in one launch (every tree reaches level btop)
-    const int l0 = levels_path() ? 1 : btop(w);
-    if (levels_path()) fmg_low_levels(w, o, hom, s);
-    else bottom(w, l0, 1, o, hom, nullptr, s);
+    if (levels) fmg_low_levels(w, o, hom, s);
+    else coarse_cycle(w, 1, o, hom, nullptr, s);
     for (int l = l0 + 1; l <= lmax; ++l) {
         Level &v = L(l);
         const int *active = masked ? fmg_mask(l) : nullptr;

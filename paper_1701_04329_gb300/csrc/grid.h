@@ -92,17 +92,20 @@ class Grid {
 
     int D, N, T, lmin, lmax;
     // a single tree whose level 1 is a block of root boxes: no device boxes
-    // below level 1 (the block bottom solve keeps those grids in shared memory)
+    // below level 1 (the coarse launch keeps those grids in shared memory)
     bool block = false;
-    // highest level of the bottom launch (k_bottom) per precision: 1, or 2
-    // for one tree of one root box whose level-2 grid fits one CTA's shared
-    // memory (FP32), and in FP64 only while that grid holds at most 1024
-    // cells (one SM's FP64 rate makes a larger one slower there than the
-    // per-level kernels: 130 us per call for 16^3 against about 110 us)
-    int btop32 = 1, btop64 = 1;
-    int btop(const Workspace &w) const { return w.fp64 ? btop64 : btop32; }
-    int block_nroot[3] = {1, 1, 1}, block_bct[6] = {0, 0, 0, 0, 0, 0};
-    int *d_root_box = nullptr;  // box id of root ri + nroot0 (rj + nroot1 rk)
+    // the levels that run in one launch per cycle (kernels_coarse.cuh), per
+    // precision: the highest one, the launch's plan and its shared memory
+    struct Coarse {
+        int top = 1;
+        CoarseArgs plan;
+        size_t smem = 0;
+    };
+    Coarse coarse32, coarse64;
+    bool faces_changed = false;  // boundary data newer than the coarse launch's copy
+    void refresh_faces(cudaStream_t s);
+    const Coarse &coarse(const Workspace &w) const { return w.fp64 ? coarse64 : coarse32; }
+    void plan_coarse(const std::vector<const HostTree *> &trees, const std::vector<std::vector<int>> &gid);
     std::vector<Level> lv;
     Level &L(int l) { return lv[l - lmin]; }
     int nbox = 0, n_leaf_boxes = 0;
@@ -174,16 +177,16 @@ class Grid {
 
     // ---- multigrid building blocks ---------------------------------------
     void smooth(Workspace &w, int l, int steps, int hom, const int *active, cudaStream_t s);
-    void down_step(Workspace &w, int l, int hom, const int *active, cudaStream_t s);
+    void down_step(Workspace &w, int l, int hom, const int *active, cudaStream_t s, bool fas = true);
     void vcycle(Workspace &w, int ltop, const MgOpts &o, int hom, const int *active, cudaStream_t s);
-    // levels lmin..1 (one box per tree): mode 0 V-cycle from ltop, mode 1 FMG steps lmin..1
-    void bottom(Workspace &w, int ltop, int mode, const MgOpts &o, int hom, const int *active, cudaStream_t s);
+    // the levels up to coarse(w).top in one launch: mode 0 V-cycle, mode 1 FMG steps
+    void coarse_cycle(Workspace &w, int mode, const MgOpts &o, int hom, const int *active, cudaStream_t s);
     void fmg(Workspace &w, const MgOpts &o, int hom, bool masked, cudaStream_t s);
     void restrict_all(Workspace &w, cudaStream_t s);
     void restrict_cf(Workspace &w, cudaStream_t s);  // only what the composite residual reads
     // restriction of u from the boxes of level l (or a list) into their parents
     void restrict_u(Workspace &w, int l, int b0, int n, const int *list, cudaStream_t s);
-    // the cycle on the per-level kernels down to the coarsest grid (no k_bottom)
+    // the cycle on the per-level kernels down to the coarsest grid (no coarse launch)
     void vcycle_levels(Workspace &w, int ltop, const MgOpts &o, int hom, const int *active, cudaStream_t s);
     void fmg_low_levels(Workspace &w, const MgOpts &o, int hom, cudaStream_t s);
     // composite residual of ws64 (restriction + leaf residual), norms to host buffer (async)

@@ -64,25 +64,21 @@ int occupancy(const void *kernel, size_t smem) {
 #define AFG_BY_DIM(FN, ...) \
     do { if (c.D == 2) DimOps<2>::FN(__VA_ARGS__); else DimOps<3>::FN(__VA_ARGS__); } while (0)
 
-void launch_bottom(const LaunchCfg &c, const BoxMeta &A, int ntrees, int N, int lmin, int ltop, int top, int mode,
-                   void *u, void *rho, void *vold, int nd, int nu, int nb, int hom, const int *lvl_b0) {
-    AFG_BY_DIM(bottom, c, A, ntrees, N, lmin, ltop, top, mode, u, rho, vold, nd, nu, nb, hom, lvl_b0);
-}
-size_t bottom_smem(int D, bool fp64, int top_m) {
-    if (D == 2) return fp64 ? bottom_smem<2, double>(top_m) : bottom_smem<2, float>(top_m);
-    return fp64 ? bottom_smem<3, double>(top_m) : bottom_smem<3, float>(top_m);
-}
-void launch_bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, const int *bct, const int *root_box,
-                         int N, int mode, void *u, void *rho, void *vold, int nd, int nu, int nb, int hom) {
-    AFG_BY_DIM(bottom_block, c, A, nroot, bct, root_box, N, mode, u, rho, vold, nd, nu, nb, hom);
+void launch_coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+                   const void *rho, void *vold) {
+    AFG_BY_DIM(coarse, c, A, G, smem, ntrees, u, rho, vold);
 }
 size_t bottom_block_smem(int D, bool fp64, int N, const int *nroot, const int *bct) {
-    BlockTree B;
-    for (int a = 0; a < 3; ++a) B.nroot[a] = a < D ? nroot[a] : 1;
-    for (int s = 0; s < 6; ++s) B.bct[s] = s < 2 * D ? bct[s] : 0;
-    B.root_box = nullptr;
-    if (D == 2) return fp64 ? block_bottom_smem<2, double>(N, B) : block_bottom_smem<2, float>(N, B);
-    return fp64 ? block_bottom_smem<3, double>(N, B) : block_bottom_smem<3, float>(N, B);
+    size_t n = 0;
+    for (int M = 2; M <= N; M *= 2) {
+        const BlkLevel L = blk_level(D, nroot, M);
+        n += 4 * (size_t)L.padded;
+        for (int s = 0; s < 2 * D; ++s) {
+            int t1, t2;
+            if (bct[s] != 2) n += (size_t)blk_faces(L, s, t1, t2);
+        }
+    }
+    return n * (fp64 ? 8 : 4);
 }
 void launch_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *u, const void *rho,
                    const void *rhoh, double h2, int colour, int hom) {

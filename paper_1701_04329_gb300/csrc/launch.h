@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "coarse_plan.h"
 #include "kernels.cuh"
 
 namespace afg {
@@ -25,23 +26,13 @@ struct LaunchCfg {
 // counts launches of this library's kernels (host side)
 extern unsigned long long g_launches;
 
-// the levels at and below the root box in one launch (one CTA per tree), and
-// level 2 as well for one tree of one root box (top = 2; otherwise top = 1):
-// mode 0 = V-cycle from ltop (<= top), mode 1 = the FMG steps up to level
-// top; lvl_b0[li] = first box of level lmin + li (li = 0 .. top - lmin)
-constexpr int kBottomLevels = 6;  // grids of 2 .. 64 cells per side
-void launch_bottom(const LaunchCfg &, const BoxMeta &, int ntrees, int N, int lmin, int ltop, int top, int mode,
-                   void *u, void *rho, void *vold, int nd, int nu, int nb, int hom, const int *lvl_b0);
-// shared memory of that launch for grids of up to top_m cells per side (bytes)
-size_t bottom_smem(int D, bool fp64, int top_m);
-// the levels at and below level 1 of one tree whose level 1 is a block of
-// root boxes (one CTA): nroot[3] roots per axis, bct[6] side types,
-// root_box (device) the box id of root ri + nroot0 (rj + nroot1 rk); mode 0 =
-// V-cycle from level 1, mode 1 = the FMG steps up to level 1.  Throws when
-// the block's grids do not fit one CTA's shared memory.
-void launch_bottom_block(const LaunchCfg &, const BoxMeta &, const int *nroot, const int *bct, const int *root_box,
-                         int N, int mode, void *u, void *rho, void *vold, int nd, int nu, int nb, int hom);
-// shared memory that launch needs (bytes)
+// the levels up to a grid's coarse top in one launch (kernels_coarse.cuh);
+// G: the grid's plan with the cycle's options (one cluster of G.R blocks per tree)
+void launch_coarse(const LaunchCfg &, const BoxMeta &, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+                   const void *rho, void *vold);
+// shared memory of one block that holds a block of root boxes and the grids
+// below it with four arrays each (bytes): what decides whether such a tree
+// keeps those grids out of device memory
 size_t bottom_block_smem(int D, bool fp64, int N, const int *nroot, const int *bct);
 // opt-in shared memory per block of the current device (bytes)
 size_t max_smem_optin();

@@ -10,8 +10,8 @@
 #include "kernels_leaf.cuh"
 #include "kernels_smooth.cuh"
 #include "kernels_full.cuh"
-#include "kernels_bottom.cuh"
-#include "kernels_block.cuh"
+#include "block_bottom.cuh"
+#include "kernels_coarse.cuh"
 #include "launch.h"
 
 namespace afg {
@@ -282,44 +282,25 @@ void do_rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, co
     ++g_launches;
 }
 
-static_assert(kBottomLevels == kBottomMaxLevels, "bottom level count");
-
 template <int D, typename T>
-void do_bottom(const LaunchCfg &c, const BoxMeta &A, int ntrees, int N, int lmin, int ltop, int top, int mode,
-               void *u, void *rho, void *vold, int nd, int nu, int nb, int hom, const int *lvl_b0) {
-    const size_t smem = bottom_smem<D, T>(top == 2 ? 2 * N : N);
-    auto k = k_bottom<D, T>;
+void do_coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+               const void *rho, void *vold) {
+    auto k = k_coarse<D, T>;
     occupancy(reinterpret_cast<const void *>(k), smem);  // sets the shared-memory limit
-    BottomArgs P = {};
-    P.ntrees = ntrees;
-    P.N = N;
-    P.lmin = lmin;
-    P.ltop = ltop;
-    P.mode = mode;
-    P.nd = nd;
-    P.nu = nu;
-    P.nb = nb;
-    P.hom = hom;
-    P.top = top;
-    for (int li = 0; li <= top - lmin && li < kBottomMaxLevels; ++li) P.b0[li] = lvl_b0[li];
-    launch_pdl_block(k, ntrees, kBottomThreads, smem, c.stream, A, P, (T *)u, (T *)rho, (T *)vold);
-    ++g_launches;
-}
-
-template <int D, typename T>
-void do_bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, const int *bct, const int *root_box,
-                     int N, int mode, void *u, void *rho, void *vold, int nd, int nu, int nb, int hom) {
-    BlockTree B;
-    for (int a = 0; a < 3; ++a) B.nroot[a] = a < D ? nroot[a] : 1;
-    for (int s = 0; s < 6; ++s) B.bct[s] = s < 2 * D ? bct[s] : 0;
-    B.root_box = root_box;
-    const size_t smem = block_bottom_smem<D, T>(N, B);
-    if (smem > max_smem_optin())
-        throw std::runtime_error("the block of root boxes is too large for one CTA's shared memory (" +
-                                 std::to_string(smem) + " bytes)");
-    auto k = k_bottom_block<D, T>;
-    occupancy(reinterpret_cast<const void *>(k), smem);  // sets the shared-memory limit once
-    launch_pdl(k, 1, smem, c.stream, A, B, N, mode, (T *)u, (T *)rho, (T *)vold, nd, nu, nb, hom);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ntrees * G.R);
+    cfg.blockDim = dim3(kCoarseThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = G.R;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = G.R > 1 ? 2 : 1;
+    cudaLaunchKernelEx(&cfg, k, A, G, (T *)u, (const T *)rho, (T *)vold);
     ++g_launches;
 }
 
@@ -360,11 +341,8 @@ void do_bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, con
 template <int D, typename T>
 struct PrecOps {
     static void rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh);
-    static void bottom(const LaunchCfg &c, const BoxMeta &A, int ntrees, int N, int lmin, int ltop, int top, int mode,
-                       void *u, void *rho, void *vold, int nd, int nu, int nb, int hom, const int *lvl_b0);
-    static void bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, const int *bct,
-                             const int *root_box, int N, int mode, void *u, void *rho, void *vold, int nd, int nu,
-                             int nb, int hom);
+    static void coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+                       const void *rho, void *vold);
     static void smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *u,
                        const void *rho, const void *rhoh, double h2, int colour, int hom);
     static void resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho, void *vold,
@@ -386,17 +364,9 @@ void PrecOps<D, T>::rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *lis
 }
 
 template <int D, typename T>
-void PrecOps<D, T>::bottom(const LaunchCfg &c, const BoxMeta &A, int ntrees, int N, int lmin, int ltop, int top,
-                           int mode, void *u, void *rho, void *vold, int nd, int nu, int nb, int hom,
-                           const int *lvl_b0) {
-    do_bottom<D, T>(c, A, ntrees, N, lmin, ltop, top, mode, u, rho, vold, nd, nu, nb, hom, lvl_b0);
-}
-
-template <int D, typename T>
-void PrecOps<D, T>::bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, const int *bct,
-                                 const int *root_box, int N, int mode, void *u, void *rho, void *vold, int nd, int nu,
-                                 int nb, int hom) {
-    do_bottom_block<D, T>(c, A, nroot, bct, root_box, N, mode, u, rho, vold, nd, nu, nb, hom);
+void PrecOps<D, T>::coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+                           const void *rho, void *vold) {
+    do_coarse<D, T>(c, A, G, smem, ntrees, u, rho, vold);
 }
 
 template <int D, typename T>
@@ -447,11 +417,8 @@ void PrecOps<D, T>::leaf_get(const LaunchCfg &c, const BoxMeta &A, const int *li
 template <int D>
 struct DimOps {
     static void rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh);
-    static void bottom(const LaunchCfg &c, const BoxMeta &A, int ntrees, int N, int lmin, int ltop, int top, int mode,
-                       void *u, void *rho, void *vold, int nd, int nu, int nb, int hom, const int *lvl_b0);
-    static void bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, const int *bct,
-                             const int *root_box, int N, int mode, void *u, void *rho, void *vold, int nd, int nu,
-                             int nb, int hom);
+    static void coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+                       const void *rho, void *vold);
     static void smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *u,
                        const void *rho, const void *rhoh, double h2, int colour, int hom);
     static void resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho, void *vold,
@@ -486,20 +453,10 @@ void DimOps<D>::rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, i
 }
 
 template <int D>
-void DimOps<D>::bottom(const LaunchCfg &c, const BoxMeta &A, int ntrees, int N, int lmin, int ltop, int top,
-                       int mode, void *u, void *rho, void *vold, int nd, int nu, int nb, int hom, const int *lvl_b0) {
-    if (c.fp64)
-        PrecOps<D, double>::bottom(c, A, ntrees, N, lmin, ltop, top, mode, u, rho, vold, nd, nu, nb, hom, lvl_b0);
-    else
-        PrecOps<D, float>::bottom(c, A, ntrees, N, lmin, ltop, top, mode, u, rho, vold, nd, nu, nb, hom, lvl_b0);
-}
-
-template <int D>
-void DimOps<D>::bottom_block(const LaunchCfg &c, const BoxMeta &A, const int *nroot, const int *bct,
-                             const int *root_box, int N, int mode, void *u, void *rho, void *vold, int nd, int nu,
-                             int nb, int hom) {
-    if (c.fp64) PrecOps<D, double>::bottom_block(c, A, nroot, bct, root_box, N, mode, u, rho, vold, nd, nu, nb, hom);
-    else PrecOps<D, float>::bottom_block(c, A, nroot, bct, root_box, N, mode, u, rho, vold, nd, nu, nb, hom);
+void DimOps<D>::coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
+                       const void *rho, void *vold) {
+    if (c.fp64) PrecOps<D, double>::coarse(c, A, G, smem, ntrees, u, rho, vold);
+    else PrecOps<D, float>::coarse(c, A, G, smem, ntrees, u, rho, vold);
 }
 
 template <int D>
