@@ -404,7 +404,7 @@ void Grid::smooth(Workspace &w, int l, int steps, int hom, const int *active, cu
     c.vpt = vpt;
     for (int it = 0; it < steps; ++it)
         for (int col = 0; col < 2; ++col) {
-            if (op) launch_var_smooth(c, A, v.b0, v.nb, w.u->p, w.rho->p, eps_of(w), col, hom, op);
+            if (op) launch_var_smooth(c, A, v.b0, v.nb, w.u->p, w.rho->p, var_args(w, l), col, hom);
             else launch_smooth(c, A, v.b0, v.nb, nullptr, w.u->p, w.rho->p, w.rhoh_p(), v.h * v.h, col, hom);
         }
 }
@@ -417,8 +417,10 @@ void Grid::down_step(Workspace &w, int l, int hom, const int *active, cudaStream
     BoxMeta A = meta;
     A.active = active;
     if (op) {
-        launch_var_resid_restrict(cfg(l, w.fp64, s), A, v.b0, v.nb, w.u->p, w.rho->p, w.vold->p, eps_of(w), hom, op);
-        launch_var_fas(cfg(l - 1, w.fp64, s), A, vc.b0, vc.nb, w.u->p, w.rho->p, w.vold->p, eps_of(w), hom, op);
+        launch_var_resid_restrict(cfg(l, w.fp64, s), A, v.b0, v.nb, w.u->p, w.rho->p, w.vold->p, var_args(w, l), hom);
+        if (fas)
+            launch_var_fas(cfg(l - 1, w.fp64, s), A, vc.b0, vc.nb, w.u->p, w.rho->p, w.vold->p, var_args(w, l - 1),
+                           hom);
         return;
     }
     launch_resid_restrict(cfg(l, w.fp64, s), A, v.b0, v.nb, w.u->p, w.rho->p, w.vold->p, 1.0 / (v.h * v.h), hom);
@@ -642,6 +644,13 @@ void Grid::set_eps(const double *eps_leaf, cudaStream_t s) {
     launch_leaf_set(leaf_cfg(true, s), meta, d_leaves, n_leaf_boxes, eps_leaf, eps64->p);
     for (int l = lmax; l > lmin; --l) launch_var_restrict(cfg(l, true, s), meta, L(l).b0, L(l).nb, nullptr, eps64->p, op);
     launch_to_f32(eps64->as<double>(), eps32->as<float>(), ncell, s);
+    const size_t nc = (size_t)ncell * (2 * D + 2);
+    if (!coef64) coef64.reset(new DevBuf(nc * 8));
+    if (!coef32) coef32.reset(new DevBuf(nc * 4));
+    for (int l = lmin; l <= lmax; ++l) {
+        launch_var_coef(cfg(l, true, s), meta, L(l).b0, L(l).nb, eps64->p, coef64->p, ncell, op);
+        launch_var_coef(cfg(l, false, s), meta, L(l).b0, L(l).nb, eps32->p, coef32->p, ncell, op);
+    }
     eps_set = true;
 }
 
@@ -656,8 +665,8 @@ void Grid::norms_async(Workspace &w, int hom, void *rout, bool rout_f32, cudaStr
     restrict_cf(w, s);
     check(cudaMemsetAsync(d_norms, 0, 2 * T * sizeof(unsigned long long), s), "memset norms");
     if (op)
-        launch_var_leaf_residual(leaf_cfg(w.fp64, s), meta, d_leaves, n_leaf_boxes, w.u->p, w.rho->p, eps_of(w), hom,
-                                 op, d_norms, d_norms + T, rout, rout_f32);
+        launch_var_leaf_residual(leaf_cfg(w.fp64, s), meta, d_leaves, n_leaf_boxes, w.u->p, w.rho->p,
+                                 var_args(w, lmax), hom, d_norms, d_norms + T, rout, rout_f32);
     else
         launch_leaf_residual(leaf_cfg(w.fp64, s), meta, d_leaves, n_leaf_boxes, w.u->p, w.rho->p, hom, d_norms,
                              d_norms + T, rout, rout_f32);

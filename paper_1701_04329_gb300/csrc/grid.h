@@ -135,6 +135,10 @@ class Grid {
     // eps on every level (leaves: the user's values, parents: restrictions) in both precisions
     int op = 0;
     std::unique_ptr<DevBuf> eps64, eps32;
+    std::unique_ptr<DevBuf> coef64, coef32;  // face coefficients of every cell (2D + 2 arrays of ncell values)
+    VarArgs var_args(const Workspace &w, int l) {
+        return VarArgs{eps_of(w), w.fp64 ? coef64->p : coef32->p, ncell, op, L(l).h};
+    }
     bool eps_set = false;
     double *d_x0 = nullptr;  // lower x coordinate of every box
     // prolongation of the coarse-grid correction (Sec. 2.5): 0 linear, 1 bi/trilinear, 2 zeroth order

@@ -544,16 +544,14 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
 // maxima of |r| and |rho| over the leaf cells (as bit patterns, reduced per
 // block and committed with one atomic per block when the block moves to
 // another tree, and at the end), and optionally r cast to R in rout.
-template <int D, int M, typename T, typename R>
-__global__ void __launch_bounds__(kThreads) k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
-                                                              const T *__restrict__ rho, int hom,
-                                                              unsigned long long *rmax, unsigned long long *pmax,
-                                                              R *rout) {
-    constexpr int GT = leaf_threads<D, M, T>();
+// lap(I, st, v, col, j, k, h0, out): h^2 times the operator on vector v of the box.
+template <int D, int M, typename T, typename R, int GT, typename Lap>
+__device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *list, int n, const T *u,
+                                                   const T *__restrict__ rho, int hom, unsigned long long *rmax,
+                                                   unsigned long long *pmax, R *rout, Lap lap_vec) {
     using F = FpCfg<D, M, T, GT>;
     constexpr int VEC = F::VEC, NVH = F::H / VEC;
     __shared__ unsigned long long red[64];
-    pdl_trigger();
     const int g = threadIdx.x / F::G;
     unsigned long long rm = 0, pm = 0;
     int cur = -1, tr = -1;  // tree of the running maxima, tree of this step's boxes (uniform in the block)
@@ -583,7 +581,7 @@ __global__ void __launch_bounds__(kThreads) k_leaf_residual_p(BoxMeta A, const i
             const int row = w / F::NVR, h0 = (w % F::NVR) * VEC;
             const int j = row % M, k = D == 2 ? 0 : row / M;
             T lap[VEC], rv[VEC];
-            fp_lap_vec<D, M, T>(st, col, j, k, h0, lap);
+            lap_vec(I, st, v, col, j, k, h0, lap);
             ldv<T, VEC>(FL + v * VEC, rv);
             R out[VEC];
 #pragma unroll
@@ -613,6 +611,18 @@ __global__ void __launch_bounds__(kThreads) k_leaf_residual_p(BoxMeta A, const i
     };
     fp_walk<D, M, T, GT, false>(A, 0, n, list, u, hom, want, flat, body, pre, post);  // register-bound: no own-thread fix
     flush_max(rm, pm, cur, cur >= 0, rmax, pmax, red);
+}
+
+template <int D, int M, typename T, typename R>
+__global__ void __launch_bounds__(kThreads) k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
+                                                              const T *__restrict__ rho, int hom,
+                                                              unsigned long long *rmax, unsigned long long *pmax,
+                                                              R *rout) {
+    pdl_trigger();
+    auto lap = [](const BoxInfo &, const T *st, int, int col, int j, int k, int h0, T *out) {
+        fp_lap_vec<D, M, T>(st, col, j, k, h0, out);
+    };
+    leaf_residual_walk<D, M, T, R, leaf_threads<D, M, T>()>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
 }
 
 // ---------------------------------------------------------------------------

@@ -305,11 +305,14 @@ __device__ __forceinline__ void sp_fix(const BoxInfo &I, const BoxMeta &A, const
 // resident blocks per SM the register allocation must allow (FP32 / FP64)
 constexpr int kSmoothMinBlocks32 = 6, kSmoothMinBlocks64 = 5;
 
-// scaled = 1: rho holds -h^2 rho / (2D) and the update is u = sum/(2D) + rho
-template <int D, int M, typename T, int VPT = 1>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 : kSmoothMinBlocks64) k_smooth_p(BoxMeta A, int b0, int n, const int *list, T *u,
-                                                       const T *__restrict__ rho, T h2, int colour, int hom,
-                                                       int scaled) {
+// The walk of a half-sweep: boxes staged through the ring, then per 16-byte
+// vector of colour-c cells upd(I, v, itv, xl, xr, ym, yp, zm, zp, rv, out) forms
+// the new values from the neighbours (in the order -x, +x, -y, +y, -z, +z) and
+// the staged source.  early(I, v, itv) runs for the same vectors before the
+// box's copies are waited for (loads of its own that upd needs).
+template <int D, int M, typename T, int VPT, typename Early, typename Upd>
+__device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const int *list, T *u,
+                                        const T *__restrict__ rho, int colour, int hom, Early early, Upd upd) {
     using S = SpCfg<D, M, T, VPT>;
     constexpr int VEC = S::VEC, MH = S::MH, H = S::H, NST = S::NST, NI = NST + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -317,7 +320,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 
     T *stages = reinterpret_cast<T *>(smem_raw);
     BoxInfo *info = reinterpret_cast<BoxInfo *>(smem_raw + sizeof(T) * S::BOX * S::BPC * NST);
     const int c = colour;
-    const T inv = T(1) / T(2 * D);
     const int stride = gridDim.x * S::BPC;
     const int first = blockIdx.x * S::BPC;
     SpPlan<D, M, T, VPT> pl;
@@ -351,9 +353,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 
     }
     int it = 0;
     for (int base = first; base < n; base += stride, ++it) {
-        cp_wait<NST - 2>();  // this box's copies (issued NST-1 boxes ago) have landed
         const BoxInfo &I = info[(it % NI) * S::BPC + g];
         const int b = I.b;
+        if (b >= 0) {
+#pragma unroll
+            for (int itv = 0; itv < S::NIT; ++itv)
+                if (lt + itv * S::G < S::NV) early(I, lt + itv * S::G, itv);
+        }
+        cp_wait<NST - 2>();  // this box's copies (issued NST-1 boxes ago) have landed
         const bool special = b >= 0 && (I.flag & BF_SPECIAL);
         const bool cf = b >= 0 && (I.flag & BF_CF);
         T *box = stages + ((it % NST) * S::BPC + g) * S::BOX;
@@ -388,20 +395,40 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 
                 }
                 ldv<T, VEC>(R + (lt + itv * S::G) * VEC, rv);
                 const bool r = cr[itv];
-                T out[VEC];
+                // the x neighbours: the cell's own half-row entry and the one beside it
+                // (towards +x for r = 1, towards -x for r = 0; `extra` past the vector)
+                T xl[VEC], xr[VEC], out[VEC];
 #pragma unroll
                 for (int x = 0; x < VEC; ++x) {
-                    // the x neighbours: the cell's own half-row entry and the one beside it
-                    // (towards +x for r = 1, towards -x for r = 0; `extra` past the vector)
                     const T side = r ? (x + 1 < VEC ? xv[x + 1] : extra) : (x ? xv[x - 1] : extra);
-                    const T sum = nb_sum6<D, T>(xv[x], side, ym[x], yp[x], D == 3 ? zm[x] : T(0), D == 3 ? zp[x] : T(0));
-                    out[x] = scaled ? fma(sum, inv, rv[x]) : (sum - h2 * rv[x]) * inv;
+                    xl[x] = r ? xv[x] : side;
+                    xr[x] = r ? side : xv[x];
                 }
+                upd(I, lt + itv * S::G, itv, xl, xr, ym, yp, zm, zp, rv, out);
                 stv<T, VEC>(u + I.coff + c * H + (lt + itv * S::G) * VEC, out);
             }
         }
     }
     cp_wait<0>();
+}
+
+// scaled = 1: rho holds -h^2 rho / (2D) and the update is u = sum/(2D) + rho
+template <int D, int M, typename T, int VPT = 1>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 : kSmoothMinBlocks64)
+    k_smooth_p(BoxMeta A, int b0, int n, const int *list, T *u, const T *__restrict__ rho, T h2, int colour, int hom,
+               int scaled) {
+    constexpr int VEC = SpCfg<D, M, T, VPT>::VEC;
+    const T inv = T(1) / T(2 * D);
+    auto early = [](const BoxInfo &, int, int) {};
+    auto upd = [&](const BoxInfo &, int, int, const T (&xl)[VEC], const T (&xr)[VEC], const T (&ym)[VEC],
+                   const T (&yp)[VEC], const T (&zm)[VEC], const T (&zp)[VEC], const T (&rv)[VEC], T (&out)[VEC]) {
+#pragma unroll
+        for (int x = 0; x < VEC; ++x) {
+            const T sum = nb_sum6<D, T>(xl[x], xr[x], ym[x], yp[x], D == 3 ? zm[x] : T(0), D == 3 ? zp[x] : T(0));
+            out[x] = scaled ? fma(sum, inv, rv[x]) : (sum - h2 * rv[x]) * inv;
+        }
+    };
+    sp_walk<D, M, T, VPT>(A, b0, n, list, u, rho, colour, hom, early, upd);
 }
 
 }  // namespace afg

@@ -86,15 +86,25 @@ void launch_leaf_absmax(const LaunchCfg &, const BoxMeta &, const int *list, int
                         double *partials, double *result);
 constexpr int kPartials = 4096;  // size of the partials buffer (doubles)
 
-// Variable-coefficient operators (kernels_var.cuh): op 1 div(eps grad u),
-// op 2 the same in (r,z) coordinates; eps in the field layout, same precision.
+// Variable-coefficient operators (kernels_var.cuh, kernels_var_staged.cuh): op
+// 1 div(eps grad u), op 2 the same in (r,z) coordinates; eps and the face
+// coefficients (2D + 2 arrays, n values apart) in the field layout, same
+// precision; h the level's cell size.
+struct VarArgs {
+    const void *eps, *coef;
+    long long n;
+    int op;
+    double h;
+};
 #define AFG_VAR_DECL(DD)                                                                                             \
+    void launch_var_coef_d##DD(const LaunchCfg &, const BoxMeta &, int b0, int n, const void *eps, void *out,        \
+                               long long nc, int op);                                                                \
     void launch_var_smooth_d##DD(const LaunchCfg &, const BoxMeta &, int b0, int n, void *u, const void *rho,        \
-                                 const void *eps, int colour, int hom, int op);                                      \
+                                 const VarArgs &, int colour, int hom);                                              \
     void launch_var_resid_restrict_d##DD(const LaunchCfg &, const BoxMeta &, int b0, int n, void *u, void *rho,      \
-                                         void *vold, const void *eps, int hom, int op);                              \
+                                         void *vold, const VarArgs &, int hom);                                      \
     void launch_var_fas_d##DD(const LaunchCfg &, const BoxMeta &, int b0, int n, const void *u, void *rho,           \
-                              void *vold, const void *eps, int hom, int op);                                         \
+                              void *vold, const VarArgs &, int hom);                                                 \
     void launch_var_restrict_d##DD(const LaunchCfg &, const BoxMeta &, int b0, int n, const int *list, void *v,      \
                                    int op);                                                                          \
     void launch_correct_x_d##DD(const LaunchCfg &, const BoxMeta &, int b0, int n, void *u, const void *vold,         \
@@ -103,26 +113,32 @@ constexpr int kPartials = 4096;  // size of the partials buffer (doubles)
                                const BoxMeta &An, double *un, const int *new_leaves, const int *src,                  \
                                const int *poff, int n, int scheme);                                                   \
     void launch_var_leaf_residual_d##DD(const LaunchCfg &, const BoxMeta &, const int *list, int n, const void *u,   \
-                                        const void *rho, const void *eps, int hom, int op, unsigned long long *rmax, \
+                                        const void *rho, const VarArgs &, int hom, unsigned long long *rmax,         \
                                         unsigned long long *pmax, void *rout, bool rout_f32);
 AFG_VAR_DECL(2)
 AFG_VAR_DECL(3)
 #undef AFG_VAR_DECL
 
+// face coefficients of the boxes of a level from eps on it and its neighbours
+inline void launch_var_coef(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *eps, void *out,
+                            long long nc, int op) {
+    if (c.D == 2) launch_var_coef_d2(c, A, b0, n, eps, out, nc, op);
+    else launch_var_coef_d3(c, A, b0, n, eps, out, nc, op);
+}
 inline void launch_var_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, const void *rho,
-                              const void *eps, int colour, int hom, int op) {
-    if (c.D == 2) launch_var_smooth_d2(c, A, b0, n, u, rho, eps, colour, hom, op);
-    else launch_var_smooth_d3(c, A, b0, n, u, rho, eps, colour, hom, op);
+                              const VarArgs &W, int colour, int hom) {
+    if (c.D == 2) launch_var_smooth_d2(c, A, b0, n, u, rho, W, colour, hom);
+    else launch_var_smooth_d3(c, A, b0, n, u, rho, W, colour, hom);
 }
 inline void launch_var_resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho,
-                                      void *vold, const void *eps, int hom, int op) {
-    if (c.D == 2) launch_var_resid_restrict_d2(c, A, b0, n, u, rho, vold, eps, hom, op);
-    else launch_var_resid_restrict_d3(c, A, b0, n, u, rho, vold, eps, hom, op);
+                                      void *vold, const VarArgs &W, int hom) {
+    if (c.D == 2) launch_var_resid_restrict_d2(c, A, b0, n, u, rho, vold, W, hom);
+    else launch_var_resid_restrict_d3(c, A, b0, n, u, rho, vold, W, hom);
 }
 inline void launch_var_fas(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *u, void *rho, void *vold,
-                           const void *eps, int hom, int op) {
-    if (c.D == 2) launch_var_fas_d2(c, A, b0, n, u, rho, vold, eps, hom, op);
-    else launch_var_fas_d3(c, A, b0, n, u, rho, vold, eps, hom, op);
+                           const VarArgs &W, int hom) {
+    if (c.D == 2) launch_var_fas_d2(c, A, b0, n, u, rho, vold, W, hom);
+    else launch_var_fas_d3(c, A, b0, n, u, rho, vold, W, hom);
 }
 // restriction of a field into the parents: the mean of the children (weighted by r when op == 2)
 inline void launch_var_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *v,
@@ -148,10 +164,10 @@ inline void launch_transfer(int D, cudaStream_t st, int N, const BoxMeta &Ao, co
     else launch_transfer_d3(st, N, Ao, uo, nball_o, An, un, new_leaves, src, poff, n, scheme);
 }
 inline void launch_var_leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u,
-                                     const void *rho, const void *eps, int hom, int op, unsigned long long *rmax,
+                                     const void *rho, const VarArgs &W, int hom, unsigned long long *rmax,
                                      unsigned long long *pmax, void *rout, bool rout_f32) {
-    if (c.D == 2) launch_var_leaf_residual_d2(c, A, list, n, u, rho, eps, hom, op, rmax, pmax, rout, rout_f32);
-    else launch_var_leaf_residual_d3(c, A, list, n, u, rho, eps, hom, op, rmax, pmax, rout, rout_f32);
+    if (c.D == 2) launch_var_leaf_residual_d2(c, A, list, n, u, rho, W, hom, rmax, pmax, rout, rout_f32);
+    else launch_var_leaf_residual_d3(c, A, list, n, u, rho, W, hom, rmax, pmax, rout, rout_f32);
 }
 
 }  // namespace afg

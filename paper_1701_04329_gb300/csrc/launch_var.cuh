@@ -4,15 +4,40 @@
 #pragma once
 #include "kernels_prolong.cuh"
 #include "kernels_transfer.cuh"
-#include "kernels_var.cuh"
+#include "kernels_var_staged.cuh"
 #include "launch_impl.cuh"
 
 namespace afg {
 
+// The staged kernels with stored coefficients wherever a half-row holds a
+// 16-byte vector; the others (grids of 2 cells per side, and of 4 in FP32)
+// stay on the kernels that form the coefficients from eps.
 template <int D, int M, typename T>
-void do_var_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, const void *rho, const void *eps,
-                   int colour, int hom, int op) {
+void do_var_coef(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *eps, void *coef, long long nc,
+                 int op) {
     if (n <= 0) return;
+    using S = VarCfg<D, M, T>;
+    auto k = k_var_coef<D, M, T>;
+    launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (const T *)eps,
+               (T *)coef, nc, op);
+    ++g_launches;
+}
+
+template <int D, int M, typename T>
+void do_var_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, const void *rho, const VarArgs &W,
+                   int colour, int hom) {
+    if (n <= 0) return;
+    if constexpr (SpCfg<D, M, T>::ok) {
+        using S = SpCfg<D, M, T>;
+        auto k = k_var_smooth_p<D, M, T>;
+        const VarCoef<T> V{(const T *)W.coef, W.n};
+        launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (T *)u,
+                   (const T *)rho, V, T(W.h * W.h), colour, hom);
+        ++g_launches;
+        return;
+    }
+    const void *eps = W.eps;
+    const int op = W.op;
     using S = VarCfg<D, M, T>;
     auto k = k_var_smooth<D, M, T>;
     launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (T *)u,
@@ -22,8 +47,19 @@ void do_var_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u,
 
 template <int D, int M, int MP, typename T>
 void do_var_resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho, void *vold,
-                           const void *eps, int hom, int op) {
+                           const VarArgs &W, int hom) {
     if (n <= 0) return;
+    if constexpr (FpCfg<D, M, T>::ok) {
+        using F = FpCfg<D, M, T, fas_threads<D, M, T>()>;
+        auto k = k_var_resid_restrict_p<D, M, MP, T>;
+        const VarCoef<T> V{(const T *)W.coef, W.n};
+        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, b0, n, (T *)u,
+                   (T *)rho, (T *)vold, V, T(1.0 / (W.h * W.h)), hom, W.op);
+        ++g_launches;
+        return;
+    }
+    const void *eps = W.eps;
+    const int op = W.op;
     using S = VarCfg<D, M, T>;
     auto k = k_var_resid_restrict<D, M, MP, T>;
     launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (T *)u, (T *)rho,
@@ -33,8 +69,19 @@ void do_var_resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, 
 
 template <int D, int M, typename T>
 void do_var_fas(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *u, void *rho, void *vold,
-                const void *eps, int hom, int op) {
+                const VarArgs &W, int hom) {
     if (n <= 0) return;
+    if constexpr (FpCfg<D, M, T>::ok) {
+        using F = FpCfg<D, M, T, fas_threads<D, M, T>()>;
+        auto k = k_var_fas_p<D, M, T>;
+        const VarCoef<T> V{(const T *)W.coef, W.n};
+        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, b0, n, (const T *)u,
+                   (T *)rho, (T *)vold, V, T(1.0 / (W.h * W.h)), hom);
+        ++g_launches;
+        return;
+    }
+    const void *eps = W.eps;
+    const int op = W.op;
     using S = VarCfg<D, M, T>;
     auto k = k_var_fas<D, M, T>;
     launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (const T *)u,
@@ -44,13 +91,15 @@ void do_var_fas(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void 
 
 template <int D, int M, typename T, typename Ro>
 void do_var_leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u,
-                          const void *rho, const void *eps, int hom, int op, unsigned long long *rmax,
+                          const void *rho, const VarArgs &W, int hom, unsigned long long *rmax,
                           unsigned long long *pmax, void *rout) {
     if (n <= 0) return;
-    using S = VarCfg<D, M, T>;
-    auto k = k_var_leaf_residual<D, M, T, Ro>;
-    launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, list, n, (const T *)u,
-               (const T *)rho, (const T *)eps, hom, op, rmax, pmax, (Ro *)rout);
+    static_assert(FpCfg<D, M, T>::ok, "leaf boxes have 4 cells per side or more, in FP64");
+    using F = FpCfg<D, M, T, leaf_threads<D, M, T>()>;
+    auto k = k_var_leaf_residual_p<D, M, T, Ro>;
+    const VarCoef<T> V{(const T *)W.coef, W.n};
+    launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, (const T *)u,
+               (const T *)rho, V, hom, rmax, pmax, (Ro *)rout);
     ++g_launches;
 }
 
@@ -106,53 +155,69 @@ struct VarOps {
         AFG_SWITCH_MMP(c.M, c.MP, (do_correct_x<D, MM, PP, T>(c, A, b0, n, u, vold, nball, scheme)));
     }
     template <typename T>
-    static void smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, const void *rho, const void *eps,
-                       int colour, int hom, int op) {
-        AFG_SWITCH_M(c.M, (do_var_smooth<D, MM, T>(c, A, b0, n, u, rho, eps, colour, hom, op)));
+    static void coef(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *eps, void *out, long long nc,
+                     int op) {
+        AFG_SWITCH_M(c.M, (do_var_coef<D, MM, T>(c, A, b0, n, eps, out, nc, op)));
+    }
+    template <typename T>
+    static void smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, const void *rho, const VarArgs &W,
+                       int colour, int hom) {
+        AFG_SWITCH_M(c.M, (do_var_smooth<D, MM, T>(c, A, b0, n, u, rho, W, colour, hom)));
     }
     template <typename T>
     static void resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho, void *vold,
-                               const void *eps, int hom, int op) {
-        AFG_SWITCH_MMP(c.M, c.MP, (do_var_resid_restrict<D, MM, PP, T>(c, A, b0, n, u, rho, vold, eps, hom, op)));
+                               const VarArgs &W, int hom) {
+        AFG_SWITCH_MMP(c.M, c.MP, (do_var_resid_restrict<D, MM, PP, T>(c, A, b0, n, u, rho, vold, W, hom)));
     }
     template <typename T>
     static void fas(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *u, void *rho, void *vold,
-                    const void *eps, int hom, int op) {
-        AFG_SWITCH_M(c.M, (do_var_fas<D, MM, T>(c, A, b0, n, u, rho, vold, eps, hom, op)));
+                    const VarArgs &W, int hom) {
+        AFG_SWITCH_M(c.M, (do_var_fas<D, MM, T>(c, A, b0, n, u, rho, vold, W, hom)));
     }
     template <typename T>
     static void restrict_v(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *v, int op) {
         AFG_SWITCH_MMP(c.M, c.MP, (do_var_restrict<D, MM, PP, T>(c, A, b0, n, list, v, op)));
     }
     static void leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u,
-                              const void *rho, const void *eps, int hom, int op, unsigned long long *rmax,
+                              const void *rho, const VarArgs &W, int hom, unsigned long long *rmax,
                               unsigned long long *pmax, void *rout, bool rout_f32) {
-        if (rout_f32) {
-            AFG_SWITCH_M(c.M, (do_var_leaf_residual<D, MM, double, float>(c, A, list, n, u, rho, eps, hom, op, rmax,
-                                                                          pmax, rout)));
-        } else {
-            AFG_SWITCH_M(c.M, (do_var_leaf_residual<D, MM, double, double>(c, A, list, n, u, rho, eps, hom, op, rmax,
-                                                                           pmax, rout)));
+        switch (c.M) {
+            case 4: go<4>(c, A, list, n, u, rho, W, hom, rmax, pmax, rout, rout_f32); break;
+            case 8: go<8>(c, A, list, n, u, rho, W, hom, rmax, pmax, rout, rout_f32); break;
+            case 16: go<16>(c, A, list, n, u, rho, W, hom, rmax, pmax, rout, rout_f32); break;
+            default: bad_size(c.M, 0);
         }
+    }
+    template <int M>
+    static void go(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u, const void *rho,
+                   const VarArgs &W, int hom, unsigned long long *rmax, unsigned long long *pmax, void *rout,
+                   bool rout_f32) {
+        if (rout_f32) do_var_leaf_residual<D, M, double, float>(c, A, list, n, u, rho, W, hom, rmax, pmax, rout);
+        else do_var_leaf_residual<D, M, double, double>(c, A, list, n, u, rho, W, hom, rmax, pmax, rout);
     }
 };
 
 // the entry points of launch.h for one dimension
 #define AFG_VAR_LAUNCHES(DD)                                                                                          \
+    void launch_var_coef_d##DD(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *eps, void *out,       \
+                               long long nc, int op) {                                                                \
+        if (c.fp64) VarOps<DD>::coef<double>(c, A, b0, n, eps, out, nc, op);                                          \
+        else VarOps<DD>::coef<float>(c, A, b0, n, eps, out, nc, op);                                                  \
+    }                                                                                                                 \
     void launch_var_smooth_d##DD(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, const void *rho,       \
-                                 const void *eps, int colour, int hom, int op) {                                      \
-        if (c.fp64) VarOps<DD>::smooth<double>(c, A, b0, n, u, rho, eps, colour, hom, op);                            \
-        else VarOps<DD>::smooth<float>(c, A, b0, n, u, rho, eps, colour, hom, op);                                    \
+                                 const VarArgs &W, int colour, int hom) {                                             \
+        if (c.fp64) VarOps<DD>::smooth<double>(c, A, b0, n, u, rho, W, colour, hom);                                  \
+        else VarOps<DD>::smooth<float>(c, A, b0, n, u, rho, W, colour, hom);                                          \
     }                                                                                                                 \
     void launch_var_resid_restrict_d##DD(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho,     \
-                                         void *vold, const void *eps, int hom, int op) {                              \
-        if (c.fp64) VarOps<DD>::resid_restrict<double>(c, A, b0, n, u, rho, vold, eps, hom, op);                      \
-        else VarOps<DD>::resid_restrict<float>(c, A, b0, n, u, rho, vold, eps, hom, op);                              \
+                                         void *vold, const VarArgs &W, int hom) {                                     \
+        if (c.fp64) VarOps<DD>::resid_restrict<double>(c, A, b0, n, u, rho, vold, W, hom);                            \
+        else VarOps<DD>::resid_restrict<float>(c, A, b0, n, u, rho, vold, W, hom);                                    \
     }                                                                                                                 \
     void launch_var_fas_d##DD(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *u, void *rho,          \
-                              void *vold, const void *eps, int hom, int op) {                                         \
-        if (c.fp64) VarOps<DD>::fas<double>(c, A, b0, n, u, rho, vold, eps, hom, op);                                 \
-        else VarOps<DD>::fas<float>(c, A, b0, n, u, rho, vold, eps, hom, op);                                         \
+                              void *vold, const VarArgs &W, int hom) {                                                \
+        if (c.fp64) VarOps<DD>::fas<double>(c, A, b0, n, u, rho, vold, W, hom);                                       \
+        else VarOps<DD>::fas<float>(c, A, b0, n, u, rho, vold, W, hom);                                               \
     }                                                                                                                 \
     void launch_var_restrict_d##DD(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *v,     \
                                    int op) {                                                                          \
@@ -170,9 +235,9 @@ struct VarOps {
         VarOps<DD>::transfer(st, N, Ao, uo, nball_o, An, un, new_leaves, src, poff, n, scheme);                       \
     }                                                                                                                 \
     void launch_var_leaf_residual_d##DD(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u,  \
-                                        const void *rho, const void *eps, int hom, int op, unsigned long long *rmax,  \
+                                        const void *rho, const VarArgs &W, int hom, unsigned long long *rmax,         \
                                         unsigned long long *pmax, void *rout, bool rout_f32) {                        \
-        VarOps<DD>::leaf_residual(c, A, list, n, u, rho, eps, hom, op, rmax, pmax, rout, rout_f32);                   \
+        VarOps<DD>::leaf_residual(c, A, list, n, u, rho, W, hom, rmax, pmax, rout, rout_f32);                         \
     }
 
 }  // namespace afg
