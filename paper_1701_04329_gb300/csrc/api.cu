@@ -398,7 +398,8 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
 }
 
 void set_dirichlet_dev(Grid &g, const double *b, cudaStream_t s) {
-    g.faces_changed = true;
+    for (auto &p : g.coarse_plans)
+        for (auto &c : p) c.faces_stale = true;
     if (g.n_bfaces > 0) {
         if (b) check(cudaMemcpyAsync(g.d_bc, b, g.n_bfaces * 8, cudaMemcpyDeviceToDevice, s), "copy b");
         else check(cudaMemsetAsync(g.d_bc, 0, g.n_bfaces * 8, s), "zero b");

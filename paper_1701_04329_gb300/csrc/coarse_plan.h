@@ -28,6 +28,16 @@ struct CoarseArgs {
     int nface = 0;                    // faces of one block's levels on the domain sides (at most)
     const int *fslot = nullptr;       // per block of a cluster: their ghost slots, -1 past the last
     double *fval = nullptr;           // per block: their boundary values
+    // variable coefficients: operator, per level its arrays (csz apart), all
+    // of them contiguous, 16-byte aligned; the packed image per block, and
+    // where mode 3 gathers it from
+    int op = 0, N = 0;
+    int oc[kCoarseMaxLevels], csz[kCoarseMaxLevels];
+    int ocoef = 0, ncoef = 0;
+    void *cpack = nullptr;
+    const void *coef = nullptr;
+    long long coef_n = 0;
+    const int *dtab[kCoarseMaxLevels];  // every level's boxes by position, per tree
     const int *dbox = nullptr;        // top level's boxes by position, per tree
     const int *tree_bc = nullptr;     // per tree: Neumann sides | periodic axes << 6
 };
@@ -36,21 +46,22 @@ inline unsigned coarse_magic(int d) { return d == 1 ? 0u : (unsigned)((((unsigne
 
 // Grids of 2 .. M cells per root box side for a block of nroot roots; ntrees
 // blocks run side by side.  Returns the shared memory of one block in bytes.
-inline size_t coarse_plan(int D, bool fp64, int M, int N, const int *nroot, int ntrees, CoarseArgs &G) {
+inline size_t coarse_plan(int D, bool fp64, int M, int N, const int *nroot, int ntrees, CoarseArgs &G,
+                          bool var = false) {
     G = CoarseArgs();
+    G.N = N;
     G.mb = std::min(M, N);
     while ((1 << G.lgmb) < G.mb) ++G.lgmb;
     const int f = M / G.mb;
     G.nbx = nroot[0] * f;
     G.nby = nroot[1] * f;
     G.nbz = D == 3 ? nroot[2] * f : 1;
-    // FP64 grids are spread over the cluster's blocks from this many cells on
-    // (one SM's FP64 rate: 16^3 on one block 130 us a visit, on eight 62 us);
-    // below, and in FP32 at any size that fits, a half-sweep costs less than
-    // the cluster barrier that spreading adds (16^3 FP32: 2300 cycles a
-    // half-sweep on one block at first, 1500 on eight; 32^3 on eight 3700,
-    // no better than the per-level launches).
-    const long long spread = fp64 ? 4096 : 1 << 30;
+    // A grid is spread over the cluster's blocks from this many cells on: below,
+    // a half-sweep costs less than the cluster barrier (350-450 cycles) that
+    // spreading adds.  16^3: FP64 62 us a visit on eight blocks, 130 us on one
+    // (one SM's FP64 rate); FP32 solves 1-10 % faster on eight (the 3 x 2 block
+    // of roots 4.4 -> 4.0 ms, 3D gradients 16.1 -> 15.8 ms).
+    const long long spread = 4096;
     size_t off = 0, dc = 0;
     for (int m = 2; m <= M; m *= 2) {
         const int li = G.nl++;
@@ -82,6 +93,18 @@ inline size_t coarse_plan(int D, bool fp64, int M, int N, const int *nroot, int 
     }
     G.odc = (int)off;
     off += dc;
+    if (var) {
+        off = (off + 3) / 4 * 4;
+        G.ocoef = (int)off;
+        for (int li = 0; li < G.nl; ++li) {
+            const size_t padded = (size_t)(G.P[li] + 2) * (G.nx[li] + 2) * (D == 3 ? G.ny[li] + 2 : 1);
+            G.csz[li] = (int)((padded + 1) / 2 * 2);
+            G.oc[li] = (int)off;
+            off += (size_t)G.csz[li] * (2 * D + 2);
+        }
+        off = (off + 3) / 4 * 4;
+        G.ncoef = (int)off - G.ocoef;
+    }
     G.total = (int)off;
     G.slab_boxes = G.nbx * G.nby * G.nbz;
     if (G.nr[G.nl - 1] > 1) {

@@ -455,9 +455,14 @@ void Grid::plan_coarse(const std::vector<const HostTree *> &trees, const std::ve
     auto table = [&](int l) {
         auto it = tables.find(l);
         if (it != tables.end()) return it->second;
+        std::vector<int> v;
+        if (l < 1) {  // one box per tree (trees of one root box)
+            for (int t = 0; t < T; ++t) v.push_back(L(l).b0 + t);
+            return tables[l] = upload(v, owned);
+        }
         const int f = 1 << (l - 1);
         const int sx = nr[0] * f, sy = nr[1] * f, sz = D == 3 ? nr[2] * f : 1;
-        std::vector<int> v((size_t)T * sx * sy * sz);
+        v.resize((size_t)T * sx * sy * sz);
         for (int t = 0; t < T; ++t)
             for (int b = trees[t]->lstart[l]; b < trees[t]->lstart[l] + trees[t]->lcount[l]; ++b) {
                 const HBox &x = trees[t]->boxes[b];
@@ -466,53 +471,65 @@ void Grid::plan_coarse(const std::vector<const HostTree *> &trees, const std::ve
             }
         return tables[l] = upload(v, owned);
     };
-    for (const bool fp64 : {false, true}) {
-        Coarse &c = fp64 ? coarse64 : coarse32;
-        for (int l = 1; l <= full; ++l) {
-            CoarseArgs plan;
-            const long long m = (long long)N << (l - 1);
-            if (m > 1024) break;
-            const size_t smem = coarse_plan(D, fp64, (int)m, N, nr, T, plan);
-            const int li = plan.nl - 1;
-            const long long work = (long long)plan.nx[li] * plan.ny[li] * plan.P[li] / 2;  // cells of a half-sweep per block
-            // up to this much the launch beats the level's 11 launches of 2.1 us (FP32)
-            // or 3.3 us (FP64): a 64^2 grid's half-sweep takes 0.75 us (FP32, one
-            // block) and 1.2 us (FP64, eight blocks), a 32^3 grid's 1.8 and 6.7 us
-            const long long most = fp64 ? 512 : 2048;
-            if (l > 1 && (smem > max_smem_optin() || work > most)) break;
-            c.top = l;
-            c.plan = plan;
-            c.smem = smem;
+    for (int fp64 = 0; fp64 < 2; ++fp64)
+        for (int var = 0; var < (block ? 1 : 2); ++var) {
+            Coarse &c = coarse_plans[fp64][var];
+            for (int l = lmin; l <= full; ++l) {
+                if (!var && l < 1) continue;
+                CoarseArgs plan;
+                const long long m = l >= 1 ? (long long)N << (l - 1) : N >> (1 - l);
+                if (m > 1024) break;
+                const size_t smem = coarse_plan(D, fp64, (int)m, N, nr, T, plan, var);
+                const int li = plan.nl - 1;
+                // cells of a half-sweep per block
+                const long long work = (long long)plan.nx[li] * plan.ny[li] * plan.P[li] / 2;
+                // up to this much the launch beats the level's 11 launches of 2.1 us (FP32)
+                // or 3.3 us (FP64): a 64^2 grid's half-sweep takes 1.2 us in FP64 on eight
+                // blocks, a 32^3 grid's 6.7 us in FP64 and 1-1.8 us in FP32
+                const long long most = fp64 ? 512 : 2048;
+                if (smem > max_smem_optin() || (c.ok && work > most)) break;
+                c.top = l;
+                c.plan = plan;
+                c.smem = smem;
+                c.ok = true;
+            }
+            if (!c.ok) continue;
+            c.plan.dbox = table(c.top);
+            if (var)
+                for (int li = 0; li < c.plan.nl; ++li) c.plan.dtab[li] = table(lmin + li);
+            c.plan.tree_bc = d_bc_types;
+            // faces: the slots of every non-periodic axis in any tree (a tree's own periodic sides are not read)
+            int all = 7;
+            for (int code : bc) all &= code >> 6;
+            std::vector<std::vector<int>> slots;
+            size_t most_faces = 0;
+            for (int r = 0; r < c.plan.R; ++r) {
+                slots.push_back(coarse_faces(D, c.plan, r, all));
+                most_faces = std::max(most_faces, slots.back().size());
+            }
+            std::vector<int> flat;
+            for (auto &v : slots) {
+                v.resize(most_faces, -1);
+                flat.insert(flat.end(), v.begin(), v.end());
+            }
+            c.plan.nface = (int)most_faces;
+            c.plan.fslot = upload(flat, owned);
+            if (fp64) c.plan.fval = upload(std::vector<double>(most_faces * c.plan.R * T, 0.0), owned);
         }
-        c.plan.dbox = table(c.top);
-        c.plan.tree_bc = d_bc_types;
-        // faces: the slots of every non-periodic axis in any tree (a tree's own periodic sides are not read)
-        int all = 7;
-        for (int code : bc) all &= code >> 6;
-        std::vector<std::vector<int>> slots;
-        size_t most_faces = 0;
-        for (int r = 0; r < c.plan.R; ++r) {
-            slots.push_back(coarse_faces(D, c.plan, r, all));
-            most_faces = std::max(most_faces, slots.back().size());
-        }
-        std::vector<int> flat;
-        for (auto &v : slots) {
-            v.resize(most_faces, -1);
-            flat.insert(flat.end(), v.begin(), v.end());
-        }
-        c.plan.nface = (int)most_faces;
-        c.plan.fslot = upload(flat, owned);
-        if (fp64) c.plan.fval = upload(std::vector<double>(most_faces * c.plan.R * T, 0.0), owned);
-    }
+}
+
+void Grid::launch_plan(Coarse &c, bool fp64, int mode, const BoxMeta &A, Workspace &w, cudaStream_t s) {
+    CoarseArgs G = c.plan;
+    G.mode = mode;
+    launch_coarse(cfg(1, fp64, s), A, G, c.smem, T, w.u->p, w.rho->p, w.vold->p);
 }
 
 // the coarse launch's copy of the boundary data, after it changed (not captured)
 void Grid::refresh_faces(cudaStream_t s) {
-    if (!faces_changed || levels_path()) return;
-    CoarseArgs G = coarse64.plan;
-    G.mode = 2;
-    launch_coarse(cfg(1, true, s), meta, G, coarse64.smem, T, ws64.u->p, ws64.rho->p, ws64.vold->p);
-    faces_changed = false;
+    Coarse &c = coarse_plans[1][op != 0];
+    if (!c.faces_stale || levels_path()) return;
+    launch_plan(c, true, 2, meta, ws64, s);
+    c.faces_stale = false;
 }
 
 void Grid::coarse_cycle(Workspace &w, int mode, const MgOpts &o, int hom, const int *active, cudaStream_t s) {
@@ -521,6 +538,7 @@ void Grid::coarse_cycle(Workspace &w, int mode, const MgOpts &o, int hom, const 
     const Coarse &c = coarse(w);
     CoarseArgs G = c.plan;
     G.mode = mode;
+    G.op = op;
     G.nd = o.n_down;
     G.nu = o.n_up;
     G.nb = o.n_base;
@@ -650,6 +668,17 @@ void Grid::set_eps(const double *eps_leaf, cudaStream_t s) {
     for (int l = lmin; l <= lmax; ++l) {
         launch_var_coef(cfg(l, true, s), meta, L(l).b0, L(l).nb, eps64->p, coef64->p, ncell, op);
         launch_var_coef(cfg(l, false, s), meta, L(l).b0, L(l).nb, eps32->p, coef32->p, ncell, op);
+    }
+    for (int fp64 = 0; fp64 < 2 && !roots_levels; ++fp64) {  // the coarse launch's packed copies
+        Coarse &c = coarse_plans[fp64][1];
+        if (!c.ok) continue;
+        if (!c.cpack) c.cpack.reset(new DevBuf((size_t)c.plan.ncoef * c.plan.R * T * (fp64 ? 8 : 4)));
+        check(cudaMemsetAsync(c.cpack->p, 0, c.cpack->bytes, s), "memset");
+        c.plan.cpack = c.cpack->p;
+        c.plan.coef = fp64 ? coef64->p : coef32->p;
+        c.plan.coef_n = ncell;
+        c.plan.op = op;
+        launch_plan(c, fp64, 3, meta, ws64, s);
     }
     eps_set = true;
 }

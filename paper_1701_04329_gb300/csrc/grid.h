@@ -95,17 +95,21 @@ class Grid {
     // below level 1 (the coarse launch keeps those grids in shared memory)
     bool block = false;
     // the levels that run in one launch per cycle (kernels_coarse.cuh), per
-    // precision: the highest one, the launch's plan and its shared memory
+    // precision and for the variable-coefficient operators: the highest one,
+    // the launch's plan, its shared memory, and what it has yet to gather
     struct Coarse {
         int top = 1;
         CoarseArgs plan;
         size_t smem = 0;
+        bool ok = false;            // false: the per-level kernels all the way down
+        bool faces_stale = false;   // boundary data newer than the plan's copy
+        std::unique_ptr<DevBuf> cpack;
     };
-    Coarse coarse32, coarse64;
-    bool faces_changed = false;  // boundary data newer than the coarse launch's copy
-    void refresh_faces(cudaStream_t s);
-    const Coarse &coarse(const Workspace &w) const { return w.fp64 ? coarse64 : coarse32; }
+    Coarse coarse_plans[2][2];  // [fp64][op != 0]
+    Coarse &coarse(const Workspace &w) { return coarse_plans[w.fp64][op != 0]; }
     void plan_coarse(const std::vector<const HostTree *> &trees, const std::vector<std::vector<int>> &gid);
+    void refresh_faces(cudaStream_t s);
+    void launch_plan(Coarse &c, bool fp64, int mode, const BoxMeta &A, Workspace &w, cudaStream_t s);
     std::vector<Level> lv;
     Level &L(int l) { return lv[l - lmin]; }
     int nbox = 0, n_leaf_boxes = 0;
@@ -144,8 +148,8 @@ class Grid {
     // prolongation of the coarse-grid correction (Sec. 2.5): 0 linear, 1 bi/trilinear, 2 zeroth order
     int prolong = 0;
     int *d_nball = nullptr;  // same-level neighbour of every box in all 3^D - 1 directions, -1 none
-    // variable coefficients or another prolongation: every level on the per-level kernels
-    bool levels_path() const { return op != 0 || prolong != 0 || roots_levels; }
+    // another prolongation, or no coarse launch: every level on the per-level kernels
+    bool levels_path() const { return prolong != 0 || roots_levels || !coarse_plans[1][op != 0].ok; }
     int vpt = 1;  // FP32 half-sweep: 16-byte vectors per thread (the threads-per-box option)
     // trees of several root boxes whose coarse grids are device boxes (one per
     // root and level): the cycle runs on the per-level kernels

@@ -24,6 +24,10 @@
 // neighbours without a branch; the ghost slots of the source hold b.  v' of
 // level top stays in global memory.
 //
+// Variable coefficients (VAR; kernels_var_staged.cuh): every level's 2D + 2
+// coefficient arrays lie in shared memory too, copied from a packed image that
+// is gathered once per eps (mode 3).
+//
 // What bounds a step is its own chain of instructions: it runs once per warp,
 // so its instruction fetches count as much as its shared-memory latencies.
 // The steps are therefore short: one copy for all levels (the sizes are
@@ -36,12 +40,16 @@
 // 62 us on eight blocks (11 launches and a one-block bottom before: 87 us).
 // Whole solves: 31 k unknowns in 2D, FP64, 2.89 -> 2.22 ms; 73 k unknowns on
 // a 3 x 2 block of root boxes, mixed, 7.40 -> 4.67 ms; 12 small quadtrees,
-// FP64, 2.30 -> 1.82 ms.  A half-sweep of a small grid is then 225 cycles in
+// FP64, 2.30 -> 1.82 ms.  With variable coefficients (every level below them
+// on per-level launches before): 107 k unknowns in 2D, FP64, 6.57 -> 3.56 ms;
+// (r,z), 294 k, mixed, 5.80 -> 2.50 ms; 3D, 3.5 M, mixed, 7.96 -> 5.70 ms.  A half-sweep of a small grid is then 225 cycles in
 // FP32; in FP64 about 1100, of which the exact neighbour sum takes 285 and
 // every dependent FP64 operation 64-76.  A cluster barrier costs 350-450.
 #pragma once
 #include "coarse_plan.h"
 #include "kernels.cuh"
+#include "kernels_smooth.cuh"  // cp_async
+#include "var_ops.cuh"
 
 namespace afg {
 
@@ -187,9 +195,10 @@ __device__ __forceinline__ void co_put(const CoLevel<D, T> &L, int a, const CoEd
 // One cell of a thread that relaxes the same cells in every half-sweep: its
 // slot, scaled source, and per axis the ghost that depends on it (offset of
 // its slot, 0 for none; value fma(m, b, +-u)).
-template <typename T>
+template <int D, typename T, bool VAR>
 struct CoCell {
     int p, ox, oy, oz;
+    T c[VAR ? 2 * D + 2 : 1];  // VAR: the coefficient arrays' values
     T rs, mx, bx, my, by, mz, bz;
     bool nx, ny, nz;  // the ghost takes +u (Neumann, periodic), not -u
 };
@@ -200,12 +209,35 @@ __device__ __forceinline__ T co_ghost_of(T m, T b, bool plus, T val) {
     return HB ? fma(m, b, v) : v;
 }
 
+// the neighbours of a cell in the order -x, +x, -y, +y, -z, +z
+template <int D, typename T>
+__device__ __forceinline__ void co_neighbours(const T *a, int W, int PS, T (&x)[2 * D]) {
+    x[0] = a[-1];
+    x[1] = a[1];
+    if constexpr (D == 3) {
+        x[2] = a[-W];
+        x[3] = a[W];
+    }
+    x[2 * D - 2] = a[-PS];
+    x[2 * D - 1] = a[PS];
+}
+
+// sum_s c_s u_s of the cell at a, its coefficients at c, n apart
+template <int D, typename T>
+__device__ __forceinline__ T co_dot(const T *c, int n, const T *a, int W, int PS) {
+    T x[2 * D], k[2 * D];
+    co_neighbours<D, T>(a, W, PS, x);
+#pragma unroll
+    for (int s = 0; s < 2 * D; ++s) k[s] = c[s * n];
+    return var_dot<D, T>(k, x);
+}
+
 // Red-black steps, one barrier per half-sweep (cells of one colour read only
 // the other): u = sum/(2D) - h^2 rho/(2D).  A thread keeps its place (h, j)
 // in the planes and walks along the last axis.  Where that leaves it one cell
 // of each colour at most, everything about them but u stays in registers, and
 // a half-sweep is the loads of the neighbours, the sum and the stores.
-template <int D, typename T, bool BC, bool HB>
+template <int D, typename T, bool BC, bool HB, bool VAR>
 __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
     const CoarseArgs &S = co_plan();
     T *sm = co_mem<T>();
@@ -215,12 +247,14 @@ __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
     const int g = ng > 1 ? co_div(threadIdx.x, S.mp[li]) : 0;
     const int first = threadIdx.x - g * plane;
     const T inv = T(1) / T(2 * D), chat = (T(-1) / T(2 * D)) * co_pow2<T>(-2 * L.lg);
+    const T h2 = co_pow2<T>(-2 * L.lg);
+    const T *cf = sm + S.oc[li];
     T *u = sm + L.u;
     const T *r = sm + L.r;
     const unsigned mh = S.mh[li];
     if (L.P <= ng && plane <= nt) {
         const bool on = g < L.P && first < plane;
-        CoCell<T> c[2];
+        CoCell<D, T, VAR> c[2];
         unsigned far = 0;  // address of the array in the block across the slab's edge
         if (on) {
             const int j = D == 3 ? co_div(first, mh) : 0, x = first - j * hx, par = (j + L.z0 + g + D) & 1;
@@ -229,11 +263,15 @@ __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
             if (oz) far = oz < 0 ? E.lo : E.hi;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {  // q: colour
-                CoCell<T> &w = c[q];
+                CoCell<D, T, VAR> &w = c[q];
                 const int up = q ? 1 - par : par;  // the cell at i = 2x + up
                 const int ox = up ? (x == hx - 1 ? 1 : 0) : (x == 0 ? -1 : 0);
                 w.p = L.slot(2 * x + up, j, g);
-                w.rs = r[w.p] * chat;
+                w.rs = r[w.p] * (VAR ? -h2 : chat);  // -h^2 rho, exactly, or -h^2 rho / (2D)
+                if (VAR) {
+#pragma unroll
+                    for (int f = 0; f < 2 * D + 2; ++f) w.c[f] = cf[f * S.csz[li] + w.p];
+                }
                 auto side = [&](int axis, int o, int stride, int n, int &off, T &m, T &b, bool &plus) {
                     const int s = 2 * axis + (o > 0);
                     const bool per = BC && ((bc >> (6 + axis)) & 1), neu = BC && ((bc >> s) & 1);
@@ -248,11 +286,20 @@ __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
                 if (far) w.oz = -oz * L.P * L.PS;
             }
         }
-        auto relax = [&](const CoCell<T> &w) {
+        auto relax = [&](const CoCell<D, T, VAR> &w) {
             T *a = u + w.p;
-            const T sum = D == 2 ? nb_sum6<D, T>(a[-1], a[1], a[-L.PS], a[L.PS], T(0), T(0))
-                                 : nb_sum6<D, T>(a[-1], a[1], a[-L.W], a[L.W], a[-L.PS], a[L.PS]);
-            const T val = fma(sum, inv, w.rs);
+            T val;
+            if constexpr (VAR) {
+                T x[2 * D], k[2 * D];
+                co_neighbours<D, T>(a, L.W, L.PS, x);
+#pragma unroll
+                for (int s = 0; s < 2 * D; ++s) k[s] = w.c[s];
+                val = var_quot<T>(var_dot<D, T>(k, x) + w.rs, w.c[2 * D], w.c[2 * D + 1]);
+            } else {
+                const T sum = D == 2 ? nb_sum6<D, T>(a[-1], a[1], a[-L.PS], a[L.PS], T(0), T(0))
+                                     : nb_sum6<D, T>(a[-1], a[1], a[-L.W], a[L.W], a[-L.PS], a[L.PS]);
+                val = fma(sum, inv, w.rs);
+            }
             a[0] = val;
             if (w.ox) a[w.ox] = co_ghost_of<T, BC, HB>(w.mx, w.bx, w.nx, val);
             if (D == 3 && w.oy) a[w.oy] = co_ghost_of<T, BC, HB>(w.my, w.by, w.ny, val);
@@ -263,7 +310,7 @@ __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
         };
         for (int half = 0; half < 2 * steps; ++half) {  // one copy of the body: its fetches count
             if (on) relax(c[0]);
-            const CoCell<T> t = c[0];
+            const CoCell<D, T, VAR> t = c[0];
             c[0] = c[1];
             c[1] = t;
             co_sync(L.nr);
@@ -277,10 +324,18 @@ __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
                 for (int k = g; k < L.P; k += ng) {
                     const int i = 2 * x + ((sweep + j + L.z0 + k + D) & 1);
                     const int p = L.slot(i, j, k);
-                    const T sum = D == 2
-                                      ? nb_sum6<D, T>(u[p - 1], u[p + 1], u[p - L.PS], u[p + L.PS], T(0), T(0))
-                                      : nb_sum6<D, T>(u[p - 1], u[p + 1], u[p - L.W], u[p + L.W], u[p - L.PS], u[p + L.PS]);
-                    co_put<D, T, BC, HB>(L, L.u, E, bc, p, i, j, k, fma(sum, inv, r[p] * chat));
+                    T val;
+                    if constexpr (VAR) {
+                        const int n = S.csz[li];
+                        val = var_quot<T>(fma(-h2, r[p], co_dot<D, T>(cf + p, n, u + p, L.W, L.PS)),
+                                          cf[2 * D * n + p], cf[(2 * D + 1) * n + p]);
+                    } else {
+                        const T sum = D == 2 ? nb_sum6<D, T>(u[p - 1], u[p + 1], u[p - L.PS], u[p + L.PS], T(0), T(0))
+                                             : nb_sum6<D, T>(u[p - 1], u[p + 1], u[p - L.W], u[p + L.W], u[p - L.PS],
+                                                             u[p + L.PS]);
+                        val = fma(sum, inv, r[p] * chat);
+                    }
+                    co_put<D, T, BC, HB>(L, L.u, E, bc, p, i, j, k, val);
                 }
             }
         co_sync(L.nr);
@@ -288,9 +343,13 @@ __device__ __noinline__ void co_smooth(int li, int steps, int rank, int bc) {
 }
 
 // h^2 A u at slot p (FP64 adds, as in the per-level kernel of the coarse right-hand side)
-template <int D, typename T>
-__device__ __forceinline__ T co_lap(const CoLevel<D, T> &L, int p) {
+template <int D, typename T, bool VAR>
+__device__ __forceinline__ T co_lap(const CoarseArgs &S, const CoLevel<D, T> &L, int li, int p) {
     const T *u = co_mem<T>() + L.u;
+    if constexpr (VAR) {
+        const T *cf = co_mem<T>() + S.oc[li] + p;
+        return fma(-cf[2 * D * S.csz[li]], u[p], co_dot<D, T>(cf, S.csz[li], u + p, L.W, L.PS));
+    }
     if (D == 2) return nb_lap6<D, T, false>(u[p], u[p - 1], u[p + 1], u[p - L.PS], u[p + L.PS], T(0), T(0));
     return nb_lap6<D, T, false>(u[p], u[p - 1], u[p + 1], u[p - L.W], u[p + L.W], u[p - L.PS], u[p + L.PS]);
 }
@@ -299,7 +358,7 @@ __device__ __forceinline__ T co_lap(const CoLevel<D, T> &L, int p) {
 // children, then rho = I r + A u): Eq. residual and Eq. coarse-rhs.  When
 // level li is spread over the blocks and li - 1 is not, every block stores
 // its coarse values in all of them.
-template <int D, typename T, bool BC, bool HB>
+template <int D, typename T, bool BC, bool HB, bool VAR>
 __device__ __noinline__ void co_down(int li, int rank, int bc) {
     const CoarseArgs &S = co_plan();
     T *sm = co_mem<T>();
@@ -314,23 +373,45 @@ __device__ __noinline__ void co_down(int li, int rank, int bc) {
     for (int c = threadIdx.x; c < n; c += nt) {
         int X, Y, Z;
         co_decode<D>(c, C.nx, mx, C.ny, my, X, Y, Z);
-        T su = T(0), sro = T(0), sout = T(0);
-        // sum_c (A u)_c = (sum_outside - D sum_c u) / h^2 over the 2^D children
+        T mu, rr;
+        if constexpr (VAR) {
+            const int nf = S.csz[li], rz = S.op == 2;
+            const T *cf = sm + S.oc[li];
+            T su = T(0), sr = T(0), sw = T(0);
+#pragma unroll 1
+            for (int q = 0; q < (1 << D); ++q) {
+                const int i = 2 * X + (q & 1), j = D == 3 ? 2 * Y + ((q >> 1) & 1) : 0, k = 2 * Z + (q >> (D - 1));
+                const int p = L.slot(i, j, k);
+                const T uu = sm[L.u + p];
+                const T lap = fma(-cf[2 * D * nf + p], uu, co_dot<D, T>(cf + p, nf, sm + L.u + p, L.W, L.PS));
+                const T res = fma(-lap, ih2, sm[L.r + p]);
+                const T wt = rz ? (T(i) + T(0.5)) * L.h() : T(1);
+                su += wt * uu;
+                sr += wt * res;
+                sw += wt;
+            }
+            mu = rz ? su / sw : su * w;
+            rr = rz ? sr / sw : sr * w;
+        } else {
+            T su = T(0), sro = T(0), sout = T(0);
+            // sum_c (A u)_c = (sum_outside - D sum_c u) / h^2 over the 2^D children
 #pragma unroll
-        for (int dz = 0; dz < 2; ++dz)
+            for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
-            for (int dy = 0; dy < (D == 3 ? 2 : 1); ++dy)
+                for (int dy = 0; dy < (D == 3 ? 2 : 1); ++dy)
 #pragma unroll
-                for (int dx = 0; dx < 2; ++dx) {
-                    const int p = L.slot(2 * X + dx, 2 * Y + dy, 2 * Z + dz);
-                    const T *u = sm + L.u + p;
-                    su += u[0];
-                    sro += sm[L.r + p];
-                    sout += u[dx ? 1 : -1];
-                    if (D == 3) sout += u[dy ? L.W : -L.W];
-                    sout += u[dz ? L.PS : -L.PS];
-                }
-        const T mu = su * w, rr = fma(-ih2, fma(T(-D), su, sout), sro) * w;
+                    for (int dx = 0; dx < 2; ++dx) {
+                        const int p = L.slot(2 * X + dx, 2 * Y + dy, 2 * Z + dz);
+                        const T *u = sm + L.u + p;
+                        su += u[0];
+                        sro += sm[L.r + p];
+                        sout += u[dx ? 1 : -1];
+                        if (D == 3) sout += u[dy ? L.W : -L.W];
+                        sout += u[dz ? L.PS : -L.PS];
+                    }
+            mu = su * w;
+            rr = fma(-ih2, fma(T(-D), su, sout), sro) * w;
+        }
         const int k = zc + Z, p = C.slot(X, Y, k);
         sm[C.v + p] = mu;
         sm[C.r + p] = rr;
@@ -360,7 +441,7 @@ __device__ __noinline__ void co_down(int li, int rank, int bc) {
         int X, Y, Z;
         co_decode<D>(c, C.nx, mx, C.ny, my, X, Y, Z);
         const int p = C.slot(X, Y, Z);
-        sm[C.r + p] = fma(ihc2, co_lap<D, T>(C, p), sm[C.r + p]);
+        sm[C.r + p] = fma(ihc2, co_lap<D, T, VAR>(S, C, li - 1, p), sm[C.r + p]);
     }
     co_sync(C.nr);  // the next half-sweep stores halo values that this pass reads
 }
@@ -408,17 +489,17 @@ __device__ __noinline__ void co_correct(int li, int rank, int bc) {
     co_sync(L.nr);
 }
 
-template <int D, typename T, bool BC, bool HB>
+template <int D, typename T, bool BC, bool HB, bool VAR>
 __device__ __noinline__ void co_vcycle(int lt, int rank, int bc) {
     const CoarseArgs &S = co_plan();
     for (int li = lt; li > 0; --li) {
-        co_smooth<D, T, BC, HB>(li, S.nd, rank, bc);
-        co_down<D, T, BC, HB>(li, rank, bc);
+        co_smooth<D, T, BC, HB, VAR>(li, S.nd, rank, bc);
+        co_down<D, T, BC, HB, VAR>(li, rank, bc);
     }
-    co_smooth<D, T, BC, HB>(0, S.nb, rank, bc);
+    co_smooth<D, T, BC, HB, VAR>(0, S.nb, rank, bc);
     for (int li = 1; li <= lt; ++li) {
         co_correct<D, T, BC, HB>(li, rank, bc);
-        co_smooth<D, T, BC, HB>(li, S.nu, rank, bc);
+        co_smooth<D, T, BC, HB, VAR>(li, S.nu, rank, bc);
     }
 }
 
@@ -520,7 +601,33 @@ __device__ __noinline__ void co_gather_faces(const BoxMeta &A, int rank, int bc,
     }
 }
 
-template <int D, typename T, bool BC, bool HB>
+// The coefficients of every level held here, packed in the layout of this
+// block's shared memory (mode 3, after eps changed).
+template <int D, typename T>
+__device__ __noinline__ void co_gather_coef(const BoxMeta &A, int rank, T *cpack) {
+    const CoarseArgs &S = co_plan();
+    T *out = cpack + (size_t)(blockIdx.x / S.R * S.R + rank) * S.ncoef;
+    const int tree = blockIdx.x / S.R;
+    for (int li = 0; li < S.nl; ++li) {
+        const CoLevel<D, T> L(li, rank);
+        int lg = 0;  // cells per box side
+        while ((2 << lg) <= S.N && lg <= li) ++lg;
+        const int mb = 1 << lg, nbx = L.nx >> lg, nby = (D == 3 ? L.ny : L.P * L.nr) >> lg;
+        const int nbz = D == 3 ? (L.P * L.nr) >> lg : 1, H = (D == 2 ? mb * mb : mb * mb * mb) / 2;
+        for (int c = threadIdx.x; c < L.nx * L.ny * L.P; c += blockDim.x) {
+            int i, j, k;
+            co_decode<D>(c, L.nx, S.mx[li], L.ny, S.my[li], i, j, k);
+            const int kz = L.z0 + k, jj = D == 3 ? j : kz, kk = D == 3 ? kz : 0, m1 = mb - 1;
+            const int b = S.dtab[li][((size_t)tree * nbz + (kk >> lg)) * nby * nbx + (jj >> lg) * nbx + (i >> lg)];
+            const long long q = A.coff[b] + ((i + j + kz + D) & 1) * H + ((kk & m1) * mb + (jj & m1)) * (mb / 2) + ((i & m1) >> 1);
+            for (int f = 0; f < 2 * D + 2; ++f)
+                out[S.oc[li] - S.ocoef + f * S.csz[li] + L.slot(i, j, k)] =
+                    reinterpret_cast<const T *>(S.coef)[f * S.coef_n + q];
+        }
+    }
+}
+
+template <int D, typename T, bool BC, bool HB, bool VAR>
 __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0, const unsigned char *refined, T *u,
                                        const T *rho, T *vold) {
     const CoarseArgs &S = co_plan();
@@ -540,6 +647,12 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
         at = ((kk & (mb - 1)) * mb + (jj & (mb - 1))) * (mb / 2) + (x & (mb / 2 - 1));
         r0 = (j + kz + D) & 1;  // red cell at 2x + r0
     };
+    if constexpr (VAR) {  // the packed coefficients, waited for before the first use
+        const char *src = reinterpret_cast<const char *>(S.cpack) + (size_t)(blockIdx.x / S.R * S.R + rank) * S.ncoef * sizeof(T);
+        char *dst = reinterpret_cast<char *>(sm + S.ocoef);
+        for (int x = tid; x < (int)(S.ncoef * sizeof(T) / 16); x += nt) cp_async<16>(dst + 16 * x, src + 16 * x);
+        cp_commit();
+    }
     constexpr int Q = 4;  // loads of a batch are in flight together
     for (int c0 = tid; c0 < n; c0 += Q * nt) {
         T ur[Q], ub[Q], rr[Q], rb[Q];
@@ -573,6 +686,7 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
             if (q >= 0) sm[q] = T(S.fval[at + x]);
         }
     }
+    if constexpr (VAR) cp_wait<0>();
     __syncthreads();
     for (int c = tid; c < n; c += nt) {  // ghosts and halos of level top's solution
         int x, j, k;
@@ -589,8 +703,8 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
             where(c, x, j, k, box, at, r0);
             const int p = L.slot(2 * x, j, k);
             if (refined[box]) {
-                sm[L.r + p] = fma(ih2, co_lap<D, T>(L, p), sm[L.r + p]);
-                sm[L.r + p + 1] = fma(ih2, co_lap<D, T>(L, p + 1), sm[L.r + p + 1]);
+                sm[L.r + p] = fma(ih2, co_lap<D, T, VAR>(S, L, lt, p), sm[L.r + p]);
+                sm[L.r + p + 1] = fma(ih2, co_lap<D, T, VAR>(S, L, lt, p + 1), sm[L.r + p + 1]);
             } else {
                 const long long g = cell0[box] + at;
                 vold[g] = sm[L.u + p + r0];
@@ -600,9 +714,9 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
         co_sync(L.nr);
     }
     if (S.mode == 0) {
-        co_vcycle<D, T, BC, HB>(lt, rank, bc);
+        co_vcycle<D, T, BC, HB, VAR>(lt, rank, bc);
     } else {
-        for (int li = lt; li > 0; --li) co_down<D, T, BC, HB>(li, rank, bc);
+        for (int li = lt; li > 0; --li) co_down<D, T, BC, HB, VAR>(li, rank, bc);
         for (int li = 0; li <= lt; ++li) {
             const CoLevel<D, T> B(li, rank);
             if (li < lt) {
@@ -620,7 +734,7 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
             }
             __syncthreads();
             if (li > 0) co_correct<D, T, BC, HB>(li, rank, bc);
-            co_vcycle<D, T, BC, HB>(li, rank, bc);
+            co_vcycle<D, T, BC, HB, VAR>(li, rank, bc);
         }
     }
     if (rank == 0 || L.nr > 1)
@@ -639,10 +753,11 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
 // coarse right-hand sides, then the FMG steps up to level top (v'_l <- v_l,
 // correction from l - 1, V-cycle from l), level top's v' going to global
 // memory; mode 2: the boundary data of the levels gathered into G.fval (after
-// it changed).  fas: level top's source holds the restricted residual; its coarse
+// it changed); mode 3 (VAR): the coefficients packed into G.cpack (after eps
+// changed).  fas: level top's source holds the restricted residual; its coarse
 // right-hand side rho + A u is completed here (refined boxes), and its leaf
 // boxes store v' = u.
-template <int D, typename T>
+template <int D, typename T, bool VAR>
 __global__ void __launch_bounds__(kCoarseThreads) k_coarse(BoxMeta A, const __grid_constant__ CoarseArgs G, T *u,
                                                            const T *rho, T *vold) {
     const int rank = G.R > 1 ? (int)(blockIdx.x % G.R) : 0, tree = blockIdx.x / G.R;
@@ -653,7 +768,8 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse(BoxMeta A, const __gr
     for (int x = tid; x < (int)(sizeof(CoarseArgs) / 4); x += nt)
         reinterpret_cast<int *>(co_smem)[x] = reinterpret_cast<const int *>(&G)[x];
     T *sm = co_mem<T>();
-    for (int x = tid; x < G.total; x += nt) sm[x] = T(0);
+    const int grids = VAR ? G.ocoef : G.total;
+    for (int x = tid; x < grids; x += nt) sm[x] = T(0);
     const int lt = G.nl - 1, z0 = G.nr[lt] > 1 ? rank * G.P[lt] : 0;
     const int layer = D == 3 ? G.nbx * G.nby : G.nbx;
     const int first = (z0 >> G.lgmb) * layer, nbox = (((z0 + G.P[lt] - 1) >> G.lgmb) + 1) * layer - first;
@@ -671,12 +787,13 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse(BoxMeta A, const __gr
     if (A.active && !A.active[tree]) return;  // R = 1 here: no barrier of a cluster is skipped
     if (G.R > 1) co_cluster_sync();           // every block has cleared its memory before another stores into it
     if (G.mode == 2) co_gather_faces<D, T>(A, rank, bc, G.fval);
+    else if (VAR && G.mode == 3) co_gather_coef<D, T>(A, rank, reinterpret_cast<T *>(G.cpack));
     else if (bc) {
-        if (G.hom) co_run<D, T, true, false>(rank, bc, cell0, refined, u, rho, vold);
-        else co_run<D, T, true, true>(rank, bc, cell0, refined, u, rho, vold);
+        if (G.hom) co_run<D, T, true, false, VAR>(rank, bc, cell0, refined, u, rho, vold);
+        else co_run<D, T, true, true, VAR>(rank, bc, cell0, refined, u, rho, vold);
     } else {
-        if (G.hom) co_run<D, T, false, false>(rank, bc, cell0, refined, u, rho, vold);
-        else co_run<D, T, false, true>(rank, bc, cell0, refined, u, rho, vold);
+        if (G.hom) co_run<D, T, false, false, VAR>(rank, bc, cell0, refined, u, rho, vold);
+        else co_run<D, T, false, true, VAR>(rank, bc, cell0, refined, u, rho, vold);
     }
     if (G.R > 1) co_cluster_sync();  // no block leaves while another may store into it
 }

@@ -24,6 +24,7 @@
 #pragma once
 #include "kernels_full.cuh"
 #include "kernels_var.cuh"
+#include "var_ops.cuh"
 
 namespace afg {
 
@@ -33,13 +34,6 @@ struct VarCoef {
     const T *c;
     long long n;
 };
-
-// n / s, with is = 1/s
-template <typename T>
-__device__ __forceinline__ T var_quot(T n, T s, T is) {
-    const T q = n * is;
-    return fma(fma(-q, s, n), is, q);
-}
 
 template <int D, int M, typename T>
 __global__ void __launch_bounds__(kThreads) k_var_coef(BoxMeta A, int b0, int n, const T *eps, T *out, long long nc,
@@ -77,15 +71,6 @@ __global__ void __launch_bounds__(kThreads) k_var_coef(BoxMeta A, int b0, int n,
             out[(2 * D + 1) * nc + I.coff + q] = T(1) / s;
         }
     }
-}
-
-// sum_s c_s u_s for the neighbours x[0..2D-1] of one cell, in side order
-template <int D, typename T>
-__device__ __forceinline__ T var_dot(const T (&c)[2 * D], const T (&x)[2 * D]) {
-    T a = T(0);
-#pragma unroll
-    for (int s = 0; s < 2 * D; ++s) a += c[s] * x[s];
-    return a;
 }
 
 // Half-sweep: per update 2D + 2 FMAs and a multiplication instead of 2D

@@ -282,10 +282,10 @@ void do_rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, co
     ++g_launches;
 }
 
-template <int D, typename T>
+template <int D, typename T, bool VAR>
 void do_coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
                const void *rho, void *vold) {
-    auto k = k_coarse<D, T>;
+    auto k = k_coarse<D, T, VAR>;
     occupancy(reinterpret_cast<const void *>(k), smem);  // sets the shared-memory limit
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ntrees * G.R);
@@ -366,7 +366,8 @@ void PrecOps<D, T>::rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *lis
 template <int D, typename T>
 void PrecOps<D, T>::coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
                            const void *rho, void *vold) {
-    do_coarse<D, T>(c, A, G, smem, ntrees, u, rho, vold);
+    if (G.op) do_coarse<D, T, true>(c, A, G, smem, ntrees, u, rho, vold);
+    else do_coarse<D, T, false>(c, A, G, smem, ntrees, u, rho, vold);
 }
 
 template <int D, typename T>

@@ -17,7 +17,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("D,N,uni,extra,op", [(2, 4, 1, 1, 2), (2, 8, 1, 0, 1), (2, 16, 2, 1, 2), (3, 4, 1, 1, 1),
-                                              (3, 8, 2, 0, 1), (3, 16, 1, 1, 1)])
+                                              (3, 8, 2, 0, 1), (3, 16, 1, 1, 1),
+                                              # levels in the coarse launch, up to grids spread over its blocks
+                                              (2, 8, 4, 1, 1), (2, 8, 5, 0, 2), (2, 16, 3, 0, 2), (2, 4, 4, 1, 1),
+                                              (3, 4, 3, 0, 1), (3, 8, 3, 0, 1), (2, 8, 1, 0, 2)])
 def test_cycles(D, N, uni, extra, op):
     a, b, rho, bv, _ = var_pair(D, N, uni, extra, 900 + N + D, op)
     load(a, b, rho, bv)
@@ -36,7 +39,8 @@ def test_new_coefficients_and_a_large_jump():
         cycles_parity(a, b, 1)
 
 
-@pytest.mark.parametrize("D,N,uni,extra,op", [(2, 4, 2, 1, 1), (3, 4, 2, 1, 1), (2, 16, 1, 1, 2), (3, 16, 1, 0, 1)])
+@pytest.mark.parametrize("D,N,uni,extra,op", [(2, 4, 2, 1, 1), (3, 4, 2, 1, 1), (2, 16, 1, 1, 2), (3, 16, 1, 0, 1),
+                                              (2, 8, 5, 0, 2), (3, 8, 2, 1, 1)])
 def test_mixed(D, N, uni, extra, op):
     a, b, rho, bv, _ = var_pair(D, N, uni, extra, 940 + N + D, op, cells=2, lo=0.5, hi=4.0)
     load(a, b, rho, 1e-3 * bv)
