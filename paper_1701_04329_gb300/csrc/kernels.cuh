@@ -37,11 +37,25 @@ namespace afg {
 
 constexpr int kThreads = 256;
 
-// Programmatic dependent launch: every kernel lets the next launch start
-// early (pdl_trigger) and waits for its predecessors to finish and their
-// memory to be visible (pdl_wait) before reading anything a kernel wrote.
-// Box metadata is written only by host uploads, so prologues may read it.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Programmatic dependent launch: a kernel of few blocks lets the next launch
+// start at once (pdl_trigger), and every kernel waits for its predecessors to
+// finish and their memory to be visible (pdl_wait) before reading anything a
+// kernel wrote.  Box metadata is written only by host uploads, so prologues
+// may read it.
+//
+// Only up to kPdlEarlyGrid blocks (about three per SM): the next kernel's
+// prologue then overlaps a kernel that leaves room (2D, 31 k unknowns: 2.22
+// against 2.43 ms without).  Behind a grid that fills the chip the next
+// kernel's blocks take slots one by one as they come free, so their number
+// per SM, and with it each SM's share of the work, comes out uneven: a larger
+// grid's dependents start when its blocks exit.  Measured with the trigger in
+// every kernel / up to 800, 500, 304 blocks / none: uniform 512^3, mixed, 63.9 /
+// 52.6, 53.0, 53.0 / 53.6 ms; 18.8 M unknowns, mixed, 12.55 / 11.52, 11.59, 11.69 /
+// 11.86 ms; the same, FP64, 29.6 / 29.6, 29.0, 29.1 / 29.7 ms.
+constexpr int kPdlEarlyGrid = 500;
+__device__ __forceinline__ void pdl_trigger() {
+    if (gridDim.x <= kPdlEarlyGrid) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 constexpr unsigned char BF_REFINED = 1, BF_SPECIAL = 2;
 constexpr int BF_NSHIFT = 2;  // flag bits 2..7: Neumann domain sides (bit 2 + s)
