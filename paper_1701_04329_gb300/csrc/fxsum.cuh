@@ -119,6 +119,67 @@ struct FxAcc {
     }
 };
 
+// x aligned to the exponent E of the largest of a set of values, in the fixed
+// point of FxAcc<W>: x = result * 2^(E - 1075 - G) but for the truncated bits.
+// x's own exponent must not exceed E.
+template <int W>
+AFG_HD int64_t fx_align(double x, int E) {
+    const uint64_t b = fx_bits(x);
+    const uint64_t m = ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << FxAcc<W>::G;
+    const int s = E - ((int)(b >> 52) & 0x7FF);
+    const int64_t a = (int64_t)(m >> (s < 63 ? s : 63));  // m < 2^(53 + G) < 2^63
+    const int64_t neg = (int64_t)b >> 63;
+    return (a ^ neg) - neg;
+}
+
+// S * 2^(E - 1075 - G), as FxAcc<W>::round: where |S| has at most 53 bits (sums
+// that nearly cancel) its bits are moved and nothing is rounded
+template <int W>
+#ifdef __CUDACC__
+__host__ __device__ __noinline__
+#endif
+    static double
+    fx_round_any(int64_t S, int E) {
+    FxAcc<W> acc(E);
+    acc.S = S;
+    return acc.round();
+}
+
+template <int W>
+AFG_HD double fx_round(int64_t S, int E) {
+    const uint64_t A = S < 0 ? (uint64_t)(-S) : (uint64_t)S;
+    if ((A >> 53) != 0 || A == 0) return fx_round_any<W>(S, E);
+    const int z = fx_clz(A);  // leading bit 63 - z <= 52
+    return fx_double(((uint64_t)(63 - z + E - 53 - FxAcc<W>::G) << 52) + (A << (z - 11)) |
+                     ((uint64_t)S & 0x8000000000000000ull));
+}
+
+// a call: inlined, the compiler would run the conversion (64 cycles of the
+// FP64 unit) for every value and select
+#ifdef __CUDACC__
+__host__ __device__ __noinline__
+#endif
+    static float
+    fx_cast(double x) {
+    return (float)x;
+}
+
+// (float)x, nearest even, without the FP64 unit while the result is a normal number
+AFG_HD float fx_to_float(double x) {
+    const uint64_t b = fx_bits(x);
+    const int e = (int)(b >> 52) & 0x7FF;
+    if (e < 897 || e > 1150) return fx_cast(x);
+    const uint64_t u = (b & 0x7FFFFFFFFFFFFFFFull) - (896ull << 52);
+    const uint32_t f = (uint32_t)((u + 0xFFFFFFFull + ((u >> 29) & 1)) >> 29) | ((uint32_t)(b >> 32) & 0x80000000u);
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(f);
+#else
+    float r;
+    std::memcpy(&r, &f, 4);
+    return r;
+#endif
+}
+
 // out = sum_k x[k] - C * c over x[0..K-1].  Returns false (out untouched)
 // when the largest exponent is outside the handled range.
 template <int K, int C = 0>

@@ -922,9 +922,13 @@ __global__ void __launch_bounds__(kThreads) k_restrict_u(BoxMeta A, int b0, int 
     }
 }
 
-// |x| as an ordered unsigned bit pattern (sign bit cleared; integer ops only)
+// |x| as an ordered unsigned bit pattern (sign bit cleared; integer ops only:
+// the mask is written in PTX, the compiler makes an FP64 instruction of the C
+// expression, which it recognises as fabs)
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
-    return static_cast<unsigned long long>(__double_as_longlong(x)) & 0x7fffffffffffffffull;
+    unsigned hi;
+    asm("and.b32 %0, %1, 0x7fffffff;" : "=r"(hi) : "r"(__double2hiint(x)));
+    return ((unsigned long long)hi << 32) | (unsigned)__double2loint(x);
 }
 __device__ __forceinline__ unsigned long long abs_bits(float x) { return abs_bits(double(x)); }
 

@@ -354,6 +354,127 @@ __device__ __forceinline__ void fp_lap_vec(const T *st, int col, int j, int k, i
     }
 }
 
+// barrier of one box's thread group (g: its number in the block)
+template <int G>
+__device__ __forceinline__ void group_sync(int g) {
+    if constexpr (G <= 32) __syncwarp(G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1) << ((threadIdx.x & 31) / G * G));
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(G) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// FP64 images in fixed point.  GB300 issues one FP64 instruction per 64 cycles
+// and warp, and aligning every term of every sum to its cell's largest
+// exponent (fx_sum) takes some 25 integer instructions a term.  A staged
+// image is read seven times over, so it is aligned once instead: every value
+// to the largest exponent E of the box and its ghosts, in place, as a 64-bit
+// integer with G guard bits below the last bit of a value of that exponent.
+// Sums of neighbours are then integer additions, exact, rounded once.
+//
+// The truncated bits are at most one unit of 2^-6 ulp (of the box's largest
+// value) per term; FP64 additions round to half an ulp of every partial sum.
+// A box whose values span more than 2^kFxSpan keeps the alignment per cell
+// (its small values would lose bits), and so does one whose largest exponent
+// is out of fx_sum's range (all zero, infinite, NaN).
+// ---------------------------------------------------------------------------
+constexpr int kFxSpan = 8;
+// FP64 leaf residuals that align their images: in 3D, and in 2D where the
+// residual goes to FP32 (R); the norms of 2D FP64 cycles keep their rounding,
+// near which hundreds of small trees decide on one more cycle.
+template <int D, typename T, typename R>
+constexpr bool fx_leaf() { return sizeof(T) == 8 && (D == 3 || sizeof(R) == 4); }
+template <int D>
+constexpr int fx_lap_weight() { return 4 * D; }  // sum_nb u - 2D u
+
+// Aligns the image st[0..n) of a box to its largest exponent (every slot that
+// no staging writes holds zero) and returns that exponent, or -1: unchanged.
+// red: 2 ints per warp of the block.
+template <int W, int GT>
+__device__ __forceinline__ int fx_image(double *st, int n, int lt, int g, int *red) {
+    static_assert(GT >= 32, "whole warps per box");
+    unsigned mx = 0, mn = 0x7fffffffu;
+    for (int v = lt; v < n / 2; v += GT) {
+        const int4 q = reinterpret_cast<const int4 *>(st)[v];
+        const unsigned a = (unsigned)q.y & 0x7fffffffu, b = (unsigned)q.w & 0x7fffffffu, m = a > b ? a : b;
+        mx = m > mx ? m : mx;
+        if (m) mn = m < mn ? m : mn;
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    if constexpr (GT > 32) {
+        const int w = threadIdx.x >> 5, w0 = g * (GT / 32);
+        if ((threadIdx.x & 31) == 0) {
+            red[2 * w] = (int)mx;
+            red[2 * w + 1] = (int)mn;
+        }
+        group_sync<GT>(g);
+#pragma unroll
+        for (int x = 0; x < GT / 32; ++x) {
+            mx = max(mx, (unsigned)red[2 * (w0 + x)]);
+            mn = min(mn, (unsigned)red[2 * (w0 + x) + 1]);
+        }
+    }
+    const int E = (int)(mx >> 20);
+    const bool ok = E >= kFxEmin && E <= kFxEmax && E - (int)(mn >> 20) <= kFxSpan;
+    if (ok)
+        for (int v = lt; v < n / 2; v += GT) {
+            const double2 q = reinterpret_cast<const double2 *>(st)[v];
+            longlong2 o;
+            o.x = fx_align<W>(q.x, E);
+            o.y = fx_align<W>(q.y, E);
+            reinterpret_cast<longlong2 *>(st)[v] = o;
+        }
+    group_sync<GT>(g);
+    return ok ? E : -1;
+}
+
+// Where a thread's vectors of an FP64 image and their neighbours lie, the same
+// for every box: the vector, the other colour's half-row beside it, the x
+// neighbour past it, and whether that one lies towards +x.
+template <int D, int M, int GT>
+struct FxPlan {
+    using F = FpCfg<D, M, double, GT>;
+    static constexpr int NIV = (F::NV + F::G - 1) / F::G;
+    int self[NIV], po[NIV], extra[NIV];  // extra: | r << 16
+    __device__ __forceinline__ void init(int lt) {
+        constexpr int MH = F::MH, NVH = F::H / F::VEC;
+#pragma unroll
+        for (int it = 0; it < NIV; ++it) {
+            const int v = lt + it * F::G;
+            const int col = v / NVH, w = v % NVH;
+            const int row = w / F::NVR, h0 = (w % F::NVR) * F::VEC;
+            const int j = row % M, k = D == 2 ? 0 : row / M, rowi = sp_row<D, M>(j, k);
+            const int r = (col + j + k + D) & 1;
+            self[it] = col * F::PT + rowi * MH + h0;
+            po[it] = (1 - col) * F::PT + rowi * MH + h0;
+            int e;
+            if (r) e = h0 + 2 < MH ? po[it] + 2 : 2 * F::PT + F::ROWS + rowi;
+            else e = h0 > 0 ? po[it] - 1 : 2 * F::PT + rowi;
+            extra[it] = e | (r << 16);
+        }
+    }
+};
+
+// h^2 times the operator on vector `it` of the thread, on an aligned image
+template <int D, int M, int GT>
+__device__ __forceinline__ void fp_lap_vec_fx(const double *st, int E, const FxPlan<D, M, GT> &pl, int it,
+                                              double *lap) {
+    constexpr int MH = M / 2;
+    const long long *im = reinterpret_cast<const long long *>(st), *po = im + pl.po[it];
+    const bool r = pl.extra[it] >> 16;
+    auto at = [](const long long *p) { return *reinterpret_cast<const longlong2 *>(p); };
+    const longlong2 self = at(im + pl.self[it]), xv = at(po), ym = at(po - MH), yp = at(po + MH);
+    const long long extra = im[pl.extra[it] & 0xffff];
+    long long s0 = xv.x + (r ? xv.y : extra) + ym.x + yp.x - 2 * D * self.x;
+    long long s1 = xv.y + (r ? extra : xv.x) + ym.y + yp.y - 2 * D * self.y;
+    if (D == 3) {
+        const longlong2 zm = at(po - (M + 2) * MH), zp = at(po + (M + 2) * MH);
+        s0 += zm.x + zp.x;
+        s1 += zm.y + zp.y;
+    }
+    lap[0] = fx_round<fx_lap_weight<D>()>(s0, E);
+    lap[1] = fx_round<fx_lap_weight<D>()>(s1, E);
+}
+
 // Prologue and ring walk shared by the kernels below.  body(I, st, lt) is
 // called once per staged box after its ghosts are complete; want(I) says
 // whether a box needs the u image, flat(I) which array goes to the flat area
@@ -365,8 +486,10 @@ __device__ __forceinline__ void fp_lap_vec(const T *st, int col, int j, int k, i
 // barrier; otherwise every box with a non-copy side takes it (fewer registers).
 // PLAN: copies and domain-side fixes through a per-thread plan (FpPlan), no
 // per-box decoding of the items (more registers).
-template <int D, int M, typename T, int GT, bool OWN = true, bool PLAN = false, typename Want, typename Flat,
-          typename Body, typename Pre, typename Post>
+// FX: the weight of the sums formed on the image; it is aligned (fx_image) before
+// body(I, st, lt, E), E its exponent or -1 (0: no alignment, E = -1).
+template <int D, int M, typename T, int GT, bool OWN = true, bool PLAN = false, int FX = 0, typename Want,
+          typename Flat, typename Body, typename Pre, typename Post>
 __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const int *list, const T *u, int hom,
                                         Want want, Flat flat, Body body, Pre pre, Post post) {
     using F = FpCfg<D, M, T, GT>;
@@ -377,6 +500,10 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
     BoxInfo *info = reinterpret_cast<BoxInfo *>(smem_raw + sizeof(T) * F::BOX * F::BPC * NST);
     const int stride = gridDim.x * F::BPC;
     const int first = blockIdx.x * F::BPC;
+    __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
+    if constexpr (FX > 0) {  // the slots that no staging writes hold zero
+        for (int x = threadIdx.x; x < F::BOX * F::BPC * NST; x += kThreads) stages[x] = T(0);
+    }
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
         info_load<D>(A, first + q * stride + g, n, b0, list, info[q * F::BPC + g], lt, F::G, false);
     pdl_wait();
@@ -413,7 +540,13 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
             if (cf) fp_fix<D, M, T, GT>(I, A, u, st, lt, hom, OWN);
             __syncthreads();
         }
-        if (I.b >= 0) body(I, st, lt);
+        if (I.b >= 0) {
+            int E = -1;
+            if constexpr (FX > 0) {
+                if (want(I)) E = fx_image<FX, GT>(st, F::UB, lt, g, fxr);
+            }
+            body(I, st, lt, E);
+        }
         post(&info[(it % NI) * F::BPC]);
     }
     cp_wait<0>();
@@ -435,14 +568,23 @@ constexpr int fas_threads() {
 }
 
 // threads per box of the leaf residual: as the FAS kernel, but FP64 boxes take
-// at most 64 threads where the several boxes per block that this gives fit in
-// 100 KB of shared memory, two blocks per SM (measured 0.288 instead of
-// 0.297 ms on a 256^3 level of 8^3 boxes)
-template <int D, int M, typename T>
+// fewer where the several boxes per block that this gives leave several blocks
+// an SM: 128 in 3D (aligned images; four blocks of 64 registers), 64 in 2D (two
+// blocks).  256^3 of 8^3 boxes: 0.165 ms with 128 threads and four blocks, 0.174
+// with three, 0.182 with 64 threads and two, 0.231 with 256 and three (per-cell
+// alignment, 64 threads and two: 0.280).  2D, 4.2 M cells, 8^2 / 16^2 boxes: four
+// blocks 56 / 39 us, three 71 / 41, no bound 97 / 54 (before 82 / 57).
+template <int D, int M, typename T, typename R>
 constexpr int leaf_threads() {
+    if (fx_leaf<D, T, R>() && D == 3)
+        return fas_threads<D, M, T>() > 128 && FpCfg<D, M, T, 128>::smem() <= 56 * 1024 ? 128 : fas_threads<D, M, T>();
     return (sizeof(T) == 8 && fas_threads<D, M, T>() > 64 && FpCfg<D, M, T, 64>::smem() <= 100 * 1024)
                ? 64
                : fas_threads<D, M, T>();
+}
+template <int D, int M, typename T, typename R>
+constexpr int leaf_blocks() {
+    return sizeof(T) == 8 && (D == 2 || leaf_threads<D, M, T, R>() == 128) ? 4 : 1;
 }
 
 // Fused residual + restriction, staged version of k_resid_restrict (same
@@ -457,7 +599,7 @@ __global__ void __launch_bounds__(kThreads) k_resid_restrict_p(BoxMeta A, int b0
     pdl_trigger();
     auto want = [](const BoxInfo &) { return true; };
     auto flat = [&](const BoxInfo &) -> const T * { return rho; };
-    auto body = [&](const BoxInfo &I, const T *st, int lt) {
+    auto body = [&](const BoxInfo &I, const T *st, int lt, int) {
         const T *X = st + 2 * F::PT, *R = st + F::UB;
         const long long cp = A.coff[I.parent];
         for (int c = lt; c < NCO; c += F::G) {
@@ -508,7 +650,7 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
     pdl_trigger();
     auto want = [](const BoxInfo &I) { return (I.flag & BF_REFINED) != 0; };
     auto flat = [&](const BoxInfo &I) -> const T * { return (I.flag & BF_REFINED) ? rho : u; };
-    auto body = [&](const BoxInfo &I, const T *st, int lt) {
+    auto body = [&](const BoxInfo &I, const T *st, int lt, int) {
         const T *FL = st + F::UB;
         if (!(I.flag & BF_REFINED)) {
             for (int v = lt; v < F::NV; v += F::G) {
@@ -544,8 +686,9 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
 // maxima of |r| and |rho| over the leaf cells (as bit patterns, reduced per
 // block and committed with one atomic per block when the block moves to
 // another tree, and at the end), and optionally r cast to R in rout.
-// lap(I, st, v, col, j, k, h0, out): h^2 times the operator on vector v of the box.
-template <int D, int M, typename T, typename R, int GT, typename Lap>
+// lap_vec(I, st, v, col, j, k, h0, out): h^2 times the operator on vector v of a box
+// whose image is not aligned; FX: weight of the aligned images' sums (0: none are).
+template <int D, int M, typename T, typename R, int GT, int FX, typename Lap>
 __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *list, int n, const T *u,
                                                    const T *__restrict__ rho, int hom, unsigned long long *rmax,
                                                    unsigned long long *pmax, R *rout, Lap lap_vec) {
@@ -553,6 +696,8 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
     constexpr int VEC = F::VEC, NVH = F::H / VEC;
     __shared__ unsigned long long red[64];
     const int g = threadIdx.x / F::G;
+    FxPlan<D, M, GT> fxp;
+    if constexpr (FX > 0) fxp.init(threadIdx.x % F::G);
     unsigned long long rm = 0, pm = 0;
     int cur = -1, tr = -1;  // tree of the running maxima, tree of this step's boxes (uniform in the block)
     bool mixed = false;
@@ -573,29 +718,47 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
             cur = -1;
         }
     };
-    auto body = [&](const BoxInfo &I, const T *st, int lt) {
+    auto body = [&](const BoxInfo &I, const T *st, int lt, int E) {
         const T ih2 = T(A.ih2[I.b]);
         const T *FL = st + F::UB;
-        for (int v = lt; v < F::NV; v += F::G) {
-            const int col = v / NVH, w = v % NVH;
-            const int row = w / F::NVR, h0 = (w % F::NVR) * VEC;
-            const int j = row % M, k = D == 2 ? 0 : row / M;
-            T lap[VEC], rv[VEC];
-            lap_vec(I, st, v, col, j, k, h0, lap);
+        auto finish = [&](int v, const T *lap) {
+            T rv[VEC];
             ldv<T, VEC>(FL + v * VEC, rv);
             R out[VEC];
 #pragma unroll
             for (int x = 0; x < VEC; ++x) {
                 // r = rho - (sum - 2D u) / h^2; |.| on the bit patterns
                 const T rr = fma(-ih2, lap[x], rv[x]);
-                out[x] = R(rr);
+                if constexpr (sizeof(T) == 8 && sizeof(R) == 4) out[x] = fx_to_float(rr);
+                else out[x] = R(rr);
                 rm = max(rm, abs_bits(rr));
                 pm = max(pm, abs_bits(rv[x]));
             }
-            if (rout) {
-#pragma unroll
+            if (!rout) return;
+            if constexpr (sizeof(R) <= sizeof(T)) stv<R, VEC>(rout + I.coff + (long long)v * VEC, out);
+            else
                 for (int x = 0; x < VEC; ++x) rout[I.coff + (long long)v * VEC + x] = out[x];
+        };
+        // two loops: in one, the compiler runs the FP64 additions of the other case too and selects
+        if constexpr (FX > 0) {
+            if (E >= 0) {
+#pragma unroll
+                for (int it = 0; it < FxPlan<D, M, GT>::NIV; ++it) {
+                    if (lt + it * F::G >= F::NV) continue;
+                    T lap[VEC];
+                    fp_lap_vec_fx<D, M, GT>(st, E, fxp, it, lap);
+                    finish(lt + it * F::G, lap);
+                }
+                return;
             }
+        }
+        for (int v = lt; v < F::NV; v += F::G) {
+            const int col = v / NVH, w = v % NVH;
+            const int row = w / F::NVR, h0 = (w % F::NVR) * VEC;
+            const int j = row % M, k = D == 2 ? 0 : row / M;
+            T lap[VEC];
+            lap_vec(I, st, v, col, j, k, h0, lap);
+            finish(v, lap);
         }
     };
     auto post = [&](const BoxInfo *slot) {
@@ -609,20 +772,21 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
             cur = tr;
         }
     };
-    fp_walk<D, M, T, GT, false>(A, 0, n, list, u, hom, want, flat, body, pre, post);  // register-bound: no own-thread fix
+    fp_walk<D, M, T, GT, (FX > 0), (FX > 0), FX>(A, 0, n, list, u, hom, want, flat, body, pre, post);
     flush_max(rm, pm, cur, cur >= 0, rmax, pmax, red);
 }
 
 template <int D, int M, typename T, typename R>
-__global__ void __launch_bounds__(kThreads) k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
+__global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>()) k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
                                                               const T *__restrict__ rho, int hom,
                                                               unsigned long long *rmax, unsigned long long *pmax,
                                                               R *rout) {
+    constexpr int GT = leaf_threads<D, M, T, R>(), FX = fx_leaf<D, T, R>() ? fx_lap_weight<D>() : 0;
     pdl_trigger();
     auto lap = [](const BoxInfo &, const T *st, int, int col, int j, int k, int h0, T *out) {
         fp_lap_vec<D, M, T>(st, col, j, k, h0, out);
     };
-    leaf_residual_walk<D, M, T, R, leaf_threads<D, M, T>()>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
+    leaf_residual_walk<D, M, T, R, GT, FX>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
 }
 
 // ---------------------------------------------------------------------------

@@ -140,13 +140,6 @@ __device__ __forceinline__ void fp_var_lap_vec(const T *st, const T *cp, long lo
     }
 }
 
-// barrier of one box's thread group
-template <int G>
-__device__ __forceinline__ void group_sync(int g) {
-    if constexpr (G <= 32) __syncwarp(G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1) << ((threadIdx.x & 31) / G * G));
-    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(G) : "memory");
-}
-
 // Residual and restriction: the residual of every cell replaces its source in
 // the stage, then the mean of the 2^D children (weighted by r in (r,z)) goes
 // to the parent.
@@ -160,7 +153,7 @@ __global__ void __launch_bounds__(kThreads) k_var_resid_restrict_p(BoxMeta A, in
     pdl_trigger();
     auto want = [](const BoxInfo &) { return true; };
     auto flat = [&](const BoxInfo &) -> const T * { return rho; };
-    auto body = [&](const BoxInfo &I, T *st, int lt) {
+    auto body = [&](const BoxInfo &I, T *st, int lt, int) {
         T *R = st + F::UB;
         for (int v = lt; v < F::NV; v += F::G) {
             const int col = v / NVH, w = v % NVH;
@@ -221,7 +214,7 @@ __global__ void __launch_bounds__(kThreads) k_var_fas_p(BoxMeta A, int b0, int n
     pdl_trigger();
     auto want = [](const BoxInfo &I) { return (I.flag & BF_REFINED) != 0; };
     auto flat = [&](const BoxInfo &I) -> const T * { return (I.flag & BF_REFINED) ? rho : u; };
-    auto body = [&](const BoxInfo &I, const T *st, int lt) {
+    auto body = [&](const BoxInfo &I, const T *st, int lt, int) {
         const T *FL = st + F::UB;
         for (int v = lt; v < F::NV; v += F::G) {
             T rv[VEC];
@@ -250,16 +243,14 @@ __global__ void __launch_bounds__(kThreads) k_var_leaf_residual_p(BoxMeta A, con
                                                                   const T *__restrict__ rho, VarCoef<T> V, int hom,
                                                                   unsigned long long *rmax, unsigned long long *pmax,
                                                                   R *rout) {
-    constexpr int GT = leaf_threads<D, M, T>();
-    using F = FpCfg<D, M, T, GT>;
-    constexpr int VEC = F::VEC, NVH = F::H / VEC;
+    constexpr int GT = leaf_threads<D, M, T, R>();
+    constexpr int VEC = FpCfg<D, M, T, GT>::VEC;
     pdl_trigger();
     auto lap = [&](const BoxInfo &I, const T *st, int v, int col, int j, int k, int h0, T *out) {
         T self[VEC];
         fp_var_lap_vec<D, M, T>(st, V.c + I.coff + v * VEC, V.n, col, j, k, h0, out, self);
     };
-    leaf_residual_walk<D, M, T, R, GT>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
-    (void)NVH;
+    leaf_residual_walk<D, M, T, R, GT, 0>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
 }
 
 }  // namespace afg

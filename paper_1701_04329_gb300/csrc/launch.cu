@@ -51,7 +51,7 @@ int occupancy(const void *kernel, size_t smem) {
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     size_t &lim = limit[std::make_pair(dev, kernel)];
-    if (smem > 48 * 1024 && smem > lim) {
+    if (smem > 40 * 1024 && smem > lim) {  // with a kernel's own static arrays, past the default 48 KB
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         lim = smem;
     }

@@ -95,7 +95,7 @@ void do_var_leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list,
                           unsigned long long *pmax, void *rout) {
     if (n <= 0) return;
     static_assert(FpCfg<D, M, T>::ok, "leaf boxes have 4 cells per side or more, in FP64");
-    using F = FpCfg<D, M, T, leaf_threads<D, M, T>()>;
+    using F = FpCfg<D, M, T, leaf_threads<D, M, T, Ro>()>;
     auto k = k_var_leaf_residual_p<D, M, T, Ro>;
     const VarCoef<T> V{(const T *)W.coef, W.n};
     launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, (const T *)u,
