@@ -132,26 +132,17 @@ AFG_HD int64_t fx_align(double x, int E) {
     return (a ^ neg) - neg;
 }
 
-// S * 2^(E - 1075 - G), as FxAcc<W>::round: where |S| has at most 53 bits (sums
-// that nearly cancel) its bits are moved and nothing is rounded
-template <int W>
-#ifdef __CUDACC__
-__host__ __device__ __noinline__
-#endif
-    static double
-    fx_round_any(int64_t S, int E) {
-    FxAcc<W> acc(E);
-    acc.S = S;
-    return acc.round();
-}
-
+// S * 2^(E - 1075 - G), nearest even: FxAcc<W>::round with the leading bit moved
+// to the top first, so that one path serves every size of S
 template <int W>
 AFG_HD double fx_round(int64_t S, int E) {
     const uint64_t A = S < 0 ? (uint64_t)(-S) : (uint64_t)S;
-    if ((A >> 53) != 0 || A == 0) return fx_round_any<W>(S, E);
-    const int z = fx_clz(A);  // leading bit 63 - z <= 52
-    return fx_double(((uint64_t)(63 - z + E - 53 - FxAcc<W>::G) << 52) + (A << (z - 11)) |
-                     ((uint64_t)S & 0x8000000000000000ull));
+    if (A == 0) return 0.0;
+    const int z = fx_clz(A);
+    const uint64_t N = A << z, M = N >> 11;
+    const uint32_t rem = (uint32_t)N & 0x7FF;
+    const uint64_t up = rem + ((uint32_t)M & 1) > 0x400;
+    return fx_double((((uint64_t)(10 - z + E - FxAcc<W>::G) << 52) + M + up) | ((uint64_t)S & 0x8000000000000000ull));
 }
 
 // a call: inlined, the compiler would run the conversion (64 cycles of the

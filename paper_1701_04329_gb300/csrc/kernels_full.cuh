@@ -354,79 +354,6 @@ __device__ __forceinline__ void fp_lap_vec(const T *st, int col, int j, int k, i
     }
 }
 
-// barrier of one box's thread group (g: its number in the block)
-template <int G>
-__device__ __forceinline__ void group_sync(int g) {
-    if constexpr (G <= 32) __syncwarp(G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1) << ((threadIdx.x & 31) / G * G));
-    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(G) : "memory");
-}
-
-// ---------------------------------------------------------------------------
-// FP64 images in fixed point.  GB300 issues one FP64 instruction per 64 cycles
-// and warp, and aligning every term of every sum to its cell's largest
-// exponent (fx_sum) takes some 25 integer instructions a term.  A staged
-// image is read seven times over, so it is aligned once instead: every value
-// to the largest exponent E of the box and its ghosts, in place, as a 64-bit
-// integer with G guard bits below the last bit of a value of that exponent.
-// Sums of neighbours are then integer additions, exact, rounded once.
-//
-// The truncated bits are at most one unit of 2^-6 ulp (of the box's largest
-// value) per term; FP64 additions round to half an ulp of every partial sum.
-// A box whose values span more than 2^kFxSpan keeps the alignment per cell
-// (its small values would lose bits), and so does one whose largest exponent
-// is out of fx_sum's range (all zero, infinite, NaN).
-// ---------------------------------------------------------------------------
-constexpr int kFxSpan = 8;
-// FP64 leaf residuals that align their images: in 3D, and in 2D where the
-// residual goes to FP32 (R); the norms of 2D FP64 cycles keep their rounding,
-// near which hundreds of small trees decide on one more cycle.
-template <int D, typename T, typename R>
-constexpr bool fx_leaf() { return sizeof(T) == 8 && (D == 3 || sizeof(R) == 4); }
-template <int D>
-constexpr int fx_lap_weight() { return 4 * D; }  // sum_nb u - 2D u
-
-// Aligns the image st[0..n) of a box to its largest exponent (every slot that
-// no staging writes holds zero) and returns that exponent, or -1: unchanged.
-// red: 2 ints per warp of the block.
-template <int W, int GT>
-__device__ __forceinline__ int fx_image(double *st, int n, int lt, int g, int *red) {
-    static_assert(GT >= 32, "whole warps per box");
-    unsigned mx = 0, mn = 0x7fffffffu;
-    for (int v = lt; v < n / 2; v += GT) {
-        const int4 q = reinterpret_cast<const int4 *>(st)[v];
-        const unsigned a = (unsigned)q.y & 0x7fffffffu, b = (unsigned)q.w & 0x7fffffffu, m = a > b ? a : b;
-        mx = m > mx ? m : mx;
-        if (m) mn = m < mn ? m : mn;
-    }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    mn = __reduce_min_sync(0xffffffffu, mn);
-    if constexpr (GT > 32) {
-        const int w = threadIdx.x >> 5, w0 = g * (GT / 32);
-        if ((threadIdx.x & 31) == 0) {
-            red[2 * w] = (int)mx;
-            red[2 * w + 1] = (int)mn;
-        }
-        group_sync<GT>(g);
-#pragma unroll
-        for (int x = 0; x < GT / 32; ++x) {
-            mx = max(mx, (unsigned)red[2 * (w0 + x)]);
-            mn = min(mn, (unsigned)red[2 * (w0 + x) + 1]);
-        }
-    }
-    const int E = (int)(mx >> 20);
-    const bool ok = E >= kFxEmin && E <= kFxEmax && E - (int)(mn >> 20) <= kFxSpan;
-    if (ok)
-        for (int v = lt; v < n / 2; v += GT) {
-            const double2 q = reinterpret_cast<const double2 *>(st)[v];
-            longlong2 o;
-            o.x = fx_align<W>(q.x, E);
-            o.y = fx_align<W>(q.y, E);
-            reinterpret_cast<longlong2 *>(st)[v] = o;
-        }
-    group_sync<GT>(g);
-    return ok ? E : -1;
-}
-
 // Where a thread's vectors of an FP64 image and their neighbours lie, the same
 // for every box: the vector, the other colour's half-row beside it, the x
 // neighbour past it, and whether that one lies towards +x.
@@ -486,10 +413,11 @@ __device__ __forceinline__ void fp_lap_vec_fx(const double *st, int E, const FxP
 // barrier; otherwise every box with a non-copy side takes it (fewer registers).
 // PLAN: copies and domain-side fixes through a per-thread plan (FpPlan), no
 // per-box decoding of the items (more registers).
-// FX: the weight of the sums formed on the image; it is aligned (fx_image) before
-// body(I, st, lt, E), E its exponent or -1 (0: no alignment, E = -1).
-template <int D, int M, typename T, int GT, bool OWN = true, bool PLAN = false, int FX = 0, typename Want,
-          typename Flat, typename Body, typename Pre, typename Post>
+// FX: the weight of the sums formed on the image, which is aligned before
+// body(I, st, lt, E), E its exponent or -1 (0: no alignment, E = -1; needs PLAN).
+// BLOCK: pre and post meet the whole block, so every step does.
+template <int D, int M, typename T, int GT, bool OWN = true, bool PLAN = false, int FX = 0, bool BLOCK = false,
+          typename Want, typename Flat, typename Body, typename Pre, typename Post>
 __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const int *list, const T *u, int hom,
                                         Want want, Flat flat, Body body, Pre pre, Post post) {
     using F = FpCfg<D, M, T, GT>;
@@ -501,9 +429,6 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
     const int stride = gridDim.x * F::BPC;
     const int first = blockIdx.x * F::BPC;
     __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
-    if constexpr (FX > 0) {  // the slots that no staging writes hold zero
-        for (int x = threadIdx.x; x < F::BOX * F::BPC * NST; x += kThreads) stages[x] = T(0);
-    }
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
         info_load<D>(A, first + q * stride + g, n, b0, list, info[q * F::BPC + g], lt, F::G, false);
     pdl_wait();
@@ -532,18 +457,29 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
             if constexpr (PLAN) fp_fix_own_plan<D, M, T, GT>(pl, I, A, st, hom);
             else fp_fix_own<D, M, T, GT>(I, A, st, lt, hom);
         }
-        const int any_cf = __syncthreads_or(cf);  // previous stage and metadata slot are free now
+        if constexpr (FX > 0) {
+            static_assert(OWN && PLAN, "aligned images need the plan");
+            if (I.b >= 0 && want(I)) fx_fold_own(pl, st, fxr);
+        }
+        const int any_cf = box_sync<BLOCK ? 1 : GT>(g, cf);  // previous stage and metadata slot are free now
         issue(it + NST - 1);
         info_load<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * F::BPC + g], lt, F::G);
         pre(&info[(it % NI) * F::BPC]);
         if (any_cf) {  // refinement-boundary ghosts read cells other threads staged
-            if (cf) fp_fix<D, M, T, GT>(I, A, u, st, lt, hom, OWN);
-            __syncthreads();
+            if (cf) {
+                fp_fix<D, M, T, GT>(I, A, u, st, lt, hom, OWN);
+                if constexpr (FX > 0) fx_fold_own(pl, st, fxr);  // the thread's own items again
+            }
+            box_sync<BLOCK ? 1 : GT>(g, false);
         }
         if (I.b >= 0) {
             int E = -1;
             if constexpr (FX > 0) {
-                if (want(I)) E = fx_image<FX, GT>(st, F::UB, lt, g, fxr);
+                if (want(I)) {
+                    E = fx_exponent<GT>(fxr, g);
+                    if (E >= 0) fx_own(pl, [&](int q, bool scalar) { fx_align_at<FX>(st + q, E, scalar); });
+                    group_sync<GT>(g);
+                }
             }
             body(I, st, lt, E);
         }
@@ -567,6 +503,12 @@ constexpr int fas_threads() {
     return NV < 32 ? 32 : (NV > kThreads ? kThreads : NV);
 }
 
+// FP64 leaf residuals that align their images: in 3D, and in 2D where the
+// residual goes to FP32 (R); the norms of 2D FP64 cycles keep their rounding,
+// near which hundreds of small trees decide on one more cycle.
+template <int D, typename T, typename R>
+constexpr bool fx_leaf() { return sizeof(T) == 8 && (D == 3 || sizeof(R) == 4); }
+
 // threads per box of the leaf residual: as the FAS kernel, but FP64 boxes take
 // fewer where the several boxes per block that this gives leave several blocks
 // an SM: 128 in 3D (aligned images; four blocks of 64 registers), 64 in 2D (two
@@ -587,8 +529,60 @@ constexpr int leaf_blocks() {
     return sizeof(T) == 8 && (D == 2 || leaf_threads<D, M, T, R>() == 128) ? 4 : 1;
 }
 
+template <int D, typename T>
+constexpr bool fx_restrict() { return sizeof(T) == 8 && D == 3; }
+// sum_outside - D sum_c u over 2^D children with D outside neighbours each
+template <int D>
+constexpr int fx_restrict_weight() { return 2 * D * (1 << D); }
+
+// Residual and restriction of one box on its aligned image (3D).  The sums are
+// exact integers, so they may be split: four threads per coarse cell take the
+// two children of a row each and add up by shuffles (a thread per coarse cell
+// left three quarters of an FP64 box's threads idle and made 43 FP64 additions,
+// 64 cycles each, in a chain).  Left in FP64: the sum of the children's source
+// and one FMA.  The two roundings run side by side, in two threads of the four.
+// 256^3: 0.213 -> 0.165 ms.
+template <int D, int M, int MP, int GT>
+__device__ __forceinline__ void rr_aligned(const BoxMeta &A, const BoxInfo &I, const double *st, int lt, int E,
+                                           double ih2, long long cp, double *u, double *rho, double *vold) {
+    static_assert(D == 3, "3D");
+    using F = FpCfg<D, M, double, GT>;
+    constexpr int MH = M / 2, NCO = MH * MH * MH, W = fx_restrict_weight<D>();
+    const long long *im = reinterpret_cast<const long long *>(st), *X = im + 2 * F::PT;
+    const double *R = st + F::UB;
+    const int q = lt & 3, dy = q & 1, dz = q >> 1;
+    static_assert(NCO * 4 % GT == 0 || GT == 4 * NCO || NCO * 4 > GT, "whole quads");
+    for (int c = lt >> 2; c < NCO; c += GT / 4) {
+        const int Xc = c % MH, Y = (c / MH) % MH, Z = c / (MH * MH);
+        const int j = 2 * Y + dy, k = 2 * Z + dz, row = sp_row<D, M>(j, k), p = (j + k + D) & 1;
+        const int oy = dy ? MH : -MH, oz = (dz ? M + 2 : -(M + 2)) * MH;
+        const long long *a = im + p * F::PT + row * MH + Xc, *b = im + (1 - p) * F::PT + row * MH + Xc;
+        long long su = a[0] + b[0];  // children 2X (colour p) and 2X + 1
+        long long so = (Xc > 0 ? b[-1] : X[row]) + (Xc + 1 < MH ? a[1] : X[F::ROWS + row]);
+        so += b[oy] + a[oy] + b[oz] + a[oz];
+        const int rq = (k * M + j) * MH + Xc;
+        double sr = R[rq] + R[F::H + rq];
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            su += __shfl_xor_sync(0xffffffffu, su, o);
+            so += __shfl_xor_sync(0xffffffffu, so, o);
+            sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        }
+        // thread 0: the mean of u; thread 1: the mean of h^2 A u
+        const double d = fx_round<W>(q == 1 ? so - D * su : su, E - D);
+        const double lap = __shfl_down_sync(0xffffffffu, d, 1);
+        if (q == 0) {
+            const int pi = unpack_off(I.poff, 0) + Xc, pj = unpack_off(I.poff, 1) + Y, pk = unpack_off(I.poff, 2) + Z;
+            const long long g = cp + rbi<D, MP>(pi, pj, pk);
+            u[g] = d;
+            vold[g] = d;
+            rho[g] = fma(-ih2, lap, sr * (1.0 / (1 << D)));
+        }
+    }
+}
+
 // Fused residual + restriction, staged version of k_resid_restrict (same
-// arithmetic and summation order).
+// arithmetic and summation order where the image is not aligned).
 template <int D, int M, int MP, typename T>
 __global__ void __launch_bounds__(kThreads) k_resid_restrict_p(BoxMeta A, int b0, int n, T *u, T *rho, T *vold,
                                                                T ih2, int hom) {
@@ -596,12 +590,19 @@ __global__ void __launch_bounds__(kThreads) k_resid_restrict_p(BoxMeta A, int b0
     using F = FpCfg<D, M, T, GT>;
     constexpr int MH = M / 2;
     constexpr int NCO = D == 2 ? MH * MH : MH * MH * MH;
+    constexpr int FX = fx_restrict<D, T>() ? fx_restrict_weight<D>() : 0;
     pdl_trigger();
     auto want = [](const BoxInfo &) { return true; };
     auto flat = [&](const BoxInfo &) -> const T * { return rho; };
-    auto body = [&](const BoxInfo &I, const T *st, int lt, int) {
+    auto body = [&](const BoxInfo &I, const T *st, int lt, int E) {
         const T *X = st + 2 * F::PT, *R = st + F::UB;
         const long long cp = A.coff[I.parent];
+        if constexpr (FX > 0) {
+            if (E >= 0) {
+                rr_aligned<D, M, MP, GT>(A, I, st, lt, E, ih2, cp, u, rho, vold);
+                return;
+            }
+        }
         for (int c = lt; c < NCO; c += F::G) {
             const int Xc = c % MH, Y = (c / MH) % MH, Z = D == 3 ? c / (MH * MH) : 0;
             // sum_c (A u)_c = (sum_outside - D sum_c u) / h^2 over the 2^D children
@@ -635,7 +636,7 @@ __global__ void __launch_bounds__(kThreads) k_resid_restrict_p(BoxMeta A, int b0
         }
     };
     auto none = [](const BoxInfo *) {};
-    fp_walk<D, M, T, GT, true, sizeof(T) == 4>(A, b0, n, nullptr, u, hom, want, flat, body, none, none);
+    fp_walk<D, M, T, GT, true, sizeof(T) == 4 || (FX > 0), FX>(A, b0, n, nullptr, u, hom, want, flat, body, none, none);
 }
 
 // FAS coarse right-hand side, staged version of k_fas: refined boxes get
@@ -647,10 +648,13 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
     constexpr int GT = fas_threads<D, M, T>();
     using F = FpCfg<D, M, T, GT>;
     constexpr int VEC = F::VEC, NVH = F::H / VEC;
+    constexpr int FX = fx_restrict<D, T>() ? fx_lap_weight<D>() : 0;
+    FxPlan<D, M, GT> fxp;
+    if constexpr (FX > 0) fxp.init(threadIdx.x % F::G);
     pdl_trigger();
     auto want = [](const BoxInfo &I) { return (I.flag & BF_REFINED) != 0; };
     auto flat = [&](const BoxInfo &I) -> const T * { return (I.flag & BF_REFINED) ? rho : u; };
-    auto body = [&](const BoxInfo &I, const T *st, int lt, int) {
+    auto body = [&](const BoxInfo &I, const T *st, int lt, int E) {
         const T *FL = st + F::UB;
         if (!(I.flag & BF_REFINED)) {
             for (int v = lt; v < F::NV; v += F::G) {
@@ -660,12 +664,8 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
             }
             return;
         }
-        for (int v = lt; v < F::NV; v += F::G) {
-            const int col = v / NVH, w = v % NVH;
-            const int row = w / F::NVR, h0 = (w % F::NVR) * VEC;
-            const int j = row % M, k = D == 2 ? 0 : row / M;
-            T lap[VEC], rv[VEC], out[VEC];
-            fp_lap_vec<D, M, T, false>(st, col, j, k, h0, lap);  // FP64 adds: the integer path costs registers here
+        auto finish = [&](int v, const T *lap) {
+            T rv[VEC], out[VEC];
             ldv<T, VEC>(FL + v * VEC, rv);
 #pragma unroll
             for (int x = 0; x < VEC; ++x) out[x] = fma(ih2, lap[x], rv[x]);
@@ -675,10 +675,30 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
                 for (int x = 0; x < VEC; ++x) out[x] *= chat;
                 stv<T, VEC>(rhoh + I.coff + (long long)v * VEC, out);
             }
+        };
+        if constexpr (FX > 0) {
+            if (E >= 0) {
+#pragma unroll
+                for (int it = 0; it < FxPlan<D, M, GT>::NIV; ++it) {
+                    if (lt + it * F::G >= F::NV) continue;
+                    T lap[VEC];
+                    fp_lap_vec_fx<D, M, GT>(st, E, fxp, it, lap);
+                    finish(lt + it * F::G, lap);
+                }
+                return;
+            }
+        }
+        for (int v = lt; v < F::NV; v += F::G) {
+            const int col = v / NVH, w = v % NVH;
+            const int row = w / F::NVR, h0 = (w % F::NVR) * VEC;
+            const int j = row % M, k = D == 2 ? 0 : row / M;
+            T lap[VEC];
+            fp_lap_vec<D, M, T, false>(st, col, j, k, h0, lap);  // FP64 adds: the integer path costs registers here
+            finish(v, lap);
         }
     };
     auto none = [](const BoxInfo *) {};
-    fp_walk<D, M, T, GT>(A, b0, n, nullptr, u, hom, want, flat, body, none, none);
+    fp_walk<D, M, T, GT, true, (FX > 0), FX>(A, b0, n, nullptr, u, hom, want, flat, body, none, none);
 }
 
 // Composite residual on the leaves (Eq. residual with the ghost rules of
@@ -772,7 +792,7 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
             cur = tr;
         }
     };
-    fp_walk<D, M, T, GT, (FX > 0), (FX > 0), FX>(A, 0, n, list, u, hom, want, flat, body, pre, post);
+    fp_walk<D, M, T, GT, (FX > 0), (FX > 0), FX, true>(A, 0, n, list, u, hom, want, flat, body, pre, post);
     flush_max(rm, pm, cur, cur >= 0, rmax, pmax, red);
 }
 

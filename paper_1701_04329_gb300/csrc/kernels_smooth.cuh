@@ -119,7 +119,7 @@ struct SpPlan {
             const int v = lt + it * S::G;
             const int row = v / S::NVR, h0 = (v % S::NVR) * S::VEC;
             const int j = row % M, k = D == 2 ? 0 : row / M;
-            vdst[it] = sp_row<D, M>(j, k) * MH + h0;
+            vdst[it] = v < S::NV ? sp_row<D, M>(j, k) * MH + h0 : -1;
             vsrc[it] = hrow<D, M>(j, k) + h0;
         }
 #pragma unroll
@@ -302,6 +302,110 @@ __device__ __forceinline__ void sp_fix(const BoxInfo &I, const BoxMeta &A, const
     }
 }
 
+// barrier of one box's thread group (g: its number in the block).  The barrier
+// numbers are constants: with one in a register a block reserves all 16, and an
+// SM holds four such blocks at most.
+template <int G, int X = 0>
+__device__ __forceinline__ void group_sync(int g) {
+    if constexpr (G <= 32) {
+        __syncwarp(G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1) << ((threadIdx.x & 31) / G * G));
+    } else if constexpr (G >= kThreads) {
+        __syncthreads();
+    } else {
+        if (g == X) asm volatile("bar.sync %0, %1;" ::"n"(X + 1), "n"(G) : "memory");
+        else if constexpr (X + 1 < kThreads / G) group_sync<G, X + 1>(g);
+    }
+}
+
+// The barrier of a box's step: a box's stages and metadata belong to its thread
+// group, so whole warps meet their group only (256^3, FP64 half-sweep: 73.9 -> 72.2 us, FP32
+// restriction 50.7 -> 49.1 us); smaller groups meet the block.  Returns whether to take the extra step:
+// `extra` of this group's box, or of any box of the block.
+template <int G>
+__device__ __forceinline__ bool box_sync(int g, bool extra) {
+    if constexpr (G >= 32) {
+        group_sync<G>(g);
+        return extra;
+    } else {
+        return __syncthreads_or(extra);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 images in fixed point.  GB300 issues one FP64 instruction per 64 cycles
+// and warp, and aligning every term of every sum to its cell's largest
+// exponent (fx_sum) takes some 25 integer instructions a term.  A staged
+// image is read seven times over, so it is aligned once instead: every value
+// to the largest exponent E of the box and its ghosts, in place, as a 64-bit
+// integer with G guard bits below the last bit of a value of that exponent.
+// Sums of neighbours are then integer additions, exact, rounded once.
+//
+// The truncated bits are at most one unit of 2^-6 ulp (of the box's largest
+// value) per term; FP64 additions round to half an ulp of every partial sum.
+// A box whose values span more than 2^kFxSpan keeps the alignment per cell
+// (its small values would lose bits), and so does one whose largest exponent
+// is out of fx_sum's range (all zero, infinite, NaN).
+// ---------------------------------------------------------------------------
+constexpr int kFxSpan = 8;
+template <int D>
+constexpr int fx_lap_weight() { return 4 * D; }  // sum_nb u - 2D u
+
+// A thread aligns what it staged itself, so finding E costs no pass over the
+// image and no barrier of its own: after its wait a thread folds its values'
+// magnitudes (fx_fold), its warp leaves their extremes in `red` (two ints per
+// warp) ahead of the barrier that every box has, every thread then knows E
+// (fx_exponent), and after the alignment the group meets once more.
+__device__ __forceinline__ void fx_fold(double x, double y, unsigned &mx, unsigned &mn) {
+    const unsigned a = (unsigned)__double2hiint(x) & 0x7fffffffu, b = (unsigned)__double2hiint(y) & 0x7fffffffu;
+    const unsigned m = a > b ? a : b;
+    mx = m > mx ? m : mx;
+    if (m) mn = m < mn ? m : mn;
+}
+__device__ __forceinline__ void fx_leave(unsigned mx, unsigned mn, int *red) {
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    if ((threadIdx.x & 31) == 0) reinterpret_cast<int2 *>(red)[threadIdx.x >> 5] = make_int2((int)mx, (int)mn);
+}
+// exponent of group g's values, or -1 where they are not aligned
+template <int G>
+__device__ __forceinline__ int fx_exponent(const int *red, int g) {
+    static_assert(G >= 32, "whole warps per box");
+    unsigned mx = 0, mn = 0x7fffffffu;
+#pragma unroll
+    for (int x = 0; x < G / 32; ++x) {
+        const int2 r = reinterpret_cast<const int2 *>(red)[g * (G / 32) + x];
+        mx = max(mx, (unsigned)r.x);
+        mn = min(mn, (unsigned)r.y);
+    }
+    const int E = (int)(mx >> 20);
+    return E >= kFxEmin && E <= kFxEmax && E - (int)(mn >> 20) <= kFxSpan ? E : -1;
+}
+template <int W>
+__device__ __forceinline__ void fx_align_at(double *p, int E, bool scalar) {
+    if (scalar) {
+        *p = __longlong_as_double(fx_align<W>(*p, E));
+    } else {
+        const double2 q = *reinterpret_cast<const double2 *>(p);
+        *reinterpret_cast<longlong2 *>(p) = make_longlong2(fx_align<W>(q.x, E), fx_align<W>(q.y, E));
+    }
+}
+// f(slot, scalar) for every value the thread staged through its plan
+template <typename Plan, typename F>
+__device__ __forceinline__ void fx_own(const Plan &pl, F f) {
+#pragma unroll
+    for (int it = 0; it < (int)(sizeof(pl.vdst) / sizeof(int)); ++it)
+        if (pl.vdst[it] >= 0) f(pl.vdst[it], false);
+#pragma unroll
+    for (int q = 0; q < Plan::NQ; ++q)
+        if (pl.gdst[q] >= 0) f(pl.gdst[q] & 0xffff, (pl.gdst[q] & (1 << 19)) != 0);
+}
+template <typename Plan>
+__device__ __forceinline__ void fx_fold_own(const Plan &pl, const double *st, int *red) {
+    unsigned mx = 0, mn = 0x7fffffffu;
+    fx_own(pl, [&](int q, bool scalar) { fx_fold(st[q], scalar ? 0.0 : st[q + 1], mx, mn); });
+    fx_leave(mx, mn, red);
+}
+
 // resident blocks per SM the register allocation must allow (FP32 / FP64)
 constexpr int kSmoothMinBlocks32 = 6, kSmoothMinBlocks64 = 5;
 
@@ -310,9 +414,12 @@ constexpr int kSmoothMinBlocks32 = 6, kSmoothMinBlocks64 = 5;
 // the new values from the neighbours (in the order -x, +x, -y, +y, -z, +z) and
 // the staged source.  early(I, v, itv) runs for the same vectors before the
 // box's copies are waited for (loads of its own that upd needs).
-template <int D, int M, typename T, int VPT, typename Early, typename Upd>
+// FX > 0 (FP64): the staged values are aligned (fx_image, sums of weight FX) and
+// upd_fx(E, ...) forms the new values from them, upd only where they are not.
+template <int D, int M, typename T, int VPT, int FX = 0, typename Early, typename Upd, typename UpdFx>
 __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const int *list, T *u,
-                                        const T *__restrict__ rho, int colour, int hom, Early early, Upd upd) {
+                                        const T *__restrict__ rho, int colour, int hom, Early early, Upd upd,
+                                        UpdFx upd_fx) {
     using S = SpCfg<D, M, T, VPT>;
     constexpr int VEC = S::VEC, MH = S::MH, H = S::H, NST = S::NST, NI = NST + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -341,6 +448,7 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
         cr[itv] = r;
     }
     pdl_trigger();
+    __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
         info_load<D>(A, first + q * stride + g, n, b0, list, info[q * S::BPC + g], lt, S::G, false);
     pdl_wait();
@@ -365,8 +473,11 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
         const bool cf = b >= 0 && (I.flag & BF_CF);
         T *box = stages + ((it % NST) * S::BPC + g) * S::BOX;
         if (special) sp_fix_own<D, M, T, VPT>(pl, I, A, box, hom);  // domain sides: this thread's own items
+        if constexpr (FX > 0) {
+            if (b >= 0) fx_fold_own(pl, box, fxr);
+        }
         // one barrier per box: the stage and metadata slot of the previous box are free after it
-        const int any_cf = __syncthreads_or(cf);
+        const int any_cf = box_sync<S::G>(g, cf);
         {
             const int q = it + NST - 1;
             const BoxInfo &In = info[(q % NI) * S::BPC + g];
@@ -375,11 +486,15 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
         }
         info_load<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * S::BPC + g], lt, S::G);
         if (any_cf) {  // refinement-boundary ghosts read cells other threads staged
-            if (cf) sp_fix<D, M, T, VPT>(I, A, u, box, lt, c, hom, true);
-            __syncthreads();
+            if (cf) {
+                sp_fix<D, M, T, VPT>(I, A, u, box, lt, c, hom, true);
+                if constexpr (FX > 0) fx_fold_own(pl, box, fxr);  // the thread's own items again
+            }
+            box_sync<S::G>(g, false);
         }
         if (b >= 0) {
             const T *R = box + S::PT + S::XT;
+            auto cells = [&](auto form) {
 #pragma unroll
             for (int itv = 0; itv < S::NIT; ++itv) {
                 if (lt + itv * S::G >= S::NV) continue;
@@ -404,20 +519,43 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
                     xl[x] = r ? xv[x] : side;
                     xr[x] = r ? side : xv[x];
                 }
-                upd(I, lt + itv * S::G, itv, xl, xr, ym, yp, zm, zp, rv, out);
+                form(I, lt + itv * S::G, itv, xl, xr, ym, yp, zm, zp, rv, out);
                 stv<T, VEC>(u + I.coff + c * H + (lt + itv * S::G) * VEC, out);
+            }
+            };
+            if constexpr (FX > 0) {
+                const int E = fx_exponent<S::G>(fxr, g);
+                if (E >= 0) fx_own(pl, [&](int q, bool scalar) { fx_align_at<FX>(box + q, E, scalar); });
+                group_sync<S::G>(g);
+                if (E >= 0)
+                    cells([&](const BoxInfo &, int, int, const T (&xl)[VEC], const T (&xr)[VEC], const T (&ym)[VEC],
+                              const T (&yp)[VEC], const T (&zm)[VEC], const T (&zp)[VEC], const T (&rv)[VEC],
+                              T (&out)[VEC]) { upd_fx(E, xl, xr, ym, yp, zm, zp, rv, out); });
+                else cells(upd);
+            } else {
+                cells(upd);
             }
         }
     }
     cp_wait<0>();
 }
 
-// scaled = 1: rho holds -h^2 rho / (2D) and the update is u = sum/(2D) + rho
+// FP64 half-sweeps in 3D whose boxes take whole warps align their images: 256^3
+// 100.5 -> 72.2 us, 194 instead of 249 instructions and one instead of five FP64
+// issues per update; 18.8 M unknowns, FP64, 29.0 -> 23.3 ms with the restriction
+// and the coarse right-hand side on aligned images too (2D keeps the per-cell
+// sums: its four terms need no FP64 addition).
+template <int D, int M, typename T, int VPT>
+constexpr bool fx_smooth() { return sizeof(T) == 8 && D == 3 && SpCfg<D, M, T, VPT>::G >= 32; }
+
+// FP64: rho holds -h^2 rho / (2D) and the update is u = sum/(2D) + rho (a choice
+// at run time would cost the other form's two FP64 instructions per update,
+// which the compiler runs too and selects)
 template <int D, int M, typename T, int VPT = 1>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 : kSmoothMinBlocks64)
-    k_smooth_p(BoxMeta A, int b0, int n, const int *list, T *u, const T *__restrict__ rho, T h2, int colour, int hom,
-               int scaled) {
+    k_smooth_p(BoxMeta A, int b0, int n, const int *list, T *u, const T *__restrict__ rho, T h2, int colour, int hom) {
     constexpr int VEC = SpCfg<D, M, T, VPT>::VEC;
+    constexpr bool kScaled = sizeof(T) == 8;
     const T inv = T(1) / T(2 * D);
     auto early = [](const BoxInfo &, int, int) {};
     auto upd = [&](const BoxInfo &, int, int, const T (&xl)[VEC], const T (&xr)[VEC], const T (&ym)[VEC],
@@ -425,10 +563,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? kSmoothMinBlocks32 
 #pragma unroll
         for (int x = 0; x < VEC; ++x) {
             const T sum = nb_sum6<D, T>(xl[x], xr[x], ym[x], yp[x], D == 3 ? zm[x] : T(0), D == 3 ? zp[x] : T(0));
-            out[x] = scaled ? fma(sum, inv, rv[x]) : (sum - h2 * rv[x]) * inv;
+            out[x] = kScaled ? fma(sum, inv, rv[x]) : (sum - h2 * rv[x]) * inv;
         }
     };
-    sp_walk<D, M, T, VPT>(A, b0, n, list, u, rho, colour, hom, early, upd);
+    auto upd_fx = [&](int E, const T (&xl)[VEC], const T (&xr)[VEC], const T (&ym)[VEC], const T (&yp)[VEC],
+                      const T (&zm)[VEC], const T (&zp)[VEC], const T (&rv)[VEC], T (&out)[VEC]) {
+        auto i = [](T v) { return __double_as_longlong(v); };
+#pragma unroll
+        for (int x = 0; x < VEC; ++x) {
+            const long long S = i(xl[x]) + i(xr[x]) + i(ym[x]) + i(yp[x]) + i(zm[x]) + i(zp[x]);
+            out[x] = fma(fx_round<2 * D>(S, E), inv, rv[x]);
+        }
+    };
+    constexpr int FX = fx_smooth<D, M, T, VPT>() ? 2 * D : 0;
+    sp_walk<D, M, T, VPT, FX>(A, b0, n, list, u, rho, colour, hom, early, upd, upd_fx);
 }
 
 }  // namespace afg

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kThreads) k_var_smooth_p(BoxMeta A, int b0, in
             out[x] = var_quot<T>(fma(-h2, rv[x], var_dot<D, T>(c, w)), cf[itv][2 * D][x], cf[itv][2 * D + 1][x]);
         }
     };
-    sp_walk<D, M, T, 1>(A, b0, n, nullptr, u, rho, colour, hom, early, upd);
+    sp_walk<D, M, T, 1>(A, b0, n, nullptr, u, rho, colour, hom, early, upd, [](auto &&...) {});
 }
 
 // For the VEC cells of colour col at half-row (j,k), h0..h0+VEC-1 (storage

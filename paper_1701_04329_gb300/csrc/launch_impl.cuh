@@ -70,7 +70,7 @@ void do_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *l
                 const size_t smem = S::smem();
                 auto k = k_smooth_p<D, M, T, 2>;
                 launch_pdl(k, grid_for(k, smem, (n + S::BPC - 1) / S::BPC), smem, c.stream, A, b0, n, list, (T *)u,
-                           (const T *)(rhoh ? rhoh : rho), T(h2), colour, hom, rhoh ? 1 : 0);
+                           (const T *)rho, T(h2), colour, hom);
                 ++g_launches;
                 return;
             }
@@ -79,8 +79,9 @@ void do_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *l
             using S = SpCfg<D, M, T>;
             const size_t smem = S::smem();
             auto k = k_smooth_p<D, M, T>;
+            if (sizeof(T) == 8 && !rhoh) throw std::runtime_error("FP64 half-sweeps read the pre-scaled source");
             launch_pdl(k, grid_for(k, smem, (n + S::BPC - 1) / S::BPC), smem, c.stream, A, b0, n, list, (T *)u,
-                       (const T *)(rhoh ? rhoh : rho), T(h2), colour, hom, rhoh ? 1 : 0);
+                       (const T *)(sizeof(T) == 8 ? rhoh : rho), T(h2), colour, hom);
             ++g_launches;
             return;
         }
