@@ -292,7 +292,7 @@ int solve_mixed(Grid &g, const afg_mg_opts &o, cudaStream_t s, std::vector<std::
 }
 
 double host_scalar(Grid &g, cudaStream_t s) {
-    check(cudaMemcpyAsync(g.h_scalar, g.d_scalar, sizeof(double), cudaMemcpyDeviceToHost, s), "scalar");
+    check(cudaMemcpyAsync(g.h_scalar, g.d_scalar, 2 * sizeof(double), cudaMemcpyDeviceToHost, s), "scalar");
     check(cudaStreamSynchronize(s), "scalar");
     return *g.h_scalar;
 }
@@ -323,26 +323,28 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
         afg::launch_leaf_absmax(lc, A, L, n, a, g.d_partials, g.d_scalar);
         return host_scalar(g, s);
     };
+    // out = a x + b y with max |out| (the result) and out . w (in *dotw)
+    auto update = [&](double *out, double a, const double *xv, double b, const double *yv, const double *w,
+                      double *dotw) {
+        afg::launch_leaf_reduce2(lc, A, L, n, out, a, xv, b, yv, w, g.d_partials, g.d_scalar);
+        const double m = host_scalar(g, s);
+        if (dotw) *dotw = g.h_scalar[1];
+        return m;
+    };
     const size_t bytes = (size_t)g.ncell * 8;
     // AFG_MIXED: M is one FP32 V-cycle (the BiCGStab recurrences and K^T stay FP64)
     const bool m32 = o.precision == AFG_MIXED;
     if (m32) g.ensure_mixed();
     auto precond = [&](const double *in, double *out, cudaStream_t cs) {
-        afg::launch_leaf_scale(g.leaf_cfg(true, cs), A, g.d_hb, L, n, g.wsadj.rho->as<double>(), in, -1);
-        if (m32) {
-            afg::launch_to_f32(g.wsadj.rho->as<double>(), g.ws32.rho->as<float>(), g.ncell, cs);
-            check(cudaMemsetAsync(g.ws32.u->p, 0, (size_t)g.ncell * 4, cs), "zero");
-            g.vcycle(g.ws32, g.lmax, mo, 1, nullptr, cs);
-            afg::launch_to_f64(g.ws32.u->as<float>(), g.wsadj.u->as<double>(), g.ncell, cs);
-        } else {
-            g.leaf_rho_hat(g.wsadj, cs);
-            check(cudaMemsetAsync(g.wsadj.u->p, 0, bytes, cs), "zero");
-            g.vcycle(g.wsadj, g.lmax, mo, 1, nullptr, cs);
-        }
-        afg::launch_leaf_scale(g.leaf_cfg(true, cs), A, g.d_hb, L, n, out, g.wsadj.u->as<double>(), 1);
+        afg::Workspace &w = m32 ? g.ws32 : g.wsadj;
+        afg::launch_precond_in(g.leaf_cfg(!m32, cs), A, L, n, in, w.rho->p, w.rhoh_p());
+        check(cudaMemsetAsync(w.u->p, 0, (size_t)g.ncell * (m32 ? 4 : 8), cs), "zero");
+        g.vcycle(w, g.lmax, mo, 1, nullptr, cs);
+        afg::launch_precond_out(g.leaf_cfg(!m32, cs), A, L, n, w.u->p, out);
     };
     auto apply_T = [&](const double *in, double *out) {
-        afg::launch_adjoint_apply(lc, A, g.d_child, g.d_hb, L, n, in, out);
+        afg::launch_adjoint_plain(lc, A, g.d_adj_plain, g.n_adj_plain, in, out);
+        afg::launch_adjoint_apply(lc, A, g.d_child, g.d_hb, g.d_adj_rest, g.n_adj_rest, in, out);
     };
     // graphs for the two preconditioner applications (fixed buffers)
     const int kp = m32 ? 22 : 20;
@@ -364,31 +366,30 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
     check(cudaMemsetAsync(p, 0, bytes, s), "zero");
     check(cudaMemsetAsync(v, 0, bytes, s), "zero");
     double rho_old = 1.0, alpha = 1.0, omega = 1.0;
+    double rho_new = dot(rh, r);
     int it = 0;
     double res = 1.0;
     for (it = 1; it <= o.max_cycles; ++it) {
-        const double rho_new = dot(rh, r);
         if (rho_new == 0.0) break;
         const double beta = (rho_new / rho_old) * (alpha / omega);
         afg::launch_leaf_axpbypcz(lc, A, L, n, p, 1.0, r, beta, p, -beta * omega, v);
         P_p();
         apply_T(ph, v);
         alpha = rho_new / dot(rh, v);
-        afg::launch_leaf_axpbypcz(lc, A, L, n, sv, 1.0, r, -alpha, v, 0.0, nullptr);
-        res = amax(sv) / bnorm;
+        res = update(sv, 1.0, r, -alpha, v, nullptr, nullptr) / bnorm;
         if (res <= o.rel_tol) {
             afg::launch_leaf_axpbypcz(lc, A, L, n, x, 1.0, x, alpha, ph, 0.0, nullptr);
             break;
         }
         P_s();
         apply_T(sh, t);
-        const double tt = dot(t, t);
-        omega = tt > 0.0 ? dot(t, sv) / tt : 0.0;
+        afg::launch_leaf_reduce2(lc, A, L, n, nullptr, 0.0, t, 0.0, sv, nullptr, g.d_partials, g.d_scalar);
+        const double tt = host_scalar(g, s);
+        omega = tt > 0.0 ? g.h_scalar[1] / tt : 0.0;
         afg::launch_leaf_axpbypcz(lc, A, L, n, x, 1.0, x, alpha, ph, omega, sh);
-        afg::launch_leaf_axpbypcz(lc, A, L, n, r, 1.0, sv, -omega, t, 0.0, nullptr);
-        res = amax(r) / bnorm;
-        if (res <= o.rel_tol || omega == 0.0) break;
         rho_old = rho_new;
+        res = update(r, 1.0, sv, -omega, t, rh, &rho_new) / bnorm;  // rho_new = rh . r, of the next step
+        if (res <= o.rel_tol || omega == 0.0) break;
     }
     // true residual
     apply_T(x, t);

@@ -300,6 +300,16 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     d_child = upload(child, own);
     d_leaves = upload(leaves, own);
     d_leaf_geo = upload(leaf_geo, own);
+    std::vector<int> plain, rest;
+    for (int g : leaves) {
+        bool ok = true;
+        for (int s = 0; s < S; ++s) ok = ok && nb[g * S + s] >= -1 && (nb[g * S + s] < 0 || !(bflag[nb[g * S + s]] & BF_REFINED));
+        (ok ? plain : rest).push_back(g);
+    }
+    n_adj_plain = (int)plain.size();
+    n_adj_rest = (int)rest.size();
+    d_adj_plain = upload(plain, own);
+    d_adj_rest = upload(rest, own);
     if (singular && T > 1) {  // forests: per-tree compatibility constants and means
         std::vector<int> leaf0(T + 1, 0);
         for (int t = 0; t < T; ++t) leaf0[t + 1] = leaf0[t] + (int)trees[t]->leaves.size();
@@ -338,13 +348,13 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     d_nactive = own.back()->as<int>();
     own.emplace_back(new DevBuf(kPartials * sizeof(double)));
     d_partials = own.back()->as<double>();
-    own.emplace_back(new DevBuf(sizeof(double)));
+    own.emplace_back(new DevBuf(2 * sizeof(double)));
     d_scalar = own.back()->as<double>();
     own.emplace_back(new DevBuf(sizeof(double)));
     d_tol = own.back()->as<double>();
     check(cudaMallocHost((void **)&h_norms, 2 * T * sizeof(unsigned long long)), "cudaMallocHost");
     check(cudaMallocHost((void **)&h_nactive, sizeof(int)), "cudaMallocHost");
-    check(cudaMallocHost((void **)&h_scalar, sizeof(double)), "cudaMallocHost");
+    check(cudaMallocHost((void **)&h_scalar, 2 * sizeof(double)), "cudaMallocHost");
     alloc_ws(ws64, true);
 }
 

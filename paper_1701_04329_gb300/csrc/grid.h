@@ -122,6 +122,9 @@ class Grid {
     double *d_leaf_geo = nullptr;  // per leaf box (canonical order): lower corner x, y, z and cell size
     int *d_cf_children = nullptr;  // children of parents that face a same-level leaf
     int n_cf_children = 0;
+    // leaf boxes without / with a refined neighbour or a refinement boundary (the adjoint's operator)
+    int *d_adj_plain = nullptr, *d_adj_rest = nullptr;
+    int n_adj_plain = 0, n_adj_rest = 0;
     int *d_child = nullptr;
     double *d_hb = nullptr;
     double *d_bc = nullptr;
@@ -220,7 +223,5 @@ void launch_flag(const Grid &g, const double *f, int power, double tau_ref, doub
 void launch_leaf_center(const Grid &g, double *f, bool with_flux, cudaStream_t s);
 // dst = (float) src, n values
 void launch_to_f32(const double *src, float *dst, long long n, cudaStream_t s);
-// dst = (double) src, n values
-void launch_to_f64(const float *src, double *dst, long long n, cudaStream_t s);
 
 }  // namespace afg

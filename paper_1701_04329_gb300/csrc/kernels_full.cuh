@@ -809,6 +809,59 @@ __global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>()) k_leaf_re
     leaf_residual_walk<D, M, T, R, GT, FX>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
 }
 
+// The transposed operator on leaf boxes whose sides all face same-level leaves
+// or the domain boundary: there K^T is the homogeneous operator itself, so the
+// box is staged, aligned and summed like a residual (h^-2 is a power of two
+// and joins the rounding: no FP64 instruction).  The others take
+// k_adjoint_apply, which gathers the coupling across refinement boundaries and
+// spends eight FP64 additions a cell (4.3 M cells: 89 us for all boxes).
+template <int D, int M>
+__global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, double, float>()) k_adjoint_plain_p(
+    BoxMeta A, const int *list, int n, const double *lam, double *out) {
+    constexpr int GT = leaf_threads<D, M, double, float>(), FX = GT >= 32 ? fx_lap_weight<D>() : 0;
+    using F = FpCfg<D, M, double, GT>;
+    constexpr int NVH = F::H / 2;
+    FxPlan<D, M, GT> fxp;
+    fxp.init(threadIdx.x % F::G);
+    pdl_trigger();
+    auto want = [](const BoxInfo &) { return true; };
+    auto flat = [](const BoxInfo &) -> const double * { return nullptr; };
+    auto body = [&](const BoxInfo &I, const double *st, int lt, int E) {
+        const double ih2 = A.ih2[I.b];
+        const int e2 = (int)(__double_as_longlong(ih2) >> 52) - 1023;
+        if (E >= 0 && E + e2 <= 2040) {
+#pragma unroll
+            for (int it = 0; it < FxPlan<D, M, GT>::NIV; ++it) {
+                const int v = lt + it * F::G;
+                if (v >= F::NV) continue;
+                double lap[2];
+                fp_lap_vec_fx<D, M, GT>(st, E + e2, fxp, it, lap);
+                stv<double, 2>(out + I.coff + v * 2, lap);
+            }
+            return;
+        }
+        for (int v = lt; v < F::NV; v += F::G) {
+            double lap[2];
+            if (E >= 0) {  // near the end of the exponent range: h^-2 by itself
+                const int col = v / NVH;
+                (void)col;
+#pragma unroll
+                for (int it = 0; it < FxPlan<D, M, GT>::NIV; ++it)
+                    if (v == lt + it * F::G) fp_lap_vec_fx<D, M, GT>(st, E, fxp, it, lap);
+            } else {
+                const int col = v / NVH, w = v % NVH;
+                const int row = w / F::NVR, h0 = (w % F::NVR) * 2;
+                fp_lap_vec<D, M, double>(st, col, row % M, D == 2 ? 0 : row / M, h0, lap);
+            }
+            lap[0] *= ih2;
+            lap[1] *= ih2;
+            stv<double, 2>(out + I.coff + v * 2, lap);
+        }
+    };
+    auto none = [](const BoxInfo *) {};
+    fp_walk<D, M, double, GT, true, true, FX>(A, 0, n, list, lam, 1, want, flat, body, none, none);
+}
+
 // ---------------------------------------------------------------------------
 // Coarse-grid correction u_h += I_H^h (v_H - v'_H) (Eq. coarse-corr), staged
 // version of k_correct: a box's own values (16-byte copies) and the parent's

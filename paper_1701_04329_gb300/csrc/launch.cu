@@ -173,8 +173,16 @@ void launch_leaf_axpbypcz(const LaunchCfg &c, const BoxMeta &A, const int *list,
                           const double *x, double b, const double *y, double cc, const double *z) {
     AFG_BY_DIM(axpbypcz, c, A, list, n, out, a, x, b, y, cc, z);
 }
-void launch_leaf_scale(const LaunchCfg &c, const BoxMeta &A, const double *hb, const int *list, int n, double *out,
-                       const double *x, int power) { AFG_BY_DIM(scale, c, A, hb, list, n, out, x, power); }
+void launch_precond_in(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x, void *rho,
+                       void *rhoh) { AFG_BY_DIM(precond_in, c, A, list, n, x, rho, rhoh); }
+void launch_precond_out(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u, double *out) {
+    AFG_BY_DIM(precond_out, c, A, list, n, u, out);
+}
+void launch_leaf_reduce2(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, double *out, double a,
+                         const double *x, double b, const double *y, const double *w, double *partials,
+                         double *result) { AFG_BY_DIM(reduce2, c, A, list, n, out, a, x, b, y, w, partials, result); }
+void launch_adjoint_plain(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *lam,
+                          double *out) { AFG_BY_DIM(adjoint_plain, c, A, list, n, lam, out); }
 void launch_leaf_dot(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x, const double *y,
                      double *partials, double *result) { AFG_BY_DIM(reduce, c, A, list, n, x, y, 0, partials, result); }
 void launch_leaf_absmax(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x,

@@ -76,9 +76,18 @@ void launch_adjoint_db(const LaunchCfg &, const BoxMeta &, const double *hb, con
 // leaf vectors (double): out = a x + b y + c z (y, z may be null)
 void launch_leaf_axpbypcz(const LaunchCfg &, const BoxMeta &, const int *list, int n, double *out, double a,
                           const double *x, double b, const double *y, double c, const double *z);
-// out = x * h^(D*power) per box (power = +1 or -1)
-void launch_leaf_scale(const LaunchCfg &, const BoxMeta &, const double *hb, const int *list, int n, double *out,
-                       const double *x, int power);
+// the adjoint's preconditioner, in the precision of cfg: rho = x / h^D (and the
+// pre-scaled source rhoh, or null), out = u h^D
+void launch_precond_in(const LaunchCfg &, const BoxMeta &, const int *list, int n, const double *x, void *rho,
+                       void *rhoh);
+void launch_precond_out(const LaunchCfg &, const BoxMeta &, const int *list, int n, const void *u, double *out);
+// result[0], result[1] (device, deterministic): x . x and x . y (out null); or, with
+// out = a x + b y, max |out| and out . w (w null: 0)
+void launch_leaf_reduce2(const LaunchCfg &, const BoxMeta &, const int *list, int n, double *out, double a,
+                         const double *x, double b, const double *y, const double *w, double *partials,
+                         double *result);
+// out = K^T lam on leaf boxes without a refinement boundary or a refined neighbour
+void launch_adjoint_plain(const LaunchCfg &, const BoxMeta &, const int *list, int n, const double *lam, double *out);
 // dot product / max norm over leaf cells into *result (device), deterministic
 void launch_leaf_dot(const LaunchCfg &, const BoxMeta &, const int *list, int n, const double *x, const double *y,
                      double *partials, double *result);

@@ -256,13 +256,44 @@ void do_axpbypcz(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, d
     ++g_launches;
 }
 
-template <int D, int M>
-void do_scale(const LaunchCfg &c, const BoxMeta &A, const double *hb, const int *list, int n, double *out,
-              const double *x, int power) {
+template <int D, int M, typename T>
+void do_precond_in(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x, void *rho,
+                   void *rhoh) {
     if (n <= 0) return;
-    auto k = k_leaf_scale<D, M>;
-    launch_pdl(k, grid_for(k, 0, work_ctas<D, M>(n)), 0, c.stream, A, hb, list, n, out, x, power);
+    auto k = k_precond_in<D, M, T>;
+    launch_pdl(k, grid_for(k, 0, work_ctas<D, M>(n)), 0, c.stream, A, list, n, x, (T *)rho, (T *)rhoh);
     ++g_launches;
+}
+
+template <int D, int M, typename T>
+void do_precond_out(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u, double *out) {
+    if (n <= 0) return;
+    auto k = k_precond_out<D, M, T>;
+    launch_pdl(k, grid_for(k, 0, work_ctas<D, M>(n)), 0, c.stream, A, list, n, (const T *)u, out);
+    ++g_launches;
+}
+
+template <int D, int M>
+void do_reduce2(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, double *out, double a, const double *x,
+                double b, const double *y, const double *w, double *partials, double *result) {
+    auto k = k_leaf_reduce2<D, M>;
+    const int grid = std::min(kPartials / 2, grid_for(k, 0, std::max(1, work_ctas<D, M>(n))));
+    launch_pdl(k, grid, 0, c.stream, A, list, n, out, a, x, b, y, w, partials);
+    k_reduce2_final<<<1, kThreads, 0, c.stream>>>(partials, grid, out != nullptr, result);
+    g_launches += 2;
+}
+
+template <int D, int M>
+void do_adjoint_plain(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *lam, double *out) {
+    if (n <= 0) return;
+    if constexpr (FpCfg<D, M, double>::ok && leaf_threads<D, M, double, float>() >= 32) {
+        using F = FpCfg<D, M, double, leaf_threads<D, M, double, float>()>;
+        auto k = k_adjoint_plain_p<D, M>;
+        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, lam, out);
+        ++g_launches;
+    } else {
+        throw std::runtime_error("leaf boxes have 4 cells per side or more");
+    }
 }
 
 template <int D, int M>
@@ -442,8 +473,14 @@ struct DimOps {
                            const double *lam, double *db);
     static void axpbypcz(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, double *out, double a,
                          const double *x, double b, const double *y, double cc, const double *z);
-    static void scale(const LaunchCfg &c, const BoxMeta &A, const double *hb, const int *list, int n, double *out,
-                      const double *x, int power);
+    static void precond_in(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x, void *rho,
+                           void *rhoh);
+    static void precond_out(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u, double *out);
+    static void reduce2(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, double *out, double a,
+                        const double *x, double b, const double *y, const double *w, double *partials,
+                        double *result);
+    static void adjoint_plain(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *lam,
+                              double *out);
     static void reduce(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x,
                        const double *y, int mode, double *partials, double *result);
 };
@@ -542,10 +579,39 @@ void DimOps<D>::axpbypcz(const LaunchCfg &c, const BoxMeta &A, const int *list, 
     AFG_SWITCH_M(c.M, (do_axpbypcz<D, MM>(c, A, list, n, out, a, x, b, y, cc, z)));
 }
 
+// leaf boxes: 4, 8 or 16 cells per side
+#define AFG_SWITCH_LEAF(M, BODY)                         \
+    switch (M) {                                         \
+        case 4: { constexpr int MM = 4; BODY; break; }   \
+        case 8: { constexpr int MM = 8; BODY; break; }   \
+        case 16: { constexpr int MM = 16; BODY; break; } \
+        default: bad_size(M, 0);                         \
+    }
+
 template <int D>
-void DimOps<D>::scale(const LaunchCfg &c, const BoxMeta &A, const double *hb, const int *list, int n, double *out,
-                      const double *x, int power) {
-    AFG_SWITCH_M(c.M, (do_scale<D, MM>(c, A, hb, list, n, out, x, power)));
+void DimOps<D>::precond_in(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x, void *rho,
+                           void *rhoh) {
+    if (c.fp64) { AFG_SWITCH_LEAF(c.M, (do_precond_in<D, MM, double>(c, A, list, n, x, rho, rhoh))); }
+    else { AFG_SWITCH_LEAF(c.M, (do_precond_in<D, MM, float>(c, A, list, n, x, rho, rhoh))); }
+}
+
+template <int D>
+void DimOps<D>::precond_out(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *u, double *out) {
+    if (c.fp64) { AFG_SWITCH_LEAF(c.M, (do_precond_out<D, MM, double>(c, A, list, n, u, out))); }
+    else { AFG_SWITCH_LEAF(c.M, (do_precond_out<D, MM, float>(c, A, list, n, u, out))); }
+}
+
+template <int D>
+void DimOps<D>::reduce2(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, double *out, double a,
+                        const double *x, double b, const double *y, const double *w, double *partials,
+                        double *result) {
+    AFG_SWITCH_LEAF(c.M, (do_reduce2<D, MM>(c, A, list, n, out, a, x, b, y, w, partials, result)));
+}
+
+template <int D>
+void DimOps<D>::adjoint_plain(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *lam,
+                              double *out) {
+    AFG_SWITCH_LEAF(c.M, (do_adjoint_plain<D, MM>(c, A, list, n, lam, out)));
 }
 
 template <int D>
