@@ -184,6 +184,7 @@ int solve_fp64(Grid &g, const afg_mg_opts &o, cudaStream_t s, std::vector<std::v
     };
     g.make_compatible(s);
     g.refresh_faces(s);
+    g.refresh_rho_hat(s);
     if (fmg_first) {
         run(g, {1, o.n_down, o.n_up, o.n_base, 0}, o.use_graph, s, [&](cudaStream_t cs) {
             g.fmg(g.ws64, mo, 0, forest, cs);
@@ -686,7 +687,7 @@ int afg_set_rhs(afg_tree *t, const double *rho) {
     AFG_ON_DEVICE(t);
     Grid &g = grid_of(t);
     afg::launch_leaf_set(g.leaf_cfg(true, t->stream), g.meta, g.d_leaves, g.n_leaf_boxes, rho, g.ws64.rho->p);
-    g.leaf_rho_hat(g.ws64, t->stream);
+    g.rhoh_stale = true;
     check(cudaGetLastError(), "afg_set_rhs");
     g.rhs_set = true;
     return AFG_OK;
@@ -801,6 +802,7 @@ static int one_cycle(afg_tree *t, const afg_mg_opts *opts, afg_stats *st, bool f
     const afg::MgOpts mo{o.n_down, o.n_up, o.n_base};
     g.make_compatible(t->stream);
     g.refresh_faces(t->stream);
+    g.refresh_rho_hat(t->stream);
     run(g, {fmg ? 30 : 31, o.n_down, o.n_up, o.n_base, 0}, o.use_graph, t->stream, [&](cudaStream_t cs) {
         if (fmg) g.fmg(g.ws64, mo, 0, false, cs);
         else g.vcycle(g.ws64, g.lmax, mo, 0, nullptr, cs);
@@ -941,7 +943,7 @@ int afg_forest_set_rhs(afg_forest *f, const double *rho) {
     AFG_ON_FOREST_DEVICE(f);
     Grid &g = *f->grid;
     afg::launch_leaf_set(g.leaf_cfg(true, f->stream), g.meta, g.d_leaves, g.n_leaf_boxes, rho, g.ws64.rho->p);
-    g.leaf_rho_hat(g.ws64, f->stream);
+    g.rhoh_stale = true;
     check(cudaGetLastError(), "afg_forest_set_rhs");
     g.rhs_set = true;
     return AFG_OK;
@@ -1016,6 +1018,7 @@ int time_kernel_on(Grid &g, cudaStream_t s, int kernel, int level, int fp64, int
     if (kernel < 3 && (level < g.lmin || level > g.lmax)) return fail(AFG_ERR_ARG, "level out of range");
     if ((kernel == 1 || kernel == 2) && level < 2) return fail(AFG_ERR_ARG, "level must be >= 2");
     if (!fp64 || kernel == 3) g.ensure_mixed();
+    g.refresh_rho_hat(s);
     afg::Workspace &w = fp64 ? g.ws64 : g.ws32;
     if (!fp64) {  // FP32 data from the FP64 source (values are irrelevant to timing)
         afg::launch_leaf_residual(g.leaf_cfg(true, s), g.meta, g.d_leaves, g.n_leaf_boxes, g.ws64.u->p,

@@ -171,6 +171,28 @@ AFG_HD float fx_to_float(double x) {
 #endif
 }
 
+#ifdef __CUDACC__
+__host__ __device__ __noinline__
+#endif
+    static double
+    fx_widen(float x) {
+    return (double)x;
+}
+
+// (double)x without the FP64 unit for zeros and normal numbers
+AFG_HD double fx_to_double(float x) {
+    uint32_t b;
+#ifdef __CUDA_ARCH__
+    b = __float_as_uint(x);
+#else
+    std::memcpy(&b, &x, 4);
+#endif
+    const uint32_t a = b & 0x7FFFFFFFu, e = a >> 23;
+    if (a == 0) return fx_double((uint64_t)b << 32);
+    if (e == 0 || e == 255) return fx_widen(x);
+    return fx_double((((uint64_t)a << 29) + (896ull << 52)) | ((uint64_t)(b & 0x80000000u) << 32));
+}
+
 // out = sum_k x[k] - C * c over x[0..K-1].  Returns false (out untouched)
 // when the largest exponent is outside the handled range.
 template <int K, int C = 0>

@@ -392,6 +392,12 @@ void Grid::leaf_rho_hat(Workspace &w, cudaStream_t s) {
     if (w.rhoh) launch_rho_hat(leaf_cfg(w.fp64, s), meta, d_leaves, n_leaf_boxes, w.rho->p, w.rhoh->p);
 }
 
+void Grid::refresh_rho_hat(cudaStream_t s) {
+    if (!rhoh_stale || op) return;
+    leaf_rho_hat(ws64, s);
+    rhoh_stale = false;
+}
+
 void Grid::ensure_mixed() {
     if (!ws32.u) alloc_ws(ws32, false);
 }
@@ -654,7 +660,7 @@ void Grid::fmg_low_levels(Workspace &w, const MgOpts &o, int hom, cudaStream_t s
 void Grid::make_compatible(cudaStream_t s) {
     if (!singular) return;
     launch_leaf_center(*this, ws64.rho->as<double>(), true, s);
-    leaf_rho_hat(ws64, s);
+    rhoh_stale = true;
 }
 
 void Grid::remove_mean(Workspace &w, cudaStream_t s) {

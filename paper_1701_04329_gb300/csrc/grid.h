@@ -173,12 +173,20 @@ class Grid {
     void set_eps(const double *eps_leaf, cudaStream_t s);
     std::vector<std::unique_ptr<DevBuf>> bicg;  // adjoint vectors
     bool rhs_set = false;
+    // the leaves' pre-scaled source of ws64 is older than their source (only
+    // FP64 half-sweeps read it: mixed solves never bring it up to date)
+    bool rhoh_stale = false;
+    void refresh_rho_hat(cudaStream_t s);
 
     LaunchCfg cfg(int l, bool fp64, cudaStream_t s) {
         auto &v = L(l);
         return LaunchCfg{s, D, v.M, v.MP, fp64, v.sibs};
     }
-    LaunchCfg leaf_cfg(bool fp64, cudaStream_t s) const { return LaunchCfg{s, D, N, N / 2, fp64}; }
+    LaunchCfg leaf_cfg(bool fp64, cudaStream_t s) const {
+        LaunchCfg c{s, D, N, N / 2, fp64};
+        c.one_tree = T == 1;
+        return c;
+    }
 
     void alloc_ws(Workspace &w, bool fp64);
     // refresh rho_hat of the leaves after their source term changed

@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(kThreads) k_rho_hat(BoxMeta A, const int *list
         if (idx >= n) continue;
         const int b = list[idx];
         const long long cb = A.coff[b];
-        const T c = T(-A.hb[b] * A.hb[b] / (2 * D));
+        const T c = T(-1.0 / (2 * D)) * T(A.hb[b] * A.hb[b]);  // h is a power of two: exact scaling, no FP64 division
         constexpr int VEC = 16 / (int)sizeof(T);  // a box is a whole number of 16-byte vectors
         for (int q = lt; q < Gm::C / VEC; q += Gm::G) {
             T v[VEC];

@@ -708,7 +708,9 @@ __global__ void __launch_bounds__(kThreads) k_fas_p(BoxMeta A, int b0, int n, co
 // another tree, and at the end), and optionally r cast to R in rout.
 // lap_vec(I, st, v, col, j, k, h0, out): h^2 times the operator on vector v of a box
 // whose image is not aligned; FX: weight of the aligned images' sums (0: none are).
-template <int D, int M, typename T, typename R, int GT, int FX, typename Lap>
+// ONE: all boxes belong to tree 0, so no step has to look for a change of tree
+// with the whole block.
+template <int D, int M, typename T, typename R, int GT, int FX, bool ONE, typename Lap>
 __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *list, int n, const T *u,
                                                    const T *__restrict__ rho, int hom, unsigned long long *rmax,
                                                    unsigned long long *pmax, R *rout, Lap lap_vec) {
@@ -724,6 +726,7 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
     auto want = [](const BoxInfo &) { return true; };
     auto flat = [&](const BoxInfo &) -> const T * { return rho; };
     auto pre = [&](const BoxInfo *slot) {
+        if constexpr (ONE) return;
         tr = -1;
         mixed = false;
         for (int x = 0; x < F::BPC; ++x) {
@@ -782,6 +785,7 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
         }
     };
     auto post = [&](const BoxInfo *slot) {
+        if constexpr (ONE) return;
         if (mixed) {  // boxes of several trees in this step: commit each box's maxima now
             for (int x = 0; x < F::BPC; ++x) {
                 const int t = slot[x].b >= 0 ? A.tree[slot[x].b] : -1;
@@ -792,11 +796,12 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
             cur = tr;
         }
     };
-    fp_walk<D, M, T, GT, (FX > 0), (FX > 0), FX, true>(A, 0, n, list, u, hom, want, flat, body, pre, post);
-    flush_max(rm, pm, cur, cur >= 0, rmax, pmax, red);
+    fp_walk<D, M, T, GT, (FX > 0), (FX > 0), FX, !ONE>(A, 0, n, list, u, hom, want, flat, body, pre, post);
+    if constexpr (ONE) flush_max(rm, pm, 0, true, rmax, pmax, red);
+    else flush_max(rm, pm, cur, cur >= 0, rmax, pmax, red);
 }
 
-template <int D, int M, typename T, typename R>
+template <int D, int M, typename T, typename R, bool ONE>
 __global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>()) k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
                                                               const T *__restrict__ rho, int hom,
                                                               unsigned long long *rmax, unsigned long long *pmax,
@@ -806,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>()) k_leaf_re
     auto lap = [](const BoxInfo &, const T *st, int, int col, int j, int k, int h0, T *out) {
         fp_lap_vec<D, M, T>(st, col, j, k, h0, out);
     };
-    leaf_residual_walk<D, M, T, R, GT, FX>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
+    leaf_residual_walk<D, M, T, R, GT, FX, ONE>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
 }
 
 // The transposed operator on leaf boxes whose sides all face same-level leaves

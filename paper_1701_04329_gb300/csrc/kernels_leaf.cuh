@@ -81,7 +81,15 @@ __global__ void __launch_bounds__(kThreads) k_mixed_update(BoxMeta A, const int 
         const int b = resolve_box<D, M>(A, base + g, n, 0, list);
         if (b < 0) continue;
         const long long cb = A.coff[b];
-        for (int q = lt; q < Gm::C; q += Gm::G) x[cb + q] += double(e[cb + q]);
+        for (int q = 2 * lt; q < Gm::C; q += 2 * Gm::G) {
+            double v[2];
+            float f[2];
+            ldv<double, 2>(x + cb + q, v);
+            ldv<float, 2>(e + cb + q, f);
+            v[0] += fx_to_double(f[0]);
+            v[1] += fx_to_double(f[1]);
+            stv<double, 2>(x + cb + q, v);
+        }
     }
 }
 

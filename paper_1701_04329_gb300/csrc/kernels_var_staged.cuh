@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kThreads) k_var_fas_p(BoxMeta A, int b0, int n
 }
 
 // Composite residual on the leaves with its norms per tree, and r in rout.
-template <int D, int M, typename T, typename R>
+template <int D, int M, typename T, typename R, bool ONE>
 __global__ void __launch_bounds__(kThreads) k_var_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
                                                                   const T *__restrict__ rho, VarCoef<T> V, int hom,
                                                                   unsigned long long *rmax, unsigned long long *pmax,
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kThreads) k_var_leaf_residual_p(BoxMeta A, con
         T self[VEC];
         fp_var_lap_vec<D, M, T>(st, V.c + I.coff + v * VEC, V.n, col, j, k, h0, out, self);
     };
-    leaf_residual_walk<D, M, T, R, GT, 0>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
+    leaf_residual_walk<D, M, T, R, GT, 0, ONE>(A, list, n, u, rho, hom, rmax, pmax, rout, lap);
 }
 
 }  // namespace afg

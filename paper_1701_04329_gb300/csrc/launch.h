@@ -21,6 +21,8 @@ struct LaunchCfg {
     // FP32 half-sweep: 16-byte vectors per thread (1: one thread per vector of
     // a box's colour half; 2: half the threads per box)
     int vpt = 1;
+    // leaf residual: all boxes belong to one tree
+    bool one_tree = false;
 };
 
 // counts launches of this library's kernels (host side)

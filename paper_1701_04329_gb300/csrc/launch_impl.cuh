@@ -186,8 +186,10 @@ void do_leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list, int
     if constexpr (FpCfg<D, M, T>::ok) {
         using F32 = FpCfg<D, M, T, leaf_threads<D, M, T, float>()>;
         using F64 = FpCfg<D, M, T, leaf_threads<D, M, T, double>()>;
-        if (rout_f32) go(k_leaf_residual_p<D, M, T, float>, F32::smem(), (n + F32::BPC - 1) / F32::BPC, (float *)rout);
-        else go(k_leaf_residual_p<D, M, T, double>, F64::smem(), (n + F64::BPC - 1) / F64::BPC, (double *)rout);
+        auto k32 = c.one_tree ? k_leaf_residual_p<D, M, T, float, true> : k_leaf_residual_p<D, M, T, float, false>;
+        auto k64 = c.one_tree ? k_leaf_residual_p<D, M, T, double, true> : k_leaf_residual_p<D, M, T, double, false>;
+        if (rout_f32) go(k32, F32::smem(), (n + F32::BPC - 1) / F32::BPC, (float *)rout);
+        else go(k64, F64::smem(), (n + F64::BPC - 1) / F64::BPC, (double *)rout);
     } else {
         const size_t smem = FullCfg<D, M, T>::smem();
         if (rout_f32) go(k_leaf_residual<D, M, T, float>, smem, work_ctas<D, M>(n), (float *)rout);

@@ -96,7 +96,7 @@ void do_var_leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list,
     if (n <= 0) return;
     static_assert(FpCfg<D, M, T>::ok, "leaf boxes have 4 cells per side or more, in FP64");
     using F = FpCfg<D, M, T, leaf_threads<D, M, T, Ro>()>;
-    auto k = k_var_leaf_residual_p<D, M, T, Ro>;
+    auto k = c.one_tree ? k_var_leaf_residual_p<D, M, T, Ro, true> : k_var_leaf_residual_p<D, M, T, Ro, false>;
     const VarCoef<T> V{(const T *)W.coef, W.n};
     launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, (const T *)u,
                (const T *)rho, V, hom, rmax, pmax, (Ro *)rout);

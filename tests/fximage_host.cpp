@@ -20,6 +20,15 @@ int main(int argc, char **argv) {
         }
         return 0;
     }
+    if (argc > 1 && argv[1][0] == 'd') {
+        uint32_t f;
+        while (std::scanf("%" SCNx32, &f) == 1) {
+            float x;
+            std::memcpy(&x, &f, 4);
+            std::printf("%016" PRIx64 "\n", fx_bits(fx_to_double(x)));
+        }
+        return 0;
+    }
     int E;
     while (std::scanf("%d", &E) == 1) {
         for (int i = 0; i < 7; ++i)

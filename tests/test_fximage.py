@@ -65,3 +65,12 @@ def test_to_float(exe):
     with np.errstate(all="ignore"):
         want = x.astype(np.float32).view(np.uint32)
     assert [int(o, 16) for o in out] == [int(w) for w in want]
+
+
+def test_to_double(exe):
+    rng = np.random.default_rng(8)
+    x = rng.integers(0, 2 ** 32, 4000, dtype=np.uint32).view(np.float32)
+    x = np.concatenate([x[~np.isnan(x)], np.array([0.0, -0.0, 1e-45, 1.17549435e-38, np.inf, -np.inf], np.float32)])
+    inp = "\n".join("%08x" % v for v in x.view(np.uint32))
+    out = subprocess.run([exe, "d"], input=inp, capture_output=True, text=True, check=True).stdout.split()
+    assert [int(o, 16) for o in out] == [int(w) for w in x.astype(np.float64).view(np.uint64)]
