@@ -297,6 +297,24 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     for (int b = 0; b < nbox; ++b) ih2[b] = 1.0 / (hb[b] * hb[b]);
     meta.ih2 = upload(ih2, own);
     meta.active = nullptr;
+    {
+        std::vector<BoxInfo> info(nbox);
+        for (int b = 0; b < nbox; ++b) {
+            BoxInfo &I = info[b];
+            std::memset(&I, 0, sizeof I);
+            I.coff = coff[b];
+            for (int s = 0; s < S; ++s) {
+                I.base[s] = nbase[b * S + s];
+                I.code[s] = nb[b * S + s];
+            }
+            I.b = b;
+            I.flag = bflag[b] | (cfmask[b] << 8);
+            I.poff = poff[b];
+            I.parent = parent[b];
+            I.nmask = (I.flag >> BF_NSHIFT) & 0x3f;
+        }
+        meta.info = upload(info, own);
+    }
     d_child = upload(child, own);
     d_leaves = upload(leaves, own);
     d_leaf_geo = upload(leaf_geo, own);

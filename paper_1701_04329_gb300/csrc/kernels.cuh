@@ -62,7 +62,10 @@ constexpr int BF_NSHIFT = 2;  // flag bits 2..7: Neumann domain sides (bit 2 + s
 // BoxInfo::flag bits 8..13 (not in the per-box byte): refinement-boundary sides (bit 8 + s)
 constexpr int BF_CF = 0x3f00;
 
+struct BoxInfo;
+
 struct BoxMeta {
+    const BoxInfo *info;  // every box's BoxInfo, ready to copy (the staged kernels)
     const int *nb;
     const int *parent;
     const int *poff;
@@ -81,7 +84,7 @@ struct BoxMeta {
 };
 
 // Metadata of one box, prefetched into shared memory one box ahead.
-struct BoxInfo {
+struct alignas(16) BoxInfo {
     long long coff;
     long long base[6];
     int code[6];
@@ -89,6 +92,8 @@ struct BoxInfo {
     long long pcoff;  // cells of the parent (k_correct)
     int nmask;        // Neumann domain sides (of the parent in k_correct)
 };
+
+static_assert(sizeof(BoxInfo) % 16 == 0, "copied as 16-byte pieces");
 
 // The activity mask is written by kernels: after pdl_wait, drop a prefetched
 // box whose tree is masked out.

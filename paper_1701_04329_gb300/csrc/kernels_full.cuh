@@ -430,9 +430,14 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
     const int first = blockIdx.x * F::BPC;
     __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
-        info_load<D>(A, first + q * stride + g, n, b0, list, info[q * F::BPC + g], lt, F::G, false);
+        info_stage<D>(A, first + q * stride + g, n, b0, list, info[q * F::BPC + g], lt, F::G);
+    cp_commit();
     pdl_wait();
-    for (int q = 0; q < NST; ++q) info_mask<D>(A, info[q * F::BPC + g], lt, F::G);
+    cp_wait<0>();
+    if (A.active) {
+        __syncthreads();
+        for (int q = 0; q < NST; ++q) info_mask<D>(A, info[q * F::BPC + g], lt, F::G);
+    }
     __syncthreads();
     FpPlan<D, M, T, GT> pl;
     if constexpr (PLAN) pl.init(lt);
@@ -443,9 +448,11 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
             if constexpr (PLAN) fp_issue_plan<D, M, T, GT>(pl, In, u, flat(In), dst, lt, want(In));
             else fp_issue<D, M, T, GT>(In, u, flat(In), dst, lt, want(In));
         }
-        cp_commit();
     };
-    for (int q = 0; q < NST - 1; ++q) issue(q);
+    for (int q = 0; q < NST - 1; ++q) {
+        issue(q);
+        cp_commit();
+    }
     int it = 0;
     for (int base = first; base < n; base += stride, ++it) {
         cp_wait<NST - 2>();
@@ -463,7 +470,10 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
         }
         const int any_cf = box_sync<BLOCK ? 1 : GT>(g, cf);  // previous stage and metadata slot are free now
         issue(it + NST - 1);
-        info_load<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * F::BPC + g], lt, F::G);
+        BoxInfo &Nx = info[((it + NST) % NI) * F::BPC + g];
+        if (!A.active) info_stage<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, F::G);
+        else info_load<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, F::G);  // masked trees drop out
+        cp_commit();
         pre(&info[(it % NI) * F::BPC]);
         if (any_cf) {  // refinement-boundary ghosts read cells other threads staged
             if (cf) {

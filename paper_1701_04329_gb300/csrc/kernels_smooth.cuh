@@ -49,6 +49,23 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// Metadata of entry `idx` of a level range or list into slot I, asynchronously:
+// the box's BoxInfo in 16-byte pieces.  (Thirteen loads whose results a thread
+// then stored made the first warp of every box's group wait for L2 ahead of
+// the box's arithmetic.)  Done after the thread's next cp_wait and a barrier.
+template <int D>
+__device__ __forceinline__ void info_stage(const BoxMeta &A, int idx, int n, int b0, const int *list, BoxInfo &I,
+                                           int lt, int G) {
+    constexpr int NP = (int)sizeof(BoxInfo) / 16;
+    if (idx >= n) {
+        if (lt == 0) I.b = -1;
+        return;
+    }
+    if (lt >= NP) return;
+    const char *src = reinterpret_cast<const char *>(A.info + (list ? list[idx] : b0 + idx));
+    for (int x = lt; x < NP; x += G) cp_async<16>(reinterpret_cast<char *>(&I) + 16 * x, src + 16 * x);
+}
+
 // VPT: 16-byte vectors of a box's colour half per thread (1: one thread per
 // vector; 2: half as many threads per box, twice the boxes per CTA)
 template <int D, int M, typename T, int VPT = 1>
@@ -450,9 +467,14 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
     pdl_trigger();
     __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
-        info_load<D>(A, first + q * stride + g, n, b0, list, info[q * S::BPC + g], lt, S::G, false);
+        info_stage<D>(A, first + q * stride + g, n, b0, list, info[q * S::BPC + g], lt, S::G);
+    cp_commit();
     pdl_wait();
-    for (int q = 0; q < NST; ++q) info_mask<D>(A, info[q * S::BPC + g], lt, S::G);
+    cp_wait<0>();
+    if (A.active) {
+        __syncthreads();
+        for (int q = 0; q < NST; ++q) info_mask<D>(A, info[q * S::BPC + g], lt, S::G);
+    }
     __syncthreads();
     for (int q = 0; q < NST - 1; ++q) {
         const BoxInfo &In = info[q * S::BPC + g];
@@ -482,9 +504,11 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
             const int q = it + NST - 1;
             const BoxInfo &In = info[(q % NI) * S::BPC + g];
             if (In.b >= 0) sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + ((q % NST) * S::BPC + g) * S::BOX, lt, c);
+            BoxInfo &Nx = info[((it + NST) % NI) * S::BPC + g];
+            if (!A.active) info_stage<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, S::G);
+            else info_load<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, S::G);  // masked trees drop out
             cp_commit();
         }
-        info_load<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * S::BPC + g], lt, S::G);
         if (any_cf) {  // refinement-boundary ghosts read cells other threads staged
             if (cf) {
                 sp_fix<D, M, T, VPT>(I, A, u, box, lt, c, hom, true);
