@@ -312,6 +312,7 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
             I.poff = poff[b];
             I.parent = parent[b];
             I.nmask = (I.flag >> BF_NSHIFT) & 0x3f;
+            I.tree = tree[b];
         }
         meta.info = upload(info, own);
     }

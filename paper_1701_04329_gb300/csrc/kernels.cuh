@@ -91,6 +91,7 @@ struct alignas(16) BoxInfo {
     int b, flag, poff, parent;
     long long pcoff;  // cells of the parent (k_correct)
     int nmask;        // Neumann domain sides (of the parent in k_correct)
+    int tree;         // set in BoxMeta::info only
 };
 
 static_assert(sizeof(BoxInfo) % 16 == 0, "copied as 16-byte pieces");

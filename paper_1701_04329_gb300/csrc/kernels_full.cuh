@@ -434,17 +434,13 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
     cp_commit();
     pdl_wait();
     cp_wait<0>();
-    if (A.active) {
-        __syncthreads();
-        for (int q = 0; q < NST; ++q) info_mask<D>(A, info[q * F::BPC + g], lt, F::G);
-    }
     __syncthreads();
     FpPlan<D, M, T, GT> pl;
     if constexpr (PLAN) pl.init(lt);
     auto issue = [&](int q) {
         const BoxInfo &In = info[(q % NI) * F::BPC + g];
         T *dst = stages + ((q % NST) * F::BPC + g) * F::BOX;
-        if (In.b >= 0) {
+        if (info_on(A, In)) {
             if constexpr (PLAN) fp_issue_plan<D, M, T, GT>(pl, In, u, flat(In), dst, lt, want(In));
             else fp_issue<D, M, T, GT>(In, u, flat(In), dst, lt, want(In));
         }
@@ -457,7 +453,8 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
     for (int base = first; base < n; base += stride, ++it) {
         cp_wait<NST - 2>();
         const BoxInfo &I = info[(it % NI) * F::BPC + g];
-        const bool special = I.b >= 0 && want(I) && (I.flag & BF_SPECIAL);
+        const bool on = info_on(A, I);
+        const bool special = on && want(I) && (I.flag & BF_SPECIAL);
         const bool cf = special && (!OWN || (I.flag & BF_CF));
         T *st = stages + ((it % NST) * F::BPC + g) * F::BOX;
         if (OWN && special) {  // domain sides: this thread's own items
@@ -466,13 +463,11 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
         }
         if constexpr (FX > 0) {
             static_assert(OWN && PLAN, "aligned images need the plan");
-            if (I.b >= 0 && want(I)) fx_fold_own(pl, st, fxr);
+            if (on && want(I)) fx_fold_own(pl, st, fxr);
         }
         const int any_cf = box_sync<BLOCK ? 1 : GT>(g, cf);  // previous stage and metadata slot are free now
         issue(it + NST - 1);
-        BoxInfo &Nx = info[((it + NST) % NI) * F::BPC + g];
-        if (!A.active) info_stage<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, F::G);
-        else info_load<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, F::G);  // masked trees drop out
+        info_stage<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * F::BPC + g], lt, F::G);
         cp_commit();
         pre(&info[(it % NI) * F::BPC]);
         if (any_cf) {  // refinement-boundary ghosts read cells other threads staged
@@ -482,7 +477,7 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
             }
             box_sync<BLOCK ? 1 : GT>(g, false);
         }
-        if (I.b >= 0) {
+        if (on) {
             int E = -1;
             if constexpr (FX > 0) {
                 if (want(I)) {

@@ -66,6 +66,12 @@ __device__ __forceinline__ void info_stage(const BoxMeta &A, int idx, int n, int
     for (int x = lt; x < NP; x += G) cp_async<16>(reinterpret_cast<char *>(&I) + 16 * x, src + 16 * x);
 }
 
+// whether a staged slot holds a box of a tree that takes part (the mask stays in
+// L1; the walks ask where they stage a box and where they compute it)
+__device__ __forceinline__ bool info_on(const BoxMeta &A, const BoxInfo &I) {
+    return I.b >= 0 && (!A.active || A.active[I.tree]);
+}
+
 // VPT: 16-byte vectors of a box's colour half per thread (1: one thread per
 // vector; 2: half as many threads per box, twice the boxes per CTA)
 template <int D, int M, typename T, int VPT = 1>
@@ -471,20 +477,16 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
     cp_commit();
     pdl_wait();
     cp_wait<0>();
-    if (A.active) {
-        __syncthreads();
-        for (int q = 0; q < NST; ++q) info_mask<D>(A, info[q * S::BPC + g], lt, S::G);
-    }
     __syncthreads();
     for (int q = 0; q < NST - 1; ++q) {
         const BoxInfo &In = info[q * S::BPC + g];
-        if (In.b >= 0) sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + (q * S::BPC + g) * S::BOX, lt, c);
+        if (info_on(A, In)) sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + (q * S::BPC + g) * S::BOX, lt, c);
         cp_commit();
     }
     int it = 0;
     for (int base = first; base < n; base += stride, ++it) {
         const BoxInfo &I = info[(it % NI) * S::BPC + g];
-        const int b = I.b;
+        const int b = info_on(A, I) ? I.b : -1;
         if (b >= 0) {
 #pragma unroll
             for (int itv = 0; itv < S::NIT; ++itv)
@@ -503,10 +505,8 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
         {
             const int q = it + NST - 1;
             const BoxInfo &In = info[(q % NI) * S::BPC + g];
-            if (In.b >= 0) sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + ((q % NST) * S::BPC + g) * S::BOX, lt, c);
-            BoxInfo &Nx = info[((it + NST) % NI) * S::BPC + g];
-            if (!A.active) info_stage<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, S::G);
-            else info_load<D>(A, base + NST * stride + g, n, b0, list, Nx, lt, S::G);  // masked trees drop out
+            if (info_on(A, In)) sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + ((q % NST) * S::BPC + g) * S::BOX, lt, c);
+            info_stage<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * S::BPC + g], lt, S::G);
             cp_commit();
         }
         if (any_cf) {  // refinement-boundary ghosts read cells other threads staged
