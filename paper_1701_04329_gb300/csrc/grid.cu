@@ -407,13 +407,9 @@ void Grid::alloc_ws(Workspace &w, bool fp64) {
     }
 }
 
-void Grid::leaf_rho_hat(Workspace &w, cudaStream_t s) {
-    if (w.rhoh) launch_rho_hat(leaf_cfg(w.fp64, s), meta, d_leaves, n_leaf_boxes, w.rho->p, w.rhoh->p);
-}
-
 void Grid::refresh_rho_hat(cudaStream_t s) {
     if (!rhoh_stale || op) return;
-    leaf_rho_hat(ws64, s);
+    launch_rho_hat(leaf_cfg(true, s), meta, d_leaves, n_leaf_boxes, ws64.rho->p, ws64.rhoh->p);
     rhoh_stale = false;
 }
 

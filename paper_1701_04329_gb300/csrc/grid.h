@@ -82,7 +82,7 @@ class Grid {
     int device = 0;  // the CUDA device holding this grid's data
 
     struct Level {
-        int l, M, MP, b0, nb;  // MP = parent box size (0 at the bottom)
+        int l, M, MP, b0, nb;  // MP = parent box size (0 on the coarsest level)
         double h;
         int *d_leaves = nullptr;
         int nleaves = 0;
@@ -189,8 +189,6 @@ class Grid {
     }
 
     void alloc_ws(Workspace &w, bool fp64);
-    // refresh rho_hat of the leaves after their source term changed
-    void leaf_rho_hat(Workspace &w, cudaStream_t s);
     void ensure_mixed();
     void ensure_adjoint();
 

@@ -519,7 +519,7 @@ constexpr bool fx_leaf() { return sizeof(T) == 8 && (D == 3 || sizeof(R) == 4); 
 // an SM: 128 in 3D (aligned images; four blocks of 64 registers), 64 in 2D (two
 // blocks).  256^3 of 8^3 boxes: 0.165 ms with 128 threads and four blocks, 0.174
 // with three, 0.182 with 64 threads and two, 0.231 with 256 and three (per-cell
-// alignment, 64 threads and two: 0.280).  2D, 4.2 M cells, 8^2 / 16^2 boxes: four
+// alignment, 64 threads and two: 0.280); 0.138 ms now (ONE, info_stage).  2D, 4.2 M cells, 8^2 / 16^2 boxes: four
 // blocks 56 / 39 us, three 71 / 41, no bound 97 / 54 (before 82 / 57).
 template <int D, int M, typename T, typename R>
 constexpr int leaf_threads() {
@@ -546,7 +546,7 @@ constexpr int fx_restrict_weight() { return 2 * D * (1 << D); }
 // left three quarters of an FP64 box's threads idle and made 43 FP64 additions,
 // 64 cycles each, in a chain).  Left in FP64: the sum of the children's source
 // and one FMA.  The two roundings run side by side, in two threads of the four.
-// 256^3: 0.213 -> 0.165 ms.
+// 256^3: 0.213 -> 0.165 ms, 0.148 ms with info_stage.
 template <int D, int M, int MP, int GT>
 __device__ __forceinline__ void rr_aligned(const BoxMeta &A, const BoxInfo &I, const double *st, int lt, int E,
                                            double ih2, long long cp, double *u, double *rho, double *vold) {
@@ -1110,15 +1110,23 @@ __global__ void __launch_bounds__(kThreads) k_correct_p(BoxMeta A, int b0, int n
 // cell, and updates all children's cells with the 2-1-1 / 1-1-1-1 scheme
 // (the same arithmetic as k_correct_p).  Parents are staged one ahead
 // (two-stage ring).
+//
+// A parent takes one thread per vector of its children, a warp to a whole block;
+// small parents share a block (2D, 8^2 boxes: 64 threads and four parents, where
+// a block per parent left three quarters of its threads idle: 4.2 M cells, FP32,
+// 32.6 -> 15.3 us, FP64 40 -> 34 us).
 template <int D, int M, typename T>
 struct PpCfg {
-    using F = FpCfg<D, M, T, kThreads>;
-    static constexpr int NC = 1 << D, C = Geo<D, M>::C, VEC = F::VEC, NV = C / VEC;
+    static constexpr int NC = 1 << D, C = Geo<D, M>::C, VEC = 16 / (int)sizeof(T), NV = C / VEC;
+    static constexpr int G = NC * NV < 32 ? 32 : (NC * NV > kThreads ? kThreads : NC * NV);
+    static constexpr int BPC = kThreads / G;
+    using F = FpCfg<D, M, T, G>;
     static constexpr int IMG = F::UB;                  // one image (u or v') with its ghosts
     static constexpr int PSZ = D == 3 ? 6 * C : 0;     // pair sums of the parent's cells
     static constexpr int NST = 2;
+    static constexpr int PARENT = 2 * IMG * NST + PSZ;
     static constexpr size_t smem() {
-        return sizeof(T) * (2 * IMG * NST + PSZ) + sizeof(BoxInfo) * (NST + 1) + sizeof(long long) * NC * (NST + 1);
+        return BPC * (sizeof(T) * PARENT + sizeof(BoxInfo) * (NST + 1) + sizeof(long long) * NC * (NST + 1));
     }
     // a vector stays inside one half-row, and at least two CTAs fit an SM
     // (3D boxes of 16^3 cells take the per-child kernel)
@@ -1131,7 +1139,7 @@ template <int D, int M, typename T>
 __device__ __forceinline__ void pp_info_load(const BoxMeta &A, int q, int np, int b0, BoxInfo &I, long long *ccoff,
                                              bool mask) {
     using S = PpCfg<D, M, T>;
-    const int lt = threadIdx.x;
+    const int lt = threadIdx.x % S::G;
     const int b = q < np ? A.parent[b0 + S::NC * q] : -1;
     bool on = b >= 0;
     if (on && mask && A.active && !A.active[A.tree[b]]) on = false;
@@ -1147,8 +1155,8 @@ __device__ __forceinline__ void pp_info_load(const BoxMeta &A, int q, int np, in
             I.flag = A.bflag[b];
             I.nmask = (I.flag >> BF_NSHIFT) & 0x3f;
         }
-    } else if (lt >= 32 && lt < 32 + S::NC) {
-        if (on) ccoff[lt - 32] = A.coff[b0 + S::NC * q + (lt - 32)];
+    } else if (lt >= 8 && lt < 8 + S::NC) {
+        if (on) ccoff[lt - 8] = A.coff[b0 + S::NC * q + (lt - 8)];
     }
 }
 
@@ -1158,48 +1166,49 @@ __global__ void __launch_bounds__(kThreads) k_correct_pp(BoxMeta A, int b0, int 
     using F = typename S::F;
     constexpr int NST = S::NST, NI = NST + 1, MH = M / 2, VEC = S::VEC, NVH = Geo<D, M>::H / VEC, NVR = F::NVR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *stages = reinterpret_cast<T *>(smem_raw);
+    const int g = threadIdx.x / S::G, lt = threadIdx.x % S::G;
+    T *stages = reinterpret_cast<T *>(smem_raw) + g * S::PARENT;
     T *PS = stages + 2 * S::IMG * NST;
-    BoxInfo *info = reinterpret_cast<BoxInfo *>(smem_raw + sizeof(T) * (2 * S::IMG * NST + S::PSZ));
-    long long *ccoff = reinterpret_cast<long long *>(info + NI);
-    const int lt = threadIdx.x;
-    const int np = n / S::NC;
+    BoxInfo *info = reinterpret_cast<BoxInfo *>(smem_raw + sizeof(T) * S::PARENT * S::BPC) + g * NI;
+    long long *ccoff = reinterpret_cast<long long *>(smem_raw + (sizeof(T) * S::PARENT + sizeof(BoxInfo) * NI) * S::BPC) +
+                       g * S::NC * NI;
+    const int np = n / S::NC, stride = gridDim.x * S::BPC, first = blockIdx.x * S::BPC + g;
     pdl_trigger();
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
-        pp_info_load<D, M, T>(A, blockIdx.x + q * gridDim.x, np, b0, info[q], ccoff + q * S::NC, false);
+        pp_info_load<D, M, T>(A, first + q * stride, np, b0, info[q], ccoff + q * S::NC, false);
     pdl_wait();
-    __syncthreads();
+    group_sync<S::G>(g);
     if (lt == 2 * D)
         for (int q = 0; q < NST; ++q)
             if (info[q].b >= 0 && A.active && !A.active[A.tree[info[q].b]]) info[q].b = -1;
-    __syncthreads();
+    group_sync<S::G>(g);
     auto issue = [&](int q) {
         const BoxInfo &In = info[q % NI];
         if (In.b >= 0) {
             T *st = stages + (q % NST) * 2 * S::IMG;
-            fp_issue<D, M, T, kThreads>(In, u, nullptr, st, lt, true);
-            fp_issue<D, M, T, kThreads>(In, vold, nullptr, st + S::IMG, lt, true);
+            fp_issue<D, M, T, S::G>(In, u, nullptr, st, lt, true);
+            fp_issue<D, M, T, S::G>(In, vold, nullptr, st + S::IMG, lt, true);
         }
         cp_commit();
     };
     for (int q = 0; q < NST - 1; ++q) issue(q);
     int it = 0;
-    for (int base = blockIdx.x; base < np; base += gridDim.x, ++it) {
+    for (int base = first; base < np; base += stride, ++it) {
         cp_wait<NST - 2>();
-        __syncthreads();  // the parent's images have landed; the previous stage and slots are free
+        group_sync<S::G>(g);  // the parent's images have landed; the previous stage and slots are free
         const BoxInfo &I = info[it % NI];
         const long long *cc = ccoff + (it % NI) * S::NC;
         T *Dd = stages + (it % NST) * 2 * S::IMG;
         const T *V = Dd + S::IMG;
         issue(it + NST - 1);
-        pp_info_load<D, M, T>(A, base + NST * gridDim.x, np, b0, info[(it + NST) % NI], ccoff + ((it + NST) % NI) * S::NC,
+        pp_info_load<D, M, T>(A, base + NST * stride, np, b0, info[(it + NST) % NI], ccoff + ((it + NST) % NI) * S::NC,
                               true);
         const bool on = I.b >= 0;
         if (on)
-            for (int e = lt; e < S::IMG; e += kThreads) Dd[e] = Dd[e] - V[e];
+            for (int e = lt; e < S::IMG; e += S::G) Dd[e] = Dd[e] - V[e];
         if (on && (I.flag & BF_SPECIAL)) {  // a Dirichlet side: the difference enters as -d
-            __syncthreads();
-            for (int item = lt; item < F::NGI; item += kThreads) {
+            group_sync<S::G>(g);
+            for (int item = lt; item < F::NGI; item += S::G) {
                 int sd, slot;
                 if (item < F::NXI) {
                     int j, k;
@@ -1216,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads) k_correct_pp(BoxMeta A, int b0, int 
                 }
             }
         }
-        __syncthreads();
+        group_sync<S::G>(g);
         // d of parent cell (i, j, k), i in [-1, M]: the planes, or the x ghosts
         auto dat = [&](int i, int j, int k) -> T {
             if (i < 0) return Dd[2 * F::PT + sp_row<D, M>(j, k)];
@@ -1225,7 +1234,7 @@ __global__ void __launch_bounds__(kThreads) k_correct_pp(BoxMeta A, int b0, int 
         };
         if constexpr (D == 3) {
             if (on)
-                for (int c = lt; c < S::C; c += kThreads) {
+                for (int c = lt; c < S::C; c += S::G) {
                     const int X = c % M, Y = (c / M) % M, Z = c / (M * M);
                     const T d0 = dat(X, Y, Z), dym = dat(X, Y - 1, Z), dyp = dat(X, Y + 1, Z);
                     const T dzm = dat(X, Y, Z - 1), dzp = dat(X, Y, Z + 1);
@@ -1236,10 +1245,10 @@ __global__ void __launch_bounds__(kThreads) k_correct_pp(BoxMeta A, int b0, int 
                     PS[4 * S::C + c] = dyp + dzm;
                     PS[5 * S::C + c] = dyp + dzp;
                 }
-            __syncthreads();
+            group_sync<S::G>(g);
         }
         if (on) {
-            for (int t = lt; t < S::NC * S::NV; t += kThreads) {
+            for (int t = lt; t < S::NC * S::NV; t += S::G) {
                 const int ch = t / S::NV, v = t % S::NV;
                 // the child's offset in the parent: bit a of ch is its half along axis a
                 const int px = (ch & 1) * MH, py = ((ch >> 1) & 1) * MH, pz = D == 3 ? ((ch >> 2) & 1) * MH : 0;

@@ -16,9 +16,6 @@
 
 namespace afg {
 
-// FP64 half-sweeps: the staged half-row kernel (true) or the table-driven one
-constexpr bool kStagedSmooth64 = true;
-
 int sm_count();
 // resident CTAs per SM of a kernel for a given dynamic shared memory size (cached)
 int occupancy(const void *kernel, size_t smem);
@@ -60,9 +57,8 @@ template <int D, int M, typename T>
 void do_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *u, const void *rho,
                const void *rhoh, double h2, int colour, int hom) {
     if (n <= 0) return;
-    // FP32: the staged half-row kernel; FP64 keeps the table-driven one unless
-    // kStagedSmooth64 is set
-    if constexpr (SpCfg<D, M, T>::ok && (sizeof(T) == 4 || kStagedSmooth64)) {
+    // the staged half-row kernel wherever a half-row holds a 16-byte vector
+    if constexpr (SpCfg<D, M, T>::ok) {
         // FP32 with half the threads per box (two vectors per thread) on request
         if constexpr (sizeof(T) == 4 && SpCfg<D, M, T>::NV >= 2) {
             if (c.vpt == 2) {
@@ -145,7 +141,8 @@ void do_correct(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, co
             using S = PpCfg<D, M, T>;
             const size_t smem = S::smem();
             auto k = k_correct_pp<D, M, T>;
-            launch_pdl(k, grid_for(k, smem, n / S::NC), smem, c.stream, A, b0, n, (T *)u, (const T *)vold);
+            launch_pdl(k, grid_for(k, smem, (n / S::NC + S::BPC - 1) / S::BPC), smem, c.stream, A, b0, n, (T *)u,
+                       (const T *)vold);
             ++g_launches;
             return;
         }
