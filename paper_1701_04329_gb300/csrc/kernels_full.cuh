@@ -494,10 +494,18 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
 }
 
 // threads per box of the restriction: one per coarse cell, at least a warp
-// (FP32); FP64 boxes take the whole block (their stages are twice as large)
+// (FP32); FP64 boxes take half their cells (their stages are twice as large).
+// On levels of many 2D boxes of 8^2 cells (`many`) two boxes share a warp: 16
+// coarse cells leave half of each warp idle, and a warp's FP64 instruction
+// costs the same (4.2 M cells, FP64 84.8 -> 48.2 us, FP32 17.2 -> 11.9 us; 128
+// quadtrees, mixed, 13.6 -> 13.1 ms).  Where a block per SM holds the level at a
+// warp per box, staging by half the threads only lengthens the launch (31 k
+// unknowns, FP64, 2.13 -> 2.15 ms with it).  16^2 boxes, FP64: 128 threads 44.0
+// us, 64 threads 45.5.
 template <int D, int M, typename T>
-constexpr int rr_threads() {
+constexpr int rr_threads(bool many) {
     constexpr int NCO = D == 2 ? (M / 2) * (M / 2) : (M / 2) * (M / 2) * (M / 2);
+    if (NCO == 16 && many) return NCO;
     return sizeof(T) == 8 ? Geo<D, M>::G : (NCO < 32 ? 32 : (NCO > kThreads ? kThreads : NCO));
 }
 
@@ -649,10 +657,10 @@ __device__ __forceinline__ void rr_rows(const BoxInfo &I, const float *st, int l
 
 // Fused residual + restriction, staged version of k_resid_restrict (the same
 // sums, in its order in FP64 where the image is not aligned).
-template <int D, int M, int MP, typename T>
+template <int D, int M, int MP, typename T, bool MANY>
 __global__ void __launch_bounds__(kThreads) k_resid_restrict_p(BoxMeta A, int b0, int n, T *u, T *rho, T *vold,
                                                                T ih2, int hom) {
-    constexpr int GT = rr_threads<D, M, T>();
+    constexpr int GT = rr_threads<D, M, T>(MANY);
     using F = FpCfg<D, M, T, GT>;
     constexpr int MH = M / 2;
     constexpr int NCO = D == 2 ? MH * MH : MH * MH * MH;

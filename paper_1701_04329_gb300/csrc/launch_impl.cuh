@@ -98,11 +98,20 @@ void do_resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void
                        double ih2, int hom) {
     if (n <= 0) return;
     if constexpr (FpCfg<D, M, T>::ok) {
-        using F = FpCfg<D, M, T, rr_threads<D, M, T>()>;
-        const size_t smem = F::smem();
-        auto k = k_resid_restrict_p<D, M, MP, T>;
-        launch_pdl(k, grid_for(k, smem, (n + F::BPC - 1) / F::BPC), smem, c.stream, A, b0, n, (T *)u, (T *)rho,
-                   (T *)vold, T(ih2), hom);
+        auto go = [&](auto many) {
+            constexpr bool MANY = decltype(many)::value;
+            using F = FpCfg<D, M, T, rr_threads<D, M, T>(MANY)>;
+            const size_t smem = F::smem();
+            auto k = k_resid_restrict_p<D, M, MP, T, MANY>;
+            launch_pdl(k, grid_for(k, smem, (n + F::BPC - 1) / F::BPC), smem, c.stream, A, b0, n, (T *)u, (T *)rho,
+                       (T *)vold, T(ih2), hom);
+        };
+        if constexpr (rr_threads<D, M, T>(true) != rr_threads<D, M, T>(false)) {
+            if (n > kThreads / 32 * sm_count()) go(std::true_type{});
+            else go(std::false_type{});
+        } else {
+            go(std::false_type{});
+        }
     } else {
         const size_t smem = FullCfg<D, M, T>::smem();
         auto k = k_resid_restrict<D, M, MP, T>;

@@ -45,3 +45,17 @@ def test_parents_per_block(N, parents):
     st = b.solve(afgpu.default_opts(rel_tol=1e-10, precision=afgpu.AFG_MIXED))
     assert st["rel_residual"] <= 1e-10
     assert rel_diff(b.get_solution(), a.get_solution()) <= 1e-8
+
+
+@pytest.mark.parametrize("parents", [304, 305, 307, 330])
+def test_levels_of_many_boxes(parents):
+    """Levels of 1216 boxes (a warp per box in the restriction) and just above
+    (two boxes per warp), also in numbers that leave blocks of 16 partly empty."""
+    a, b, rho, bv = pair_with_parents(8, 6, parents)
+    load(a, b, rho, bv)
+    cycles_parity(a, b, 2)
+    load(a, b, rho, bv)
+    a.solve(1e-12, 60)
+    st = b.solve(afgpu.default_opts(rel_tol=1e-10, precision=afgpu.AFG_MIXED))
+    assert st["rel_residual"] <= 1e-10
+    assert rel_diff(b.get_solution(), a.get_solution()) <= 1e-8
