@@ -599,8 +599,8 @@ __device__ __forceinline__ void rr_aligned(const BoxMeta &A, const BoxInfo &I, c
 // their four row pairs -- with its outward neighbour rows, and the four threads
 // of a coarse row add up by shuffles, each keeping a quarter of the cells.  Eight
 // vector and two scalar shared-memory reads a thread, without bank conflicts
-// (consecutive threads, consecutive rows), for a coarse cell that took 40 scalar
-// ones, half of them in conflict; shared memory was what bounded the kernel.
+// (consecutive threads, consecutive rows), in place of 40 scalar ones per coarse
+// cell, many of them in conflict.
 // 256^3: 45.7 -> 38.1 us (4.2 TB/s); uniform 512^3, mixed, 41.5 -> 37.1 ms (the sums
 // over a row's differences also round better than the sums over all 32 values).
 template <int D, int M, int MP, int GT>

@@ -571,7 +571,7 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
 // issues per update; 18.8 M unknowns, FP64, 29.0 -> 23.3 ms with the restriction
 // and the coarse right-hand side on aligned images too (2D keeps the per-cell
 // sums: its four terms need no FP64 addition).  Now 64.4 us (info_stage): issue
-// bound, 51 M warp instructions and 187 MB of DRAM traffic (2.9 TB/s) a launch.
+// bound, 52.6 M warp instructions and 191 MB of DRAM traffic (3.0 TB/s) a launch.
 template <int D, int M, typename T, int VPT>
 constexpr bool fx_smooth() { return sizeof(T) == 8 && D == 3 && SpCfg<D, M, T, VPT>::G >= 32; }
 
