@@ -428,7 +428,7 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
     BoxInfo *info = reinterpret_cast<BoxInfo *>(smem_raw + sizeof(T) * F::BOX * F::BPC * NST);
     const int stride = gridDim.x * F::BPC;
     const int first = blockIdx.x * F::BPC;
-    __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
+    __shared__ int2 fxr[FX ? kThreads / 32 : 1];
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
         info_stage<D>(A, first + q * stride + g, n, b0, list, info[q * F::BPC + g], lt, F::G);
     cp_commit();

@@ -377,28 +377,29 @@ constexpr int fx_lap_weight() { return 4 * D; }  // sum_nb u - 2D u
 
 // A thread aligns what it staged itself, so finding E costs no pass over the
 // image and no barrier of its own: after its wait a thread folds its values'
-// magnitudes (fx_fold), its warp leaves their extremes in `red` (two ints per
-// warp) ahead of the barrier that every box has, every thread then knows E
-// (fx_exponent), and after the alignment the group meets once more.
+// magnitudes (fx_fold), its warp leaves their extremes in `red` (one int2 per
+// warp, accessed as such: the type gives the array its 8-byte alignment) ahead
+// of the barrier that every box has, every thread then knows E (fx_exponent),
+// and after the alignment the group meets once more.
 __device__ __forceinline__ void fx_fold(double x, double y, unsigned &mx, unsigned &mn) {
     const unsigned a = (unsigned)__double2hiint(x) & 0x7fffffffu, b = (unsigned)__double2hiint(y) & 0x7fffffffu;
     const unsigned m = a > b ? a : b;
     mx = m > mx ? m : mx;
     if (m) mn = m < mn ? m : mn;
 }
-__device__ __forceinline__ void fx_leave(unsigned mx, unsigned mn, int *red) {
+__device__ __forceinline__ void fx_leave(unsigned mx, unsigned mn, int2 *red) {
     mx = __reduce_max_sync(0xffffffffu, mx);
     mn = __reduce_min_sync(0xffffffffu, mn);
-    if ((threadIdx.x & 31) == 0) reinterpret_cast<int2 *>(red)[threadIdx.x >> 5] = make_int2((int)mx, (int)mn);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_int2((int)mx, (int)mn);
 }
 // exponent of group g's values, or -1 where they are not aligned
 template <int G>
-__device__ __forceinline__ int fx_exponent(const int *red, int g) {
+__device__ __forceinline__ int fx_exponent(const int2 *red, int g) {
     static_assert(G >= 32, "whole warps per box");
     unsigned mx = 0, mn = 0x7fffffffu;
 #pragma unroll
     for (int x = 0; x < G / 32; ++x) {
-        const int2 r = reinterpret_cast<const int2 *>(red)[g * (G / 32) + x];
+        const int2 r = red[g * (G / 32) + x];
         mx = max(mx, (unsigned)r.x);
         mn = min(mn, (unsigned)r.y);
     }
@@ -425,7 +426,7 @@ __device__ __forceinline__ void fx_own(const Plan &pl, F f) {
         if (pl.gdst[q] >= 0) f(pl.gdst[q] & 0xffff, (pl.gdst[q] & (1 << 19)) != 0);
 }
 template <typename Plan>
-__device__ __forceinline__ void fx_fold_own(const Plan &pl, const double *st, int *red) {
+__device__ __forceinline__ void fx_fold_own(const Plan &pl, const double *st, int2 *red) {
     unsigned mx = 0, mn = 0x7fffffffu;
     fx_own(pl, [&](int q, bool scalar) { fx_fold(st[q], scalar ? 0.0 : st[q + 1], mx, mn); });
     fx_leave(mx, mn, red);
@@ -473,7 +474,7 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
         cr[itv] = r;
     }
     pdl_trigger();
-    __shared__ int fxr[FX ? 2 * kThreads / 32 : 1];
+    __shared__ int2 fxr[FX ? kThreads / 32 : 1];
     for (int q = 0; q < NST; ++q)  // static metadata: before the wait
         info_stage<D>(A, first + q * stride + g, n, b0, list, info[q * S::BPC + g], lt, S::G);
     cp_commit();
