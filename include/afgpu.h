@@ -317,7 +317,9 @@ int afg_residual_norm(afg_tree *t, double *max_abs_r, double *max_abs_rho);
  * (Neumann side) at the boundary-adjacent cell of every leaf boundary face.
  * BiCGStab with the preconditioner W M W^-1 (M one V-cycle, W the cell
  * volumes); opts->precision AFG_MIXED runs M in FP32 (K^T, the recurrences
- * and the tolerance stay FP64).  Output pointers may be NULL. */
+ * and the tolerance stay FP64).  Output pointers may be NULL.
+ * AFG_ERR_NOT_CONVERGED when the residual is above rel_tol after max_cycles or
+ * a breakdown, or not a number (stats->rel_residual NaN: g is not finite). */
 int afg_adjoint(afg_tree *t, const double *g_leaf_dev, double *lambda_leaf_dev,
                 double *dL_db_face_dev, const afg_mg_opts *opts, afg_stats *stats);
 

@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstring>
 #include <exception>
+#include <limits>
 #include <memory>
 #include <string>
 #include <vector>
@@ -303,7 +304,9 @@ double host_scalar(Grid &g, cudaStream_t s) {
 // preconditioner W M W^-1, where M is one linear FP64 V-cycle from zero with
 // homogeneous boundary data and W the diagonal of cell volumes.  W K is
 // symmetric up to the refinement-boundary terms, so W M W^-1 approximates
-// K^-T.  Returns iterations; sets *rel to max|g - K^T lam| / max|g|.
+// K^-T.  Returns iterations; sets *rel to max|g - K^T lam| / max|g|, NaN when g
+// is not finite.  A step whose scalars are not finite (a breakdown) ends the
+// iteration with the lam of the step before.
 int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g_leaf, double *rel) {
     g.ensure_adjoint();
     const afg::MgOpts mo{o.n_down, o.n_up, o.n_base};
@@ -358,8 +361,8 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
 
     const double bnorm = amax(bvec);
     check(cudaMemsetAsync(x, 0, bytes, s), "zero");
-    if (bnorm == 0.0) {
-        *rel = 0.0;
+    if (bnorm == 0.0 || !std::isfinite(bnorm)) {
+        *rel = bnorm == 0.0 ? 0.0 : std::numeric_limits<double>::quiet_NaN();
         return 0;
     }
     afg::launch_leaf_axpbypcz(lc, A, L, n, r, 1.0, bvec, 0.0, nullptr, 0.0, nullptr);
@@ -371,13 +374,14 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
     int it = 0;
     double res = 1.0;
     for (it = 1; it <= o.max_cycles; ++it) {
-        if (rho_new == 0.0) break;
+        if (rho_new == 0.0 || !std::isfinite(rho_new)) break;
         const double beta = (rho_new / rho_old) * (alpha / omega);
         afg::launch_leaf_axpbypcz(lc, A, L, n, p, 1.0, r, beta, p, -beta * omega, v);
         P_p();
         apply_T(ph, v);
         alpha = rho_new / dot(rh, v);
         res = update(sv, 1.0, r, -alpha, v, nullptr, nullptr) / bnorm;
+        if (!std::isfinite(res)) break;
         if (res <= o.rel_tol) {
             afg::launch_leaf_axpbypcz(lc, A, L, n, x, 1.0, x, alpha, ph, 0.0, nullptr);
             break;
@@ -387,10 +391,11 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
         afg::launch_leaf_reduce2(lc, A, L, n, nullptr, 0.0, t, 0.0, sv, nullptr, g.d_partials, g.d_scalar);
         const double tt = host_scalar(g, s);
         omega = tt > 0.0 ? g.h_scalar[1] / tt : 0.0;
+        if (!std::isfinite(tt) || !std::isfinite(omega)) break;
         afg::launch_leaf_axpbypcz(lc, A, L, n, x, 1.0, x, alpha, ph, omega, sh);
         rho_old = rho_new;
         res = update(r, 1.0, sv, -omega, t, rh, &rho_new) / bnorm;  // rho_new = rh . r, of the next step
-        if (res <= o.rel_tol || omega == 0.0) break;
+        if (res <= o.rel_tol || omega == 0.0 || !std::isfinite(res)) break;
     }
     // true residual
     apply_T(x, t);
@@ -885,7 +890,7 @@ int afg_adjoint(afg_tree *t, const double *g_leaf, double *lambda_leaf, double *
         st->rel_residual = rel;
         st->seconds = std::chrono::duration<double>(clk::now() - t0).count();
     }
-    if (rel > o.rel_tol) return fail(AFG_ERR_NOT_CONVERGED, "adjoint did not reach rel_tol");
+    if (!(rel <= o.rel_tol)) return fail(AFG_ERR_NOT_CONVERGED, "adjoint did not reach rel_tol");
     return AFG_OK;
     AFG_API_END
 }

@@ -325,6 +325,12 @@ __global__ void __launch_bounds__(kThreads) k_precond_out(BoxMeta A, const int *
     }
 }
 
+// max(m, |x|) for m >= 0 on the magnitudes' bit patterns: a NaN stays (fmax drops
+// it, and a vector of NaN then has norm 0)
+__device__ __forceinline__ double max_mag(double m, double x) {
+    return __longlong_as_double((long long)max((unsigned long long)__double_as_longlong(m), abs_bits(x)));
+}
+
 // Two reductions of leaf vectors in one pass, per-CTA partials at [block] and
 // [gridDim + block] (fixed grid: deterministic).
 //   out null: x . x and x . y
@@ -348,7 +354,7 @@ __global__ void __launch_bounds__(kThreads) k_leaf_reduce2(BoxMeta A, const int 
             if (out) {
                 const double v = a * xv + b * yv;
                 out[cb + q] = v;
-                p = fmax(p, fabs(v));
+                p = max_mag(p, v);
                 if (w) s += v * w[cb + q];
             } else {
                 p += xv * xv;
@@ -362,7 +368,7 @@ __global__ void __launch_bounds__(kThreads) k_leaf_reduce2(BoxMeta A, const int 
     for (int o = kThreads / 2; o > 0; o >>= 1) {
         if ((int)threadIdx.x < o) {
             const double q = red[0][threadIdx.x + o];
-            red[0][threadIdx.x] = out ? fmax(red[0][threadIdx.x], q) : red[0][threadIdx.x] + q;
+            red[0][threadIdx.x] = out ? max_mag(red[0][threadIdx.x], q) : red[0][threadIdx.x] + q;
             red[1][threadIdx.x] += red[1][threadIdx.x + o];
         }
         __syncthreads();
@@ -378,7 +384,7 @@ static __global__ void __launch_bounds__(kThreads) k_reduce2_final(const double 
     __shared__ double red[2][kThreads];
     double p = 0.0, s = 0.0;
     for (int i = threadIdx.x; i < n; i += kThreads) {
-        p = is_max ? fmax(p, partials[i]) : p + partials[i];
+        p = is_max ? max_mag(p, partials[i]) : p + partials[i];
         s += partials[n + i];
     }
     red[0][threadIdx.x] = p;
@@ -387,7 +393,7 @@ static __global__ void __launch_bounds__(kThreads) k_reduce2_final(const double 
     for (int o = kThreads / 2; o > 0; o >>= 1) {
         if ((int)threadIdx.x < o) {
             const double q = red[0][threadIdx.x + o];
-            red[0][threadIdx.x] = is_max ? fmax(red[0][threadIdx.x], q) : red[0][threadIdx.x] + q;
+            red[0][threadIdx.x] = is_max ? max_mag(red[0][threadIdx.x], q) : red[0][threadIdx.x] + q;
             red[1][threadIdx.x] += red[1][threadIdx.x + o];
         }
         __syncthreads();
@@ -414,14 +420,14 @@ __global__ void __launch_bounds__(kThreads) k_leaf_reduce(BoxMeta A, const int *
         const long long cb = A.coff[bi];
         for (int q = lt; q < Gm::C; q += Gm::G) {
             if (mode == 0) acc += x[cb + q] * y[cb + q];
-            else acc = fmax(acc, fabs(x[cb + q]));
+            else acc = max_mag(acc, x[cb + q]);
         }
     }
     red[threadIdx.x] = acc;
     __syncthreads();
     for (int o = kThreads / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] = mode == 0 ? red[threadIdx.x] + red[threadIdx.x + o]
-                                                          : fmax(red[threadIdx.x], red[threadIdx.x + o]);
+                                                          : max_mag(red[threadIdx.x], red[threadIdx.x + o]);
         __syncthreads();
     }
     if (threadIdx.x == 0) partials[blockIdx.x] = red[0];
@@ -430,12 +436,12 @@ __global__ void __launch_bounds__(kThreads) k_leaf_reduce(BoxMeta A, const int *
 static __global__ void __launch_bounds__(kThreads) k_reduce_final(const double *partials, int n, int mode, double *result) {
     __shared__ double red[kThreads];
     double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += kThreads) acc = mode == 0 ? acc + partials[i] : fmax(acc, partials[i]);
+    for (int i = threadIdx.x; i < n; i += kThreads) acc = mode == 0 ? acc + partials[i] : max_mag(acc, partials[i]);
     red[threadIdx.x] = acc;
     __syncthreads();
     for (int o = kThreads / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] = mode == 0 ? red[threadIdx.x] + red[threadIdx.x + o]
-                                                          : fmax(red[threadIdx.x], red[threadIdx.x + o]);
+                                                          : max_mag(red[threadIdx.x], red[threadIdx.x + o]);
         __syncthreads();
     }
     if (threadIdx.x == 0) *result = red[0];
