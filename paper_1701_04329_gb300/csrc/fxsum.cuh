@@ -120,7 +120,8 @@ struct FxAcc {
 };
 
 // x aligned to the exponent E of the largest of a set of values, in the fixed
-// point of FxAcc<W>: x = result * 2^(E - 1075 - G) but for the truncated bits.
+// point of FxAcc<W>: x = result * 2^(E - 1075 - G), exactly where its own exponent
+// is within G of E, and but for the truncated bits below that.
 // x's own exponent must not exceed E.
 template <int W>
 AFG_HD int64_t fx_align(double x, int E) {
@@ -130,6 +131,25 @@ AFG_HD int64_t fx_align(double x, int E) {
     const int64_t a = (int64_t)(m >> (s < 63 ? s : 63));  // m < 2^(53 + G) < 2^63
     const int64_t neg = (int64_t)b >> 63;
     return (a ^ neg) - neg;
+}
+
+// The extremes of a set of values' magnitudes, as their upper words (mx from 0,
+// mn from 0xffffffff): the largest, and the smallest but for zeros less one.  A
+// value whose upper word is zero counts as zero: it is below 2^-1042, far below
+// the last guard bit of any exponent that is aligned to.
+AFG_HD void fx_fold(double x, uint32_t &mx, uint32_t &mn) {
+    const uint32_t m = (uint32_t)(fx_bits(x) >> 32) & 0x7fffffffu;
+    mx = m > mx ? m : mx;
+    mn = m - 1 < mn ? m - 1 : mn;
+}
+
+// The exponent to align the set to for sums of weight W: that of the largest
+// value, where every other value's exponent lies within the G guard bits of it,
+// so that no bit is lost and the sums are exact; else -1.
+template <int W>
+AFG_HD int fx_common_exponent(uint32_t mx, uint32_t mn) {
+    const int E = (int)(mx >> 20);
+    return E >= kFxEmin && E <= kFxEmax && E - (int)((mn + 1) >> 20) <= FxAcc<W>::G ? E : -1;
 }
 
 // S * 2^(E - 1075 - G), nearest even: FxAcc<W>::round with the leading bit moved

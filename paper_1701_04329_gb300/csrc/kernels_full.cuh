@@ -481,7 +481,7 @@ __device__ __forceinline__ void fp_walk(const BoxMeta &A, int b0, int n, const i
             int E = -1;
             if constexpr (FX > 0) {
                 if (want(I)) {
-                    E = fx_exponent<GT>(fxr, g);
+                    E = fx_exponent<GT, FX>(fxr, g);
                     if (E >= 0) fx_own(pl, [&](int q, bool scalar) { fx_align_at<FX>(st + q, E, scalar); });
                     group_sync<GT>(g);
                 }

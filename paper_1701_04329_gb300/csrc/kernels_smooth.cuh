@@ -362,49 +362,46 @@ __device__ __forceinline__ bool box_sync(int g, bool extra) {
 // exponent (fx_sum) takes some 25 integer instructions a term.  A staged
 // image is read seven times over, so it is aligned once instead: every value
 // to the largest exponent E of the box and its ghosts, in place, as a 64-bit
-// integer with G guard bits below the last bit of a value of that exponent.
-// Sums of neighbours are then integer additions, exact, rounded once.
+// integer with G guard bits below the last bit of a value of that exponent
+// (G = FxAcc<W>::G for sums of weight W: 7 for the half-sweep, 6 for the
+// operator, 4 for the restriction in 3D).  Sums of neighbours are then integer
+// additions, exact, rounded once.
 //
-// The truncated bits are at most one unit of 2^-6 ulp (of the box's largest
-// value) per term; FP64 additions round to half an ulp of every partial sum.
-// A box whose values span more than 2^kFxSpan keeps the alignment per cell
-// (its small values would lose bits), and so does one whose largest exponent
-// is out of fx_sum's range (all zero, infinite, NaN).
+// A box is aligned only where that loses no bit of any value (fx_common_exponent).
+// So the aligned sums are the correctly rounded ones, and never further from the
+// exact sum than the sums per cell (fx_sum, or FP64 additions), which a box of a
+// wider span takes, and one whose largest exponent is out of fx_sum's range (all
+// zero, infinite, NaN).  Where the sign of the field changes a box has small
+// values beside large ones; such boxes are few (18.8 M unknowns, FP64: 21.5 ms
+// with boxes of a span of 2^8 and more aligned too, 21.7 ms; 4.3 M, FP64, forward
+// and adjoint, 24.3 and 24.8 ms).
 // ---------------------------------------------------------------------------
-constexpr int kFxSpan = 8;
 template <int D>
 constexpr int fx_lap_weight() { return 4 * D; }  // sum_nb u - 2D u
 
 // A thread aligns what it staged itself, so finding E costs no pass over the
 // image and no barrier of its own: after its wait a thread folds its values'
-// magnitudes (fx_fold), its warp leaves their extremes in `red` (one int2 per
-// warp, accessed as such: the type gives the array its 8-byte alignment) ahead
-// of the barrier that every box has, every thread then knows E (fx_exponent),
-// and after the alignment the group meets once more.
-__device__ __forceinline__ void fx_fold(double x, double y, unsigned &mx, unsigned &mn) {
-    const unsigned a = (unsigned)__double2hiint(x) & 0x7fffffffu, b = (unsigned)__double2hiint(y) & 0x7fffffffu;
-    const unsigned m = a > b ? a : b;
-    mx = m > mx ? m : mx;
-    if (m) mn = m < mn ? m : mn;
-}
+// magnitudes (fx_fold, every value by itself), its warp leaves their extremes in
+// `red` (one int2 per warp, accessed as such: the type gives the array its 8-byte
+// alignment) ahead of the barrier that every box has, every thread then knows E
+// (fx_exponent), and after the alignment the group meets once more.
 __device__ __forceinline__ void fx_leave(unsigned mx, unsigned mn, int2 *red) {
     mx = __reduce_max_sync(0xffffffffu, mx);
     mn = __reduce_min_sync(0xffffffffu, mn);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_int2((int)mx, (int)mn);
 }
-// exponent of group g's values, or -1 where they are not aligned
-template <int G>
+// exponent of group g's values, or -1 where they are not aligned (W: the sums' weight)
+template <int G, int W>
 __device__ __forceinline__ int fx_exponent(const int2 *red, int g) {
     static_assert(G >= 32, "whole warps per box");
-    unsigned mx = 0, mn = 0x7fffffffu;
+    unsigned mx = 0, mn = 0xffffffffu;
 #pragma unroll
     for (int x = 0; x < G / 32; ++x) {
         const int2 r = red[g * (G / 32) + x];
         mx = max(mx, (unsigned)r.x);
         mn = min(mn, (unsigned)r.y);
     }
-    const int E = (int)(mx >> 20);
-    return E >= kFxEmin && E <= kFxEmax && E - (int)(mn >> 20) <= kFxSpan ? E : -1;
+    return fx_common_exponent<W>(mx, mn);
 }
 template <int W>
 __device__ __forceinline__ void fx_align_at(double *p, int E, bool scalar) {
@@ -427,8 +424,11 @@ __device__ __forceinline__ void fx_own(const Plan &pl, F f) {
 }
 template <typename Plan>
 __device__ __forceinline__ void fx_fold_own(const Plan &pl, const double *st, int2 *red) {
-    unsigned mx = 0, mn = 0x7fffffffu;
-    fx_own(pl, [&](int q, bool scalar) { fx_fold(st[q], scalar ? 0.0 : st[q + 1], mx, mn); });
+    unsigned mx = 0, mn = 0xffffffffu;
+    fx_own(pl, [&](int q, bool scalar) {
+        fx_fold(st[q], mx, mn);
+        if (!scalar) fx_fold(st[q + 1], mx, mn);
+    });
     fx_leave(mx, mn, red);
 }
 
@@ -440,7 +440,7 @@ constexpr int kSmoothMinBlocks32 = 6, kSmoothMinBlocks64 = 5;
 // the new values from the neighbours (in the order -x, +x, -y, +y, -z, +z) and
 // the staged source.  early(I, v, itv) runs for the same vectors before the
 // box's copies are waited for (loads of its own that upd needs).
-// FX > 0 (FP64): the staged values are aligned (fx_image, sums of weight FX) and
+// FX > 0 (FP64): the staged values are aligned (fx_align_at, sums of weight FX) and
 // upd_fx(E, ...) forms the new values from them, upd only where they are not.
 template <int D, int M, typename T, int VPT, int FX = 0, typename Early, typename Upd, typename UpdFx>
 __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const int *list, T *u,
@@ -551,7 +551,7 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
             }
             };
             if constexpr (FX > 0) {
-                const int E = fx_exponent<S::G>(fxr, g);
+                const int E = fx_exponent<S::G, FX>(fxr, g);
                 if (E >= 0) fx_own(pl, [&](int q, bool scalar) { fx_align_at<FX>(box + q, E, scalar); });
                 group_sync<S::G>(g);
                 if (E >= 0)

@@ -15,7 +15,7 @@ SRC = r"""
 template <typename R, typename P> constexpr size_t slot_align(R (*)(unsigned, unsigned, P *)) { return alignof(P); }
 template <typename P> constexpr size_t slot_align(int (*)(const P *, int)) { return alignof(P); }
 static_assert(slot_align(&afg::fx_leave) >= sizeof(int2), "slots a warp writes as one int2");
-static_assert(slot_align(&afg::fx_exponent<32>) >= sizeof(int2), "slots a thread reads as one int2");
+static_assert(slot_align(&afg::fx_exponent<32, 6>) >= sizeof(int2), "slots a thread reads as one int2");
 """
 
 
