@@ -392,19 +392,17 @@ void Grid::clear_graphs() {
     graphs.clear();
 }
 
+// all of a workspace or, when it throws, none
 void Grid::alloc_ws(Workspace &w, bool fp64) {
     const size_t bytes = (size_t)ncell * (fp64 ? 8 : 4);
-    w.fp64 = fp64;
-    w.u.reset(new DevBuf(bytes));
-    w.rho.reset(new DevBuf(bytes));
-    w.vold.reset(new DevBuf(bytes));
-    check(cudaMemset(w.u->p, 0, bytes), "memset");
-    check(cudaMemset(w.rho->p, 0, bytes), "memset");
-    check(cudaMemset(w.vold->p, 0, bytes), "memset");
-    if (fp64) {
-        w.rhoh.reset(new DevBuf(bytes));
-        check(cudaMemset(w.rhoh->p, 0, bytes), "memset");
+    Workspace n;
+    n.fp64 = fp64;
+    for (auto *b : {&n.u, &n.rho, &n.vold, &n.rhoh}) {
+        if (b == &n.rhoh && !fp64) break;
+        b->reset(new DevBuf(bytes));
+        check(cudaMemset((*b)->p, 0, bytes), "memset");
     }
+    w = std::move(n);
 }
 
 void Grid::refresh_rho_hat(cudaStream_t s) {
