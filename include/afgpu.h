@@ -291,7 +291,14 @@ int afg_set_operator(afg_tree *t, int op);
 int afg_set_prolongation(afg_tree *t, int scheme);
 
 /* eps > 0 on leaf cells (n_leaf_cells doubles, canonical order, device
- * memory): stored on the leaves and restricted to every coarser level. */
+ * memory): stored on the leaves and restricted to every coarser level.  The
+ * call also forms the face coefficients, 2 dim + 2 values per cell in FP64 and,
+ * once mixed solves run, in FP32 (3D: 64 and 32 bytes per cell beside the 44 of
+ * the FP64 fields and eps and the 12 of the FP32 ones).  They are left out, and
+ * formed again on every use (solves two to four times slower), where they would
+ * take more than a quarter of the free device memory, where the allocator
+ * callback refuses them, or, given back, where the FP32 fields do not fit
+ * beside them. */
 int afg_set_eps(afg_tree *t, const double *eps_leaf_dev);
 
 /* Initial guess / warm start on leaf cells; without it the guess is zero. */

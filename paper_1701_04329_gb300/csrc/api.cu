@@ -222,7 +222,7 @@ int solve_fp64(Grid &g, const afg_mg_opts &o, cudaStream_t s, std::vector<std::v
 // first pass, inner_vcycles V-cycles afterwards); x += e in FP64.  Repeats
 // until the FP64 relative residual reaches rel_tol.
 int solve_mixed(Grid &g, const afg_mg_opts &o, cudaStream_t s, std::vector<std::vector<double>> &hist) {
-    g.ensure_mixed();
+    g.ensure_mixed(s);
     const afg::MgOpts mo{o.n_down, o.n_up, o.n_base};
     const bool forest = g.T > 1;
     std::vector<int> ones(g.T, 1);
@@ -338,7 +338,7 @@ int adjoint_solve(Grid &g, const afg_mg_opts &o, cudaStream_t s, const double *g
     const size_t bytes = (size_t)g.ncell * 8;
     // AFG_MIXED: M is one FP32 V-cycle (the BiCGStab recurrences and K^T stay FP64)
     const bool m32 = o.precision == AFG_MIXED;
-    if (m32) g.ensure_mixed();
+    if (m32) g.ensure_mixed(s);
     auto precond = [&](const double *in, double *out, cudaStream_t cs) {
         afg::Workspace &w = m32 ? g.ws32 : g.wsadj;
         afg::launch_precond_in(g.leaf_cfg(!m32, cs), A, L, n, in, w.rho->p, w.rhoh_p());
@@ -579,6 +579,7 @@ int afg_adapt_transfer(afg_tree *t, const int8_t *flags, int n_buf, int scheme, 
     if (n_added) *n_added = added;
     if (n_removed) *n_removed = removed;
     std::unique_ptr<Grid> fresh;
+    old.drop_coef();  // the old grid solves no more: room for the new one
     {
         std::vector<const HostTree *> v{&t->ht};
         fresh.reset(new Grid(v, t->op || t->prolong));
@@ -716,6 +717,10 @@ int afg_set_operator(afg_tree *t, int op) {
         t->grid->op = op;
         t->grid->eps_set = false;
         t->grid->clear_graphs();
+        if (!op) {  // the next eps asks for their memory anew
+            t->grid->drop_coef();
+            t->grid->coef_off[0] = t->grid->coef_off[1] = false;
+        }
     }
     return AFG_OK;
     AFG_API_END
@@ -1022,7 +1027,7 @@ int time_kernel_on(Grid &g, cudaStream_t s, int kernel, int level, int fp64, int
     if (g.op) return fail(AFG_ERR_STATE, "kernel timing covers the Laplacian's kernels");
     if (kernel < 3 && (level < g.lmin || level > g.lmax)) return fail(AFG_ERR_ARG, "level out of range");
     if ((kernel == 1 || kernel == 2) && level < 2) return fail(AFG_ERR_ARG, "level must be >= 2");
-    if (!fp64 || kernel == 3) g.ensure_mixed();
+    if (!fp64 || kernel == 3) g.ensure_mixed(s);
     g.refresh_rho_hat(s);
     afg::Workspace &w = fp64 ? g.ws64 : g.ws32;
     if (!fp64) {  // FP32 data from the FP64 source (values are irrelevant to timing)

@@ -411,8 +411,17 @@ void Grid::refresh_rho_hat(cudaStream_t s) {
     rhoh_stale = false;
 }
 
-void Grid::ensure_mixed() {
-    if (!ws32.u) alloc_ws(ws32, false);
+void Grid::ensure_mixed(cudaStream_t s) {
+    if (!ws32.u) {
+        try {
+            alloc_ws(ws32, false);
+        } catch (const NoMem &) {
+            if (!coef[1]) throw;
+            drop_coef();
+            alloc_ws(ws32, false);
+        }
+    }
+    if (op && coef32_stale) form_coef(false, s);
 }
 
 void Grid::ensure_adjoint() {
@@ -556,7 +565,7 @@ void Grid::launch_plan(Coarse &c, bool fp64, int mode, const BoxMeta &A, Workspa
 // the coarse launch's copy of the boundary data, after it changed (not captured)
 void Grid::refresh_faces(cudaStream_t s) {
     Coarse &c = coarse_plans[1][op != 0];
-    if (!c.faces_stale || levels_path()) return;
+    if (!c.faces_stale || levels_path(ws64)) return;
     launch_plan(c, true, 2, meta, ws64, s);
     c.faces_stale = false;
 }
@@ -580,7 +589,7 @@ void Grid::coarse_cycle(Workspace &w, int mode, const MgOpts &o, int hom, const 
 // FAS V-cycle (Sec. 3.2) from ltop down to the coarsest grid and back.  The
 // levels up to coarse(w).top run in one launch.
 void Grid::vcycle(Workspace &w, int ltop, const MgOpts &o, int hom, const int *active, cudaStream_t s) {
-    if (levels_path()) {
+    if (levels_path(w)) {
         vcycle_levels(w, ltop, o, hom, active, s);
         return;
     }
@@ -602,7 +611,7 @@ void Grid::vcycle(Workspace &w, int ltop, const MgOpts &o, int hom, const int *a
 // own finest level (masked).
 void Grid::fmg(Workspace &w, const MgOpts &o, int hom, bool masked, cudaStream_t s) {
     // the levels up to l0 in one launch (every tree reaches level l0)
-    const bool levels = levels_path();
+    const bool levels = levels_path(w);
     const int l0 = levels ? 1 : coarse(w).top, low = levels ? lmin : l0;
     for (int l = lmax; l > low; --l) restrict_u(w, l, L(l).b0, L(l).nb, nullptr, s);
     for (int l = lmax; l > low; --l) down_step(w, l, hom, nullptr, s, levels || l - 1 > low);
@@ -631,9 +640,9 @@ void Grid::restrict_u(Workspace &w, int l, int b0, int n, const int *list, cudaS
     else launch_restrict_u(cfg(l, w.fp64, s), meta, b0, n, list, w.u->p);
 }
 
-// Variable-coefficient operators: the V-cycle on the per-level kernels all
-// the way down (the coarse grids below the root have one box per tree),
-// N_base steps on the 2^D-cell grid.
+// Where the coarse launch does not run (levels_path): the V-cycle on the
+// per-level kernels all the way down, N_base steps on the coarsest grid of 2^D
+// cells per root box.
 void Grid::vcycle_levels(Workspace &w, int ltop, const MgOpts &o, int hom, const int *active, cudaStream_t s) {
     for (int l = ltop; l > lmin; --l) {
         smooth(w, l, o.n_down, hom, active, s);
@@ -655,7 +664,7 @@ void Grid::correct(Workspace &w, int l, const int *active, cudaStream_t s) {
     else launch_correct(cfg(l, w.fp64, s), A, v.b0, v.nb, w.u->p, w.vold->p);
 }
 
-// the FMG steps l = lmin..1 (Sec. 3.2) for the variable-coefficient operators
+// the FMG steps l = lmin..1 (Sec. 3.2) where the coarse launch does not run
 void Grid::fmg_low_levels(Workspace &w, const MgOpts &o, int hom, cudaStream_t s) {
     const size_t es = w.fp64 ? 8 : 4;
     for (int l = lmin; l <= 1; ++l) {
@@ -691,25 +700,62 @@ void Grid::set_eps(const double *eps_leaf, cudaStream_t s) {
     launch_leaf_set(leaf_cfg(true, s), meta, d_leaves, n_leaf_boxes, eps_leaf, eps64->p);
     for (int l = lmax; l > lmin; --l) launch_var_restrict(cfg(l, true, s), meta, L(l).b0, L(l).nb, nullptr, eps64->p, op);
     launch_to_f32(eps64->as<double>(), eps32->as<float>(), ncell, s);
-    const size_t nc = (size_t)ncell * (2 * D + 2);
-    if (!coef64) coef64.reset(new DevBuf(nc * 8));
-    if (!coef32) coef32.reset(new DevBuf(nc * 4));
-    for (int l = lmin; l <= lmax; ++l) {
-        launch_var_coef(cfg(l, true, s), meta, L(l).b0, L(l).nb, eps64->p, coef64->p, ncell, op);
-        launch_var_coef(cfg(l, false, s), meta, L(l).b0, L(l).nb, eps32->p, coef32->p, ncell, op);
-    }
-    for (int fp64 = 0; fp64 < 2 && !roots_levels; ++fp64) {  // the coarse launch's packed copies
-        Coarse &c = coarse_plans[fp64][1];
-        if (!c.ok) continue;
-        if (!c.cpack) c.cpack.reset(new DevBuf((size_t)c.plan.ncoef * c.plan.R * T * (fp64 ? 8 : 4)));
-        check(cudaMemsetAsync(c.cpack->p, 0, c.cpack->bytes, s), "memset");
-        c.plan.cpack = c.cpack->p;
-        c.plan.coef = fp64 ? coef64->p : coef32->p;
-        c.plan.coef_n = ncell;
-        c.plan.op = op;
-        launch_plan(c, fp64, 3, meta, ws64, s);
-    }
+    form_coef(true, s);
+    if (ws32.u) form_coef(false, s);
+    else coef32_stale = true;
     eps_set = true;
+}
+
+// The face coefficients in one precision from eps, and the coarse launch's packed
+// copy of them.  With 2D + 2 values a cell they take more than all other fields of
+// an FP64 solve, and a size that fits without them has to run: they may have a
+// quarter of the device memory that is free when they are first wanted (a caller's
+// allocator says by itself what there is), so that later fields and other trees
+// find room.
+void Grid::form_coef(bool fp64, cudaStream_t s) {
+    if (!fp64) coef32_stale = false;
+    if (coef_off[fp64]) return;
+    const size_t es = fp64 ? 8 : 4, bytes = (size_t)ncell * (2 * D + 2) * es;
+    Coarse &c = coarse_plans[fp64][1];
+    const bool pack = c.ok && !roots_levels;
+    auto &buf = coef[fp64];
+    if (!buf) {
+        try {
+            size_t avail = 0, all = 0;
+            if (!allocator().alloc) {
+                check(cudaMemGetInfo(&avail, &all), "cudaMemGetInfo");
+                if (bytes > avail / 4) throw NoMem("face coefficients");
+            }
+            std::unique_ptr<DevBuf> arrays(new DevBuf(bytes)), packed;
+            if (pack) packed.reset(new DevBuf((size_t)c.plan.ncoef * c.plan.R * T * es));
+            buf = std::move(arrays);
+            c.cpack = std::move(packed);
+        } catch (const NoMem &) {
+            coef_off[fp64] = true;
+            return;
+        }
+    }
+    for (int l = lmin; l <= lmax; ++l)
+        launch_var_coef(cfg(l, fp64, s), meta, L(l).b0, L(l).nb, fp64 ? eps64->p : eps32->p, buf->p, ncell, op);
+    if (!pack) return;
+    check(cudaMemsetAsync(c.cpack->p, 0, c.cpack->bytes, s), "memset");
+    c.plan.cpack = c.cpack->p;
+    c.plan.coef = buf->p;
+    c.plan.coef_n = ncell;
+    c.plan.op = op;
+    launch_plan(c, fp64, 3, meta, ws64, s);
+}
+
+// gives the coefficients' memory back, with the graphs that hold its addresses
+void Grid::drop_coef() {
+    if (!coef[0] && !coef[1]) return;
+    check(cudaDeviceSynchronize(), "drop_coef");
+    clear_graphs();
+    for (int fp64 = 0; fp64 < 2; ++fp64) {
+        coef[fp64].reset();
+        coarse_plans[fp64][1].cpack.reset();
+        coef_off[fp64] = true;
+    }
 }
 
 // The composite residual reads a parent's values only where the parent

@@ -142,17 +142,27 @@ class Grid {
     // eps on every level (leaves: the user's values, parents: restrictions) in both precisions
     int op = 0;
     std::unique_ptr<DevBuf> eps64, eps32;
-    std::unique_ptr<DevBuf> coef64, coef32;  // face coefficients of every cell (2D + 2 arrays of ncell values)
+    // face coefficients of every cell (2D + 2 arrays of ncell values) per
+    // precision [fp64], formed for the precisions that run: FP32 with the first
+    // mixed solve.  They are a copy that saves time, not data: where their memory
+    // is not there they are left out (coef_off) and the kernels form them from eps.
+    std::unique_ptr<DevBuf> coef[2];
+    bool coef_off[2] = {false, false}, coef32_stale = false;
+    void form_coef(bool fp64, cudaStream_t s);
+    void drop_coef();
     VarArgs var_args(const Workspace &w, int l) {
-        return VarArgs{eps_of(w), w.fp64 ? coef64->p : coef32->p, ncell, op, L(l).h};
+        const auto &c = coef[w.fp64];
+        return VarArgs{eps_of(w), c ? c->p : nullptr, ncell, op, L(l).h};
     }
     bool eps_set = false;
     double *d_x0 = nullptr;  // lower x coordinate of every box
     // prolongation of the coarse-grid correction (Sec. 2.5): 0 linear, 1 bi/trilinear, 2 zeroth order
     int prolong = 0;
     int *d_nball = nullptr;  // same-level neighbour of every box in all 3^D - 1 directions, -1 none
-    // another prolongation, or no coarse launch: every level on the per-level kernels
-    bool levels_path() const { return prolong != 0 || roots_levels || !coarse_plans[1][op != 0].ok; }
+    // another prolongation, no coarse launch, or no coefficients for it: every level on the per-level kernels
+    bool levels_path(const Workspace &w) const {
+        return prolong != 0 || roots_levels || !coarse_plans[1][op != 0].ok || (op && !coarse_plans[w.fp64][1].cpack);
+    }
     int vpt = 1;  // FP32 half-sweep: 16-byte vectors per thread (the threads-per-box option)
     // trees of several root boxes whose coarse grids are device boxes (one per
     // root and level): the cycle runs on the per-level kernels
@@ -189,7 +199,7 @@ class Grid {
     }
 
     void alloc_ws(Workspace &w, bool fp64);
-    void ensure_mixed();
+    void ensure_mixed(cudaStream_t s);
     void ensure_adjoint();
 
     // ---- multigrid building blocks ---------------------------------------

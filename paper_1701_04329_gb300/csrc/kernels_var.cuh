@@ -22,7 +22,9 @@
 //
 // These kernels are table-driven: a thread group stages one box (u and eps
 // with all side ghosts, and rho where needed) in shared memory and walks
-// the box's cells.
+// the box's cells.  The cycle runs on them where the face coefficients are not
+// kept (kernels_var_staged.cuh): on grids too small for the staged kernels, and
+// where the memory for the coefficients is not there.
 #pragma once
 #include "kernels.cuh"
 
@@ -247,6 +249,58 @@ __global__ void __launch_bounds__(kThreads) k_var_fas(BoxMeta A, int b0, int n, 
         }
     };
     var_walk<D, M, T>(A, b0, n, nullptr, u, eps, rho, hom, true, body, VarNoPost());
+}
+
+// Composite residual on the leaf boxes of a list: per tree the maxima of |r|
+// and |rho| (reduced as magnitude bit patterns, so a NaN stays), and r (cast to
+// R) in rout when it is not null.
+template <int D, int M, typename T, typename Ro>
+__global__ void __launch_bounds__(kThreads) k_var_leaf_residual(BoxMeta A, const int *list, int n, const T *u,
+                                                                const T *rho, const T *eps, int hom, int op,
+                                                                unsigned long long *rmax, unsigned long long *pmax,
+                                                                Ro *rout) {
+    using S = VarCfg<D, M, T>;
+    pdl_trigger();
+    __shared__ unsigned long long red[2 * kThreads / 32];
+    unsigned long long rm = 0, pm = 0;
+    auto body = [&](const BoxInfo &I, const T *U, const T *E, const T *R, int lt, const short *tix) {
+        const T h = T(A.hb[I.b]), x0 = T(A.x0[I.b]), ih2 = T(1) / (h * h);
+        for (int q = lt; q < S::C; q += S::G) {
+            int i, j, k;
+            rb_cell<D, M>(q, i, j, k);
+            const int t = tix[q];
+            T sv, sc;
+            var_sums<D, M, T>(U, E, t, i, h, x0, op, sv, sc);
+            const T r = R[q] - (sv - sc * U[t]) * ih2;
+            if (rout) rout[I.coff + q] = Ro(r);
+            rm = max(rm, abs_bits(r));
+            pm = max(pm, abs_bits(R[q]));
+        }
+    };
+    // per box: maxima over its thread group (shuffles within a warp, then
+    // shared memory across the group's warps), one atomic per box and norm
+    auto post = [&](const BoxInfo &I, int lt) {
+        constexpr int W = S::G < 32 ? S::G : 32;
+        for (int off = W / 2; off > 0; off >>= 1) {
+            rm = max(rm, __shfl_xor_sync(0xffffffffu, rm, off));
+            pm = max(pm, __shfl_xor_sync(0xffffffffu, pm, off));
+        }
+        if constexpr (S::G > 32) {
+            const int w = threadIdx.x / 32;
+            if ((threadIdx.x & 31) == 0) { red[2 * w] = rm; red[2 * w + 1] = pm; }
+            __syncthreads();
+            if (lt == 0)
+                for (int x = 1; x < S::G / 32; ++x) { rm = max(rm, red[2 * (w + x)]); pm = max(pm, red[2 * (w + x) + 1]); }
+        }
+        if (lt == 0 && I.b >= 0) {
+            const int tr = A.tree[I.b];
+            atomicMax(rmax + tr, rm);
+            atomicMax(pmax + tr, pm);
+        }
+        rm = 0;
+        pm = 0;
+    };
+    var_walk<D, M, T>(A, 0, n, list, u, eps, rho, hom, true, body, post);
 }
 
 // Restriction of a field (u or eps) from the boxes of a level (or a list of

@@ -99,8 +99,8 @@ constexpr int kPartials = 4096;  // size of the partials buffer (doubles)
 
 // Variable-coefficient operators (kernels_var.cuh, kernels_var_staged.cuh): op
 // 1 div(eps grad u), op 2 the same in (r,z) coordinates; eps and the face
-// coefficients (2D + 2 arrays, n values apart) in the field layout, same
-// precision; h the level's cell size.
+// coefficients (2D + 2 arrays, n values apart; null: formed from eps on every
+// use) in the field layout, same precision; h the level's cell size.
 struct VarArgs {
     const void *eps, *coef;
     long long n;

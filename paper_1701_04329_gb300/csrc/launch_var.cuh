@@ -10,8 +10,9 @@
 namespace afg {
 
 // The staged kernels with stored coefficients wherever a half-row holds a
-// 16-byte vector; the others (grids of 2 cells per side, and of 4 in FP32)
-// stay on the kernels that form the coefficients from eps.
+// 16-byte vector; the others (grids of 2 cells per side, and of 4 in FP32), and
+// all grids where the coefficients are not kept (W.coef null), take the kernels
+// that form the coefficients from eps.
 template <int D, int M, typename T>
 void do_var_coef(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void *eps, void *coef, long long nc,
                  int op) {
@@ -28,13 +29,15 @@ void do_var_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u,
                    int colour, int hom) {
     if (n <= 0) return;
     if constexpr (SpCfg<D, M, T>::ok) {
-        using S = SpCfg<D, M, T>;
-        auto k = k_var_smooth_p<D, M, T>;
-        const VarCoef<T> V{(const T *)W.coef, W.n};
-        launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (T *)u,
-                   (const T *)rho, V, T(W.h * W.h), colour, hom);
-        ++g_launches;
-        return;
+        if (W.coef) {
+            using S = SpCfg<D, M, T>;
+            auto k = k_var_smooth_p<D, M, T>;
+            const VarCoef<T> V{(const T *)W.coef, W.n};
+            launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, b0, n, (T *)u,
+                       (const T *)rho, V, T(W.h * W.h), colour, hom);
+            ++g_launches;
+            return;
+        }
     }
     const void *eps = W.eps;
     const int op = W.op;
@@ -50,13 +53,15 @@ void do_var_resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, 
                            const VarArgs &W, int hom) {
     if (n <= 0) return;
     if constexpr (FpCfg<D, M, T>::ok) {
-        using F = FpCfg<D, M, T, fas_threads<D, M, T>()>;
-        auto k = k_var_resid_restrict_p<D, M, MP, T>;
-        const VarCoef<T> V{(const T *)W.coef, W.n};
-        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, b0, n, (T *)u,
-                   (T *)rho, (T *)vold, V, T(1.0 / (W.h * W.h)), hom, W.op);
-        ++g_launches;
-        return;
+        if (W.coef) {
+            using F = FpCfg<D, M, T, fas_threads<D, M, T>()>;
+            auto k = k_var_resid_restrict_p<D, M, MP, T>;
+            const VarCoef<T> V{(const T *)W.coef, W.n};
+            launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, b0, n, (T *)u,
+                       (T *)rho, (T *)vold, V, T(1.0 / (W.h * W.h)), hom, W.op);
+            ++g_launches;
+            return;
+        }
     }
     const void *eps = W.eps;
     const int op = W.op;
@@ -72,13 +77,15 @@ void do_var_fas(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const void 
                 const VarArgs &W, int hom) {
     if (n <= 0) return;
     if constexpr (FpCfg<D, M, T>::ok) {
-        using F = FpCfg<D, M, T, fas_threads<D, M, T>()>;
-        auto k = k_var_fas_p<D, M, T>;
-        const VarCoef<T> V{(const T *)W.coef, W.n};
-        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, b0, n, (const T *)u,
-                   (T *)rho, (T *)vold, V, T(1.0 / (W.h * W.h)), hom);
-        ++g_launches;
-        return;
+        if (W.coef) {
+            using F = FpCfg<D, M, T, fas_threads<D, M, T>()>;
+            auto k = k_var_fas_p<D, M, T>;
+            const VarCoef<T> V{(const T *)W.coef, W.n};
+            launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, b0, n, (const T *)u,
+                       (T *)rho, (T *)vold, V, T(1.0 / (W.h * W.h)), hom);
+            ++g_launches;
+            return;
+        }
     }
     const void *eps = W.eps;
     const int op = W.op;
@@ -95,11 +102,18 @@ void do_var_leaf_residual(const LaunchCfg &c, const BoxMeta &A, const int *list,
                           unsigned long long *pmax, void *rout) {
     if (n <= 0) return;
     static_assert(FpCfg<D, M, T>::ok, "leaf boxes have 4 cells per side or more, in FP64");
-    using F = FpCfg<D, M, T, leaf_threads<D, M, T, Ro>()>;
-    auto k = c.one_tree ? k_var_leaf_residual_p<D, M, T, Ro, true> : k_var_leaf_residual_p<D, M, T, Ro, false>;
-    const VarCoef<T> V{(const T *)W.coef, W.n};
-    launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, (const T *)u,
-               (const T *)rho, V, hom, rmax, pmax, (Ro *)rout);
+    if (W.coef) {
+        using F = FpCfg<D, M, T, leaf_threads<D, M, T, Ro>()>;
+        auto k = c.one_tree ? k_var_leaf_residual_p<D, M, T, Ro, true> : k_var_leaf_residual_p<D, M, T, Ro, false>;
+        const VarCoef<T> V{(const T *)W.coef, W.n};
+        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n,
+                   (const T *)u, (const T *)rho, V, hom, rmax, pmax, (Ro *)rout);
+    } else {
+        using S = VarCfg<D, M, T>;
+        auto k = k_var_leaf_residual<D, M, T, Ro>;
+        launch_pdl(k, grid_for(k, S::smem(), (n + S::BPC - 1) / S::BPC), S::smem(), c.stream, A, list, n,
+                   (const T *)u, (const T *)rho, (const T *)W.eps, hom, W.op, rmax, pmax, (Ro *)rout);
+    }
     ++g_launches;
 }
 
