@@ -374,7 +374,7 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     check(cudaMallocHost((void **)&h_norms, 2 * T * sizeof(unsigned long long)), "cudaMallocHost");
     check(cudaMallocHost((void **)&h_nactive, sizeof(int)), "cudaMallocHost");
     check(cudaMallocHost((void **)&h_scalar, 2 * sizeof(double)), "cudaMallocHost");
-    alloc_ws(ws64, true);
+    alloc_ws(ws64, true);  // and waits for the memsets and copies above
 }
 
 Grid::~Grid() {
@@ -392,7 +392,8 @@ void Grid::clear_graphs() {
     graphs.clear();
 }
 
-// all of a workspace or, when it throws, none
+// All of a workspace or, when it throws, none.  The memsets run on the default
+// stream and a caller's stream need not wait for that one, so they are waited for.
 void Grid::alloc_ws(Workspace &w, bool fp64) {
     const size_t bytes = (size_t)ncell * (fp64 ? 8 : 4);
     Workspace n;
@@ -402,6 +403,7 @@ void Grid::alloc_ws(Workspace &w, bool fp64) {
         b->reset(new DevBuf(bytes));
         check(cudaMemset((*b)->p, 0, bytes), "memset");
     }
+    check(cudaStreamSynchronize(nullptr), "memset");
     w = std::move(n);
 }
 
@@ -426,10 +428,12 @@ void Grid::ensure_mixed(cudaStream_t s) {
 
 void Grid::ensure_adjoint() {
     if (!wsadj.u) alloc_ws(wsadj, true);
+    if (bicg.size() == 10) return;
     while (bicg.size() < 10) {
         bicg.emplace_back(new DevBuf((size_t)ncell * 8));
         check(cudaMemset(bicg.back()->p, 0, (size_t)ncell * 8), "memset");
     }
+    check(cudaStreamSynchronize(nullptr), "memset");
 }
 
 // ---- multigrid building blocks --------------------------------------------
