@@ -297,25 +297,9 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     for (int b = 0; b < nbox; ++b) ih2[b] = 1.0 / (hb[b] * hb[b]);
     meta.ih2 = upload(ih2, own);
     meta.active = nullptr;
-    {
-        std::vector<BoxInfo> info(nbox);
-        for (int b = 0; b < nbox; ++b) {
-            BoxInfo &I = info[b];
-            std::memset(&I, 0, sizeof I);
-            I.coff = coff[b];
-            for (int s = 0; s < S; ++s) {
-                I.base[s] = nbase[b * S + s];
-                I.code[s] = nb[b * S + s];
-            }
-            I.b = b;
-            I.flag = bflag[b] | (cfmask[b] << 8);
-            I.poff = poff[b];
-            I.parent = parent[b];
-            I.nmask = (I.flag >> BF_NSHIFT) & 0x3f;
-            I.tree = tree[b];
-        }
-        meta.info = upload(info, own);
-    }
+    own.emplace_back(new DevBuf((size_t)nbox * sizeof(BoxInfo)));
+    launch_box_info(meta, nbox, S, own.back()->as<BoxInfo>());
+    meta.info = own.back()->as<BoxInfo>();
     d_child = upload(child, own);
     d_leaves = upload(leaves, own);
     d_leaf_geo = upload(leaf_geo, own);
@@ -327,8 +311,9 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     }
     n_adj_plain = (int)plain.size();
     n_adj_rest = (int)rest.size();
+    plain.insert(plain.end(), rest.begin(), rest.end());
     d_adj_plain = upload(plain, own);
-    d_adj_rest = upload(rest, own);
+    d_adj_rest = d_adj_plain + n_adj_plain;
     if (singular && T > 1) {  // forests: per-tree compatibility constants and means
         std::vector<int> leaf0(T + 1, 0);
         for (int t = 0; t < T; ++t) leaf0[t + 1] = leaf0[t] + (int)trees[t]->leaves.size();
@@ -492,15 +477,26 @@ void Grid::plan_coarse(const std::vector<const HostTree *> &trees, const std::ve
         }
         bc.push_back(code);
     }
-    const int *d_bc_types = upload(bc, owned);
-    std::map<int, const int *> tables;  // boxes of a level by position, per tree
+    // every table of the plans, copied to the device together: the plans' pointers
+    // are filled in when it lies there
+    std::vector<int> all = bc;
+    struct Slot {
+        const int **to;
+        size_t at;
+    };
+    std::vector<Slot> slots;
+    auto append = [&](const std::vector<int> &v) {
+        all.insert(all.end(), v.begin(), v.end());
+        return all.size() - v.size();
+    };
+    std::map<int, size_t> tables;  // boxes of a level by position, per tree
     auto table = [&](int l) {
         auto it = tables.find(l);
         if (it != tables.end()) return it->second;
         std::vector<int> v;
         if (l < 1) {  // one box per tree (trees of one root box)
             for (int t = 0; t < T; ++t) v.push_back(L(l).b0 + t);
-            return tables[l] = upload(v, owned);
+            return tables[l] = append(v);
         }
         const int f = 1 << (l - 1);
         const int sx = nr[0] * f, sy = nr[1] * f, sz = D == 3 ? nr[2] * f : 1;
@@ -511,8 +507,9 @@ void Grid::plan_coarse(const std::vector<const HostTree *> &trees, const std::ve
                 const int z = D == 3 ? x.idx[2] - 1 : 0;
                 v[(((size_t)t * sz + z) * sy + (x.idx[1] - 1)) * sx + (x.idx[0] - 1)] = gid[t][b];
             }
-        return tables[l] = upload(v, owned);
+        return tables[l] = append(v);
     };
+    size_t nfval = 0;
     for (int fp64 = 0; fp64 < 2; ++fp64)
         for (int var = 0; var < (block ? 1 : 2); ++var) {
             Coarse &c = coarse_plans[fp64][var];
@@ -536,28 +533,39 @@ void Grid::plan_coarse(const std::vector<const HostTree *> &trees, const std::ve
                 c.ok = true;
             }
             if (!c.ok) continue;
-            c.plan.dbox = table(c.top);
+            slots.push_back({&c.plan.dbox, table(c.top)});
             if (var)
-                for (int li = 0; li < c.plan.nl; ++li) c.plan.dtab[li] = table(lmin + li);
-            c.plan.tree_bc = d_bc_types;
+                for (int li = 0; li < c.plan.nl; ++li) slots.push_back({&c.plan.dtab[li], table(lmin + li)});
+            slots.push_back({&c.plan.tree_bc, 0});
             // faces: the slots of every non-periodic axis in any tree (a tree's own periodic sides are not read)
-            int all = 7;
-            for (int code : bc) all &= code >> 6;
-            std::vector<std::vector<int>> slots;
+            int periodic = 7;
+            for (int code : bc) periodic &= code >> 6;
+            std::vector<std::vector<int>> faces;
             size_t most_faces = 0;
             for (int r = 0; r < c.plan.R; ++r) {
-                slots.push_back(coarse_faces(D, c.plan, r, all));
-                most_faces = std::max(most_faces, slots.back().size());
+                faces.push_back(coarse_faces(D, c.plan, r, periodic));
+                most_faces = std::max(most_faces, faces.back().size());
             }
             std::vector<int> flat;
-            for (auto &v : slots) {
+            for (auto &v : faces) {
                 v.resize(most_faces, -1);
                 flat.insert(flat.end(), v.begin(), v.end());
             }
             c.plan.nface = (int)most_faces;
-            c.plan.fslot = upload(flat, owned);
-            if (fp64) c.plan.fval = upload(std::vector<double>(most_faces * c.plan.R * T, 0.0), owned);
+            slots.push_back({&c.plan.fslot, append(flat)});
+            if (fp64) nfval += most_faces * c.plan.R * T;
         }
+    const int *d_all = upload(all, owned);
+    for (const Slot &x : slots) *x.to = d_all + x.at;
+    // the boundary values of the FP64 plans, zero until there are any
+    owned.emplace_back(new DevBuf(std::max<size_t>(1, nfval) * sizeof(double)));
+    double *fval = owned.back()->as<double>();
+    check(cudaMemset(fval, 0, owned.back()->bytes), "memset");
+    for (Coarse &c : coarse_plans[1]) {
+        if (!c.ok) continue;
+        c.plan.fval = fval;
+        fval += (size_t)c.plan.nface * c.plan.R * T;
+    }
 }
 
 void Grid::launch_plan(Coarse &c, bool fp64, int mode, const BoxMeta &A, Workspace &w, cudaStream_t s) {

@@ -229,6 +229,8 @@ class Grid {
     void clear_graphs();
 };
 
+// every box's record (A.info) from the other arrays of the metadata; S sides, on the default stream
+void launch_box_info(const BoxMeta &A, int nbox, int S, BoxInfo *out);
 // leaf cell centres (canonical order, D doubles per cell) into device memory
 void launch_cell_centers(const Grid &g, double *xyz, cudaStream_t s);
 // refinement flags of the leaf cells from a leaf field (canonical order)

@@ -21,6 +21,25 @@ __global__ void k_cell_centers(const double *geo, int D, int N, long long ncells
         for (int a = 0; a < D; ++a) xyz[q * D + a] = g[a] + (ci[a] + 0.5) * g[3];
     }
 }
+// the record of a box that the staged kernels copy, from the metadata arrays
+__global__ void k_box_info(BoxMeta A, int nbox, int S, BoxInfo *out) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= nbox) return;
+    BoxInfo I = {};
+    I.coff = A.coff[b];
+    for (int s = 0; s < S; ++s) {
+        I.base[s] = A.nbase[b * S + s];
+        I.code[s] = A.nb[b * S + s];
+    }
+    I.b = b;
+    I.flag = A.bflag[b] | (A.cfmask[b] << 8);
+    I.poff = A.poff[b];
+    I.parent = A.parent[b];
+    I.nmask = (I.flag >> BF_NSHIFT) & 0x3f;
+    I.tree = A.tree[b];
+    out[b] = I;
+}
+
 // refinement flags from a leaf field f: +1 where |f| h^power > tau_refine,
 // -1 where |f| h^power < tau_coarsen, 0 elsewhere (h the cell size)
 __global__ void k_flag(const double *geo, int D, int N, long long ncells, const double *f, int power, double tau_ref,
@@ -191,6 +210,12 @@ void launch_leaf_center(const Grid &g, double *f, bool with_flux, cudaStream_t s
     k_leaf_shift<<<blocks, 256, 0, s>>>(g.meta, g.d_leaves, g.n_leaf_boxes, C, f, g.d_scalar);
     g_launches += 3;
     check(cudaGetLastError(), "k_leaf_vsum");
+}
+
+void launch_box_info(const BoxMeta &A, int nbox, int S, BoxInfo *out) {
+    k_box_info<<<(nbox + 255) / 256, 256>>>(A, nbox, S, out);
+    ++g_launches;
+    check(cudaGetLastError(), "k_box_info");
 }
 
 void launch_cell_centers(const Grid &g, double *xyz, cudaStream_t s) {
