@@ -739,7 +739,10 @@ void Grid::form_coef(bool fp64, cudaStream_t s) {
                 if (bytes > avail / 4) throw NoMem("face coefficients");
             }
             std::unique_ptr<DevBuf> arrays(new DevBuf(bytes)), packed;
-            if (pack) packed.reset(new DevBuf((size_t)c.plan.ncoef * c.plan.R * T * es));
+            if (pack) {
+                packed.reset(new DevBuf((size_t)c.plan.ncoef * c.plan.R * T * es));
+                check(cudaMemsetAsync(packed->p, 0, packed->bytes, s), "memset");  // the ghost slots stay zero
+            }
             buf = std::move(arrays);
             c.cpack = std::move(packed);
         } catch (const NoMem &) {
@@ -747,10 +750,11 @@ void Grid::form_coef(bool fp64, cudaStream_t s) {
             return;
         }
     }
-    for (int l = lmin; l <= lmax; ++l)
-        launch_var_coef(cfg(l, fp64, s), meta, L(l).b0, L(l).nb, fp64 ? eps64->p : eps32->p, buf->p, ncell, op);
+    // the boxes of level 1 and up are of one size and consecutive: one launch
+    for (int l = lmin; l <= 1; ++l)
+        launch_var_coef(cfg(l, fp64, s), meta, L(l).b0, l < 1 ? L(l).nb : nbox - L(l).b0,
+                        fp64 ? eps64->p : eps32->p, buf->p, ncell, op);
     if (!pack) return;
-    check(cudaMemsetAsync(c.cpack->p, 0, c.cpack->bytes, s), "memset");
     c.plan.cpack = c.cpack->p;
     c.plan.coef = buf->p;
     c.plan.coef_n = ncell;
