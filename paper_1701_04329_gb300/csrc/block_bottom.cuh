@@ -6,15 +6,19 @@
 // functions hold it: one array per field with a ghost layer, cells
 // lexicographic with x fastest.
 //
+// No kernel is built from these functions: the coarse launch (kernels_coarse.cuh)
+// has its own steps, and the tests of the GPU path compare that with the oracle.
+// This is the plain statement of the same steps on such a grid, compiled for the
+// host and pinned against the oracle bit by bit.
+//
 // Each function performs one step of the multigrid cycle on such grids with
 // the arithmetic of the per-box operators (sums in the order
 // ((x- + x+) + (y- + y+)) + (z- + z+), the same ghost rules), for any number
 // of threads: a call handles the items tid, tid + nth, ... of its step, and
-// the caller separates steps by a barrier (one CTA on the GPU, one thread on
-// the host).  Ghost cells: Dirichlet g = 2b - u_1, Neumann g = u_1 + h b (b
-// = 0 for homogeneous data and for the correction), periodic sides copy the
-// cell at the other end of the row.  Edge and corner ghosts are not filled:
-// nothing here reads them.
+// the caller separates steps (one thread on the host).  Ghost cells: Dirichlet
+// g = 2b - u_1, Neumann g = u_1 + h b (b = 0 for homogeneous data and for the
+// correction), periodic sides copy the cell at the other end of the row.  Edge
+// and corner ghosts are not filled: nothing here reads them.
 #pragma once
 
 #ifdef __CUDACC__

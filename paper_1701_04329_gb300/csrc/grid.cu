@@ -91,7 +91,10 @@ Grid::Grid(const std::vector<const HostTree *> &trees, bool levels_only) {
     // one root box and for a single tree whose level 1 is a small block of
     // root boxes; for several roots otherwise they are device boxes, one per
     // root and level, and the cycle runs on the per-level kernels down to the
-    // coarsest grid (`roots_levels`).
+    // coarsest grid (`roots_levels`).  Small means the limit documented for
+    // afg_tree_create_roots.  The coarse launch would hold larger blocks too, but a
+    // tree solved in it takes no operator or prolongation after its data, and the
+    // trees above that limit do.
     bool multi = false;
     for (const HostTree *h : trees) multi |= h->nroots() != 1;
     block = T == 1 && multi && !levels_only &&
@@ -394,7 +397,8 @@ void Grid::alloc_ws(Workspace &w, bool fp64) {
 
 void Grid::refresh_rho_hat(cudaStream_t s) {
     if (!rhoh_stale || op) return;
-    launch_rho_hat(leaf_cfg(true, s), meta, d_leaves, n_leaf_boxes, ws64.rho->p, ws64.rhoh->p);
+    launch_rho_hat(leaf_cfg(true, s), meta, d_leaves, n_leaf_boxes, ws64.rho->as<double>(),
+                   ws64.rhoh->as<double>());
     rhoh_stale = false;
 }
 

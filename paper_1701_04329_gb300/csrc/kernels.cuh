@@ -877,8 +877,9 @@ __global__ void __launch_bounds__(kThreads) k_correct(BoxMeta A, int b0, int n, 
 }
 
 // rho_hat = -h^2 rho / (2D) on a list of boxes (after the source term changed)
-template <int D, int M, typename T>
-__global__ void __launch_bounds__(kThreads) k_rho_hat(BoxMeta A, const int *list, int n, const T *rho, T *rhoh) {
+template <int D, int M>
+__global__ void __launch_bounds__(kThreads) k_rho_hat(BoxMeta A, const int *list, int n, const double *rho,
+                                                      double *rhoh) {
     using Gm = Geo<D, M>;
     const int lt = threadIdx.x % Gm::G, g = threadIdx.x / Gm::G;
     pdl_trigger();
@@ -888,14 +889,13 @@ __global__ void __launch_bounds__(kThreads) k_rho_hat(BoxMeta A, const int *list
         if (idx >= n) continue;
         const int b = list[idx];
         const long long cb = A.coff[b];
-        const T c = T(-1.0 / (2 * D)) * T(A.hb[b] * A.hb[b]);  // h is a power of two: exact scaling, no FP64 division
-        constexpr int VEC = 16 / (int)sizeof(T);  // a box is a whole number of 16-byte vectors
-        for (int q = lt; q < Gm::C / VEC; q += Gm::G) {
-            T v[VEC];
-            ldv<T, VEC>(rho + cb + q * VEC, v);
-#pragma unroll
-            for (int x = 0; x < VEC; ++x) v[x] *= c;
-            stv<T, VEC>(rhoh + cb + q * VEC, v);
+        const double c = (-1.0 / (2 * D)) * (A.hb[b] * A.hb[b]);  // h is a power of two: exact scaling, no FP64 division
+        for (int q = 2 * lt; q < Gm::C; q += 2 * Gm::G) {
+            double v[2];
+            ldv<double, 2>(rho + cb + q, v);
+            v[0] *= c;
+            v[1] *= c;
+            stv<double, 2>(rhoh + cb + q, v);
         }
     }
 }

@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>()) k_leaf_re
 template <int D, int M>
 __global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, double, float>()) k_adjoint_plain_p(
     BoxMeta A, const int *list, int n, const double *lam, double *out) {
-    constexpr int GT = leaf_threads<D, M, double, float>(), FX = GT >= 32 ? fx_lap_weight<D>() : 0;
+    constexpr int GT = leaf_threads<D, M, double, float>(), FX = fx_lap_weight<D>();
     using F = FpCfg<D, M, double, GT>;
     constexpr int NVH = F::H / 2;
     FxPlan<D, M, GT> fxp;
@@ -912,30 +912,30 @@ __global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, double, float>()) 
     auto body = [&](const BoxInfo &I, const double *st, int lt, int E) {
         const double ih2 = A.ih2[I.b];
         const int e2 = (int)(__double_as_longlong(ih2) >> 52) - 1023;
-        if (E >= 0 && E + e2 <= 2040) {
+        auto aligned = [&](int e, auto scale) {  // scale: h^-2 by itself, near the end of the exponent range
 #pragma unroll
             for (int it = 0; it < FxPlan<D, M, GT>::NIV; ++it) {
                 const int v = lt + it * F::G;
                 if (v >= F::NV) continue;
                 double lap[2];
-                fp_lap_vec_fx<D, M, GT>(st, E + e2, fxp, it, lap);
+                fp_lap_vec_fx<D, M, GT>(st, e, fxp, it, lap);
+                if constexpr (decltype(scale)::value) {
+                    lap[0] *= ih2;
+                    lap[1] *= ih2;
+                }
                 stv<double, 2>(out + I.coff + v * 2, lap);
             }
+        };
+        if (E >= 0) {
+            if (E + e2 <= 2040) aligned(E + e2, std::false_type{});
+            else aligned(E, std::true_type{});
             return;
         }
         for (int v = lt; v < F::NV; v += F::G) {
+            const int col = v / NVH, w = v % NVH;
+            const int row = w / F::NVR, h0 = (w % F::NVR) * 2;
             double lap[2];
-            if (E >= 0) {  // near the end of the exponent range: h^-2 by itself
-                const int col = v / NVH;
-                (void)col;
-#pragma unroll
-                for (int it = 0; it < FxPlan<D, M, GT>::NIV; ++it)
-                    if (v == lt + it * F::G) fp_lap_vec_fx<D, M, GT>(st, E, fxp, it, lap);
-            } else {
-                const int col = v / NVH, w = v % NVH;
-                const int row = w / F::NVR, h0 = (w % F::NVR) * 2;
-                fp_lap_vec<D, M, double>(st, col, row % M, D == 2 ? 0 : row / M, h0, lap);
-            }
+            fp_lap_vec<D, M, double>(st, col, row % M, D == 2 ? 0 : row / M, h0, lap);
             lap[0] *= ih2;
             lap[1] *= ih2;
             stv<double, 2>(out + I.coff + v * 2, lap);

@@ -71,12 +71,14 @@ void launch_coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, si
 size_t bottom_block_smem(int D, bool fp64, int N, const int *nroot, const int *bct) {
     size_t n = 0;
     for (int M = 2; M <= N; M *= 2) {
-        const BlkLevel L = blk_level(D, nroot, M);
-        n += 4 * (size_t)L.padded;
-        for (int s = 0; s < 2 * D; ++s) {
-            int t1, t2;
-            if (bct[s] != 2) n += (size_t)blk_faces(L, s, t1, t2);
+        size_t padded = 1, cells = 1;
+        for (int a = 0; a < D; ++a) {
+            padded *= nroot[a] * M + 2;
+            cells *= nroot[a] * M;
         }
+        n += 4 * padded;
+        for (int s = 0; s < 2 * D; ++s)
+            if (bct[s] != 2) n += cells / (nroot[s / 2] * M);
     }
     return n * (fp64 ? 8 : 4);
 }
@@ -84,7 +86,7 @@ void launch_smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const in
                    const void *rhoh, double h2, int colour, int hom) {
     AFG_BY_DIM(smooth, c, A, b0, n, list, u, rho, rhoh, h2, colour, hom);
 }
-void launch_rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh) {
+void launch_rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *rho, double *rhoh) {
     AFG_BY_DIM(rho_hat, c, A, list, n, rho, rhoh);
 }
 void launch_resid_restrict(const LaunchCfg &c, const BoxMeta &A, int b0, int n, void *u, void *rho, void *vold,

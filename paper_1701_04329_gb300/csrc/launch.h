@@ -32,9 +32,9 @@ extern unsigned long long g_launches;
 // G: the grid's plan with the cycle's options (one cluster of G.R blocks per tree)
 void launch_coarse(const LaunchCfg &, const BoxMeta &, const CoarseArgs &G, size_t smem, int ntrees, void *u,
                    const void *rho, void *vold);
-// shared memory of one block that holds a block of root boxes and the grids
-// below it with four arrays each (bytes): what decides whether such a tree
-// keeps those grids out of device memory
+// bytes of four arrays of every grid of a block of root boxes and below it, with
+// the data of the sides: up to one block's shared memory, such a tree keeps those
+// grids out of device memory (the coarse launch needs less, Grid::Grid)
 size_t bottom_block_smem(int D, bool fp64, int N, const int *nroot, const int *bct);
 // opt-in shared memory per block of the current device (bytes)
 size_t max_smem_optin();
@@ -46,8 +46,8 @@ void launch_resid_restrict(const LaunchCfg &, const BoxMeta &, int b0, int n, vo
 // rhoh (may be null): also store the pre-scaled coarse source
 void launch_fas(const LaunchCfg &, const BoxMeta &, int b0, int n, const void *u, void *rho, void *vold, double ih2,
                 int hom, void *rhoh);
-// rhoh = -h^2 rho / (2D) on a list of boxes
-void launch_rho_hat(const LaunchCfg &, const BoxMeta &, const int *list, int n, const void *rho, void *rhoh);
+// rhoh = -h^2 rho / (2D) on a list of leaf boxes
+void launch_rho_hat(const LaunchCfg &, const BoxMeta &, const int *list, int n, const double *rho, double *rhoh);
 void launch_correct(const LaunchCfg &, const BoxMeta &, int b0, int n, void *u, const void *vold);
 // boxes b0..b0+n-1, or the n boxes of list (list != nullptr)
 void launch_restrict_u(const LaunchCfg &, const BoxMeta &, int b0, int n, const int *list, void *u);

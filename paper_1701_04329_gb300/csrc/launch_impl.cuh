@@ -10,7 +10,6 @@
 #include "kernels_leaf.cuh"
 #include "kernels_smooth.cuh"
 #include "kernels_full.cuh"
-#include "block_bottom.cuh"
 #include "kernels_coarse.cuh"
 #include "launch.h"
 
@@ -294,14 +293,11 @@ void do_reduce2(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, do
 template <int D, int M>
 void do_adjoint_plain(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *lam, double *out) {
     if (n <= 0) return;
-    if constexpr (FpCfg<D, M, double>::ok && leaf_threads<D, M, double, float>() >= 32) {
-        using F = FpCfg<D, M, double, leaf_threads<D, M, double, float>()>;
-        auto k = k_adjoint_plain_p<D, M>;
-        launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, lam, out);
-        ++g_launches;
-    } else {
-        throw std::runtime_error("leaf boxes have 4 cells per side or more");
-    }
+    static_assert(FpCfg<D, M, double>::ok, "leaf boxes have 4 cells per side or more");
+    using F = FpCfg<D, M, double, leaf_threads<D, M, double, float>()>;
+    auto k = k_adjoint_plain_p<D, M>;
+    launch_pdl(k, grid_for(k, F::smem(), (n + F::BPC - 1) / F::BPC), F::smem(), c.stream, A, list, n, lam, out);
+    ++g_launches;
 }
 
 template <int D, int M>
@@ -314,11 +310,11 @@ void do_reduce(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, con
     g_launches += 2;
 }
 
-template <int D, int M, typename T>
-void do_rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh) {
+template <int D, int M>
+void do_rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *rho, double *rhoh) {
     if (n <= 0) return;
-    auto k = k_rho_hat<D, M, T>;
-    launch_pdl(k, grid_for(k, 0, work_ctas<D, M>(n)), 0, c.stream, A, list, n, (const T *)rho, (T *)rhoh);
+    auto k = k_rho_hat<D, M>;
+    launch_pdl(k, grid_for(k, 0, work_ctas<D, M>(n)), 0, c.stream, A, list, n, rho, rhoh);
     ++g_launches;
 }
 
@@ -380,7 +376,6 @@ void do_coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t
 // launch_d<D>_f64.cu / launch_d<D>_f32.cu so those compile in parallel.
 template <int D, typename T>
 struct PrecOps {
-    static void rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh);
     static void coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
                        const void *rho, void *vold);
     static void smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *u,
@@ -397,11 +392,6 @@ struct PrecOps {
     static void leaf_set(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *src, void *dst);
     static void leaf_get(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *src, double *dst);
 };
-
-template <int D, typename T>
-void PrecOps<D, T>::rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh) {
-    AFG_SWITCH_M(c.M, (do_rho_hat<D, MM, T>(c, A, list, n, rho, rhoh)));
-}
 
 template <int D, typename T>
 void PrecOps<D, T>::coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
@@ -457,7 +447,8 @@ void PrecOps<D, T>::leaf_get(const LaunchCfg &c, const BoxMeta &A, const int *li
 
 template <int D>
 struct DimOps {
-    static void rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh);
+    static void rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *rho,
+                        double *rhoh);
     static void coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
                        const void *rho, void *vold);
     static void smooth(const LaunchCfg &c, const BoxMeta &A, int b0, int n, const int *list, void *u,
@@ -492,12 +483,6 @@ struct DimOps {
     static void reduce(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x,
                        const double *y, int mode, double *partials, double *result);
 };
-
-template <int D>
-void DimOps<D>::rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const void *rho, void *rhoh) {
-    if (c.fp64) PrecOps<D, double>::rho_hat(c, A, list, n, rho, rhoh);
-    else PrecOps<D, float>::rho_hat(c, A, list, n, rho, rhoh);
-}
 
 template <int D>
 void DimOps<D>::coarse(const LaunchCfg &c, const BoxMeta &A, const CoarseArgs &G, size_t smem, int ntrees, void *u,
@@ -595,6 +580,12 @@ void DimOps<D>::axpbypcz(const LaunchCfg &c, const BoxMeta &A, const int *list, 
         case 16: { constexpr int MM = 16; BODY; break; } \
         default: bad_size(M, 0);                         \
     }
+
+template <int D>
+void DimOps<D>::rho_hat(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *rho,
+                        double *rhoh) {
+    AFG_SWITCH_LEAF(c.M, (do_rho_hat<D, MM>(c, A, list, n, rho, rhoh)));
+}
 
 template <int D>
 void DimOps<D>::precond_in(const LaunchCfg &c, const BoxMeta &A, const int *list, int n, const double *x, void *rho,
