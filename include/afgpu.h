@@ -139,11 +139,11 @@ int afg_tree_create(int dim, int box_n, int max_level, afg_tree **out);
  * Every call accepts such trees: below level 1 the coarse grids of N/2, ...,
  * 2 cells hold one box per root, connected like the roots (Sec. 3.2: the
  * coarsest grid holds several boxes, relaxed together).  A single tree whose
- * block fits one CTA's shared memory (227 KB on GB300: per grid of M = 2, 4,
- * ..., N cells per root, 4 FP64 arrays of (r_x M + 2)(r_y M + 2)
- * (x (r_z M + 2)) values plus the face data of the non-periodic sides -- up
- * to 8 x 8 roots of 8^2 boxes, 4 x 4 of 16^2, 6 x 1 x 1 or 3 x 2 x 1 of 8^3,
- * no block of 16^3 boxes) solves them in that CTA, one launch per cycle;
+ * block is small solves them in one launch per cycle, in shared memory: where 4
+ * FP64 arrays of (r_x M + 2)(r_y M + 2) (x (r_z M + 2)) values per grid of M = 2,
+ * 4, ..., N cells per root, plus the face data of the non-periodic sides, come to
+ * no more than one CTA's shared memory (227 KB on GB300) -- up to 8 x 8 roots of
+ * 8^2 boxes, 4 x 4 of 16^2, 6 x 1 x 1 or 3 x 2 x 1 of 8^3, no block of 16^3 boxes;
  * larger blocks, every tree of a forest that holds a block tree, and a tree
  * given a variable-coefficient operator or another prolongation before its
  * data (afg_set_operator, afg_set_prolongation; afterwards AFG_ERR_STATE
@@ -267,7 +267,7 @@ int afg_set_dirichlet(afg_tree *t, const double *b_face_dev);
  * keeps the linear prolongation.  Host call; changing it keeps the field data
  * but requires afg_set_eps again.  AFG_ERR_ARG for an unknown op, (r,z) on a
  * 3D tree or with a periodic -x side; AFG_ERR_STATE on a tree of several
- * root boxes whose data were set for the one-CTA block solve (set the
+ * root boxes whose data were set for the one-launch block solve (set the
  * operator first).  Not covered with these operators: afg_adjoint and
  * afg_forest_residual_norms_noalloc (AFG_ERR_STATE), afg_time_kernel. */
 #define AFG_OP_LAPLACE 0
@@ -284,7 +284,7 @@ int afg_set_operator(afg_tree *t, int op);
  * every level, the coarse grids below the root included, runs on the
  * per-level kernels.  Host call; AFG_ERR_ARG for an unknown scheme;
  * AFG_ERR_STATE on a tree of several root boxes whose data were set for the
- * one-CTA block solve (set the scheme first). */
+ * one-launch block solve (set the scheme first). */
 #define AFG_PROLONG_LINEAR 0
 #define AFG_PROLONG_MULTILINEAR 1
 #define AFG_PROLONG_ZEROTH 2
@@ -295,7 +295,7 @@ int afg_set_prolongation(afg_tree *t, int scheme);
  * call also forms the face coefficients, 2 dim + 2 values per cell in FP64 and,
  * once mixed solves run, in FP32 (3D: 64 and 32 bytes per cell beside the 44 of
  * the FP64 fields and eps and the 12 of the FP32 ones).  They are left out, and
- * formed again on every use (solves two to four times slower), where they would
+ * formed again on every use (solves three to four times slower), where they would
  * take more than a quarter of the free device memory, where the allocator
  * callback refuses them, or, given back, where the FP32 fields do not fit
  * beside them. */

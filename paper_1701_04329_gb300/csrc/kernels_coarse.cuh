@@ -36,15 +36,17 @@
 //
 // Measured on a GB300 at 2 GHz, one V-cycle's visit: 2D, 64^2 and below, FP64
 // 63 us (levels 3-4 as 22 launches and a one-block bottom up to 32^2 before:
-// 120 us), FP32 30 us (77 us); 3D, 16^3 and below, FP32 28 us (49 us), FP64
-// 62 us on eight blocks (11 launches and a one-block bottom before: 87 us).
+// 120 us), FP32 30 us (77 us); 3D on eight blocks, FP64, 16^3 and below, 62 us
+// (11 launches and a one-block bottom before: 87 us), FP32 up to 32^3 for one
+// tree, 50 us with cold caches (16^3 and below alone 28 us, 49 us before).
 // Whole solves: 31 k unknowns in 2D, FP64, 2.89 -> 2.22 ms; 73 k unknowns on
 // a 3 x 2 block of root boxes, mixed, 7.40 -> 4.67 ms; 12 small quadtrees,
 // FP64, 2.30 -> 1.82 ms.  With variable coefficients (every level below them
 // on per-level launches before): 107 k unknowns in 2D, FP64, 6.57 -> 3.56 ms;
-// (r,z), 294 k, mixed, 5.80 -> 2.50 ms; 3D, 3.5 M, mixed, 7.96 -> 5.70 ms.  A half-sweep of a small grid is then 225 cycles in
-// FP32; in FP64 about 1100, of which the exact neighbour sum takes 285 and
-// every dependent FP64 operation 64-76.  A cluster barrier costs 350-450.
+// (r,z), 294 k, mixed, 5.80 -> 2.50 ms; 3D, 3.5 M, mixed, 7.96 -> 5.70 ms.  A
+// half-sweep of a small grid is then 225 cycles in FP32; in FP64 about 1100, of
+// which the exact neighbour sum takes 285 and every dependent FP64 operation
+// 64-76.  A cluster barrier costs 350-450.
 #pragma once
 #include "coarse_plan.h"
 #include "kernels.cuh"
@@ -619,7 +621,8 @@ __device__ __noinline__ void co_gather_coef(const BoxMeta &A, int rank, T *cpack
             co_decode<D>(c, L.nx, S.mx[li], L.ny, S.my[li], i, j, k);
             const int kz = L.z0 + k, jj = D == 3 ? j : kz, kk = D == 3 ? kz : 0, m1 = mb - 1;
             const int b = S.dtab[li][((size_t)tree * nbz + (kk >> lg)) * nby * nbx + (jj >> lg) * nbx + (i >> lg)];
-            const long long q = A.coff[b] + ((i + j + kz + D) & 1) * H + ((kk & m1) * mb + (jj & m1)) * (mb / 2) + ((i & m1) >> 1);
+            const long long q = A.coff[b] + ((i + j + kz + D) & 1) * H + ((kk & m1) * mb + (jj & m1)) * (mb / 2) +
+                                ((i & m1) >> 1);
             for (int f = 0; f < 2 * D + 2; ++f)
                 out[S.oc[li] - S.ocoef + f * S.csz[li] + L.slot(i, j, k)] =
                     reinterpret_cast<const T *>(S.coef)[f * S.coef_n + q];
@@ -648,7 +651,8 @@ __device__ __forceinline__ void co_run(int rank, int bc, const long long *cell0,
         r0 = (j + kz + D) & 1;  // red cell at 2x + r0
     };
     if constexpr (VAR) {  // the packed coefficients, waited for before the first use
-        const char *src = reinterpret_cast<const char *>(S.cpack) + (size_t)(blockIdx.x / S.R * S.R + rank) * S.ncoef * sizeof(T);
+        const char *src = reinterpret_cast<const char *>(S.cpack) +
+                          (size_t)(blockIdx.x / S.R * S.R + rank) * S.ncoef * sizeof(T);
         char *dst = reinterpret_cast<char *>(sm + S.ocoef);
         for (int x = tid; x < (int)(S.ncoef * sizeof(T) / 16); x += nt) cp_async<16>(dst + 16 * x, src + 16 * x);
         cp_commit();
@@ -773,7 +777,8 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse(BoxMeta A, const __gr
     const int lt = G.nl - 1, z0 = G.nr[lt] > 1 ? rank * G.P[lt] : 0;
     const int layer = D == 3 ? G.nbx * G.nby : G.nbx;
     const int first = (z0 >> G.lgmb) * layer, nbox = (((z0 + G.P[lt] - 1) >> G.lgmb) + 1) * layer - first;
-    long long *cell0 = reinterpret_cast<long long *>(co_smem + kCoarseHead + ((size_t)G.total * sizeof(T) + 15) / 16 * 16);
+    long long *cell0 =
+        reinterpret_cast<long long *>(co_smem + kCoarseHead + ((size_t)G.total * sizeof(T) + 15) / 16 * 16);
     unsigned char *refined = reinterpret_cast<unsigned char *>(cell0 + G.slab_boxes);
     const int *dbox = G.dbox + (size_t)tree * G.nbx * G.nby * G.nbz;
     for (int x = tid; x < nbox; x += nt) {

@@ -527,8 +527,9 @@ constexpr bool fx_leaf() { return sizeof(T) == 8 && (D == 3 || sizeof(R) == 4); 
 // an SM: 128 in 3D (aligned images; four blocks of 64 registers), 64 in 2D (two
 // blocks).  256^3 of 8^3 boxes: 0.165 ms with 128 threads and four blocks, 0.174
 // with three, 0.182 with 64 threads and two, 0.231 with 256 and three (per-cell
-// alignment, 64 threads and two: 0.280); 0.138 ms now (ONE, info_stage).  2D, 4.2 M cells, 8^2 / 16^2 boxes: four
-// blocks 56 / 39 us, three 71 / 41, no bound 97 / 54 (before 82 / 57).
+// alignment, 64 threads and two: 0.280); 0.137 ms with ONE and info_stage.  2D,
+// 4.2 M cells, 8^2 / 16^2 boxes: four blocks 56 / 39 us, three 71 / 41, no bound
+// 97 / 54 (before 82 / 57).
 template <int D, int M, typename T, typename R>
 constexpr int leaf_threads() {
     if (fx_leaf<D, T, R>() && D == 3)
@@ -554,7 +555,7 @@ constexpr int fx_restrict_weight() { return 2 * D * (1 << D); }
 // left three quarters of an FP64 box's threads idle and made 43 FP64 additions,
 // 64 cycles each, in a chain).  Left in FP64: the sum of the children's source
 // and one FMA.  The two roundings run side by side, in two threads of the four.
-// 256^3: 0.213 -> 0.165 ms, 0.148 ms with info_stage.
+// 256^3: 0.213 -> 0.165 ms, 0.150 ms with info_stage.
 template <int D, int M, int MP, int GT>
 __device__ __forceinline__ void rr_aligned(const BoxMeta &A, const BoxInfo &I, const double *st, int lt, int E,
                                            double ih2, long long cp, double *u, double *rho, double *vold) {
@@ -880,10 +881,9 @@ __device__ __forceinline__ void leaf_residual_walk(const BoxMeta &A, const int *
 }
 
 template <int D, int M, typename T, typename R, bool ONE>
-__global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>()) k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u,
-                                                              const T *__restrict__ rho, int hom,
-                                                              unsigned long long *rmax, unsigned long long *pmax,
-                                                              R *rout) {
+__global__ void __launch_bounds__(kThreads, leaf_blocks<D, M, T, R>())
+    k_leaf_residual_p(BoxMeta A, const int *list, int n, const T *u, const T *__restrict__ rho, int hom,
+                      unsigned long long *rmax, unsigned long long *pmax, R *rout) {
     constexpr int GT = leaf_threads<D, M, T, R>(), FX = fx_leaf<D, T, R>() ? fx_lap_weight<D>() : 0;
     pdl_trigger();
     auto lap = [](const BoxInfo &, const T *st, int, int col, int j, int k, int h0, T *out) {

@@ -343,9 +343,10 @@ __device__ __forceinline__ void group_sync(int g) {
 }
 
 // The barrier of a box's step: a box's stages and metadata belong to its thread
-// group, so whole warps meet their group only (256^3, FP64 half-sweep: 73.9 -> 72.2 us, FP32
-// restriction 50.7 -> 49.1 us); smaller groups meet the block.  Returns whether to take the extra step:
-// `extra` of this group's box, or of any box of the block.
+// group, so whole warps meet their group only (256^3, FP64 half-sweep: 73.9 ->
+// 72.2 us, FP32 restriction 50.7 -> 49.1 us); smaller groups meet the block.
+// Returns whether to take the extra step: `extra` of this group's box, or of any
+// box of the block.
 template <int G>
 __device__ __forceinline__ bool box_sync(int g, bool extra) {
     if constexpr (G >= 32) {
@@ -508,7 +509,8 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
         {
             const int q = it + NST - 1;
             const BoxInfo &In = info[(q % NI) * S::BPC + g];
-            if (info_on(A, In)) sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + ((q % NST) * S::BPC + g) * S::BOX, lt, c);
+            if (info_on(A, In))
+                sp_issue<D, M, T, VPT>(pl, In, u, rho, stages + ((q % NST) * S::BPC + g) * S::BOX, lt, c);
             info_stage<D>(A, base + NST * stride + g, n, b0, list, info[((it + NST) % NI) * S::BPC + g], lt, S::G);
             cp_commit();
         }
@@ -568,11 +570,11 @@ __device__ __forceinline__ void sp_walk(const BoxMeta &A, int b0, int n, const i
 }
 
 // FP64 half-sweeps in 3D whose boxes take whole warps align their images: 256^3
-// 100.5 -> 72.2 us, 194 instead of 249 instructions and one instead of five FP64
+// 100.5 -> 72.2 us, 201 instead of 249 instructions and one instead of five FP64
 // issues per update; 18.8 M unknowns, FP64, 29.0 -> 23.3 ms with the restriction
 // and the coarse right-hand side on aligned images too (2D keeps the per-cell
-// sums: its four terms need no FP64 addition).  Now 64.4 us (info_stage): issue
-// bound, 52.6 M warp instructions and 191 MB of DRAM traffic (3.0 TB/s) a launch.
+// sums: its four terms need no FP64 addition).  With info_stage 66 us: issue
+// bound, 52.7 M warp instructions and 191 MB of DRAM traffic (2.9 TB/s) a launch.
 template <int D, int M, typename T, int VPT>
 constexpr bool fx_smooth() { return sizeof(T) == 8 && D == 3 && SpCfg<D, M, T, VPT>::G >= 32; }
 

@@ -1,6 +1,7 @@
 // Set-up kernels, not part of the solve: leaf cell centres written straight
-// into device memory (the device form of afg_cell_centers), and the FP32
-// copy of a field (the coefficient of the variable-coefficient operators).
+// into device memory (the device form of afg_cell_centers), the boxes' records
+// that the staged kernels copy, and the FP32 copy of a field (the coefficient of
+// the variable-coefficient operators).
 #include <algorithm>
 
 #include "grid.h"
